@@ -6,6 +6,7 @@
 #include <new>
 #include <vector>
 
+#include "fp64_math.cuh"
 #include "mixed_common.cuh"
 
 namespace {
@@ -90,7 +91,7 @@ void free_plan(fmm_plan_s* pl) {
     void* bufs[] = {pl->keys, pl->rank, pl->counts, pl->leaf_start, pl->block_sums, pl->leaf_bstart,
                     pl->blk_map, pl->sorted_key,
                     pl->sorted64, pl->sorted32, pl->sorted_lo, pl->phi_far, pl->near_grad, pl->far_part,
-                    pl->T64, pl->T32, pl->U32,
+                    pl->T64, pl->logtab, pl->T32, pl->U32,
                     pl->d_status,
                     pl->d_counters, pl->d_xy_stage[0], pl->d_q_stage[0], pl->d_phi_stage[0], pl->d_xy_stage[1],
                     pl->d_q_stage[1], pl->d_phi_stage[1]};
@@ -235,12 +236,12 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
     FMM_TRY(dev_alloc(pl, &pl->counts, sizeof(uint32_t) * m));
     FMM_TRY(dev_alloc(pl, &pl->leaf_start, sizeof(uint32_t) * (m + 1)));
     pl->scan_blocks = fmm_scan_blocks(m);
-    // 64-bit partials in the mixed path (one scan of populations and near-field blocks)
+    // 64-bit partials (one scan of populations and near-field blocks)
     FMM_TRY(dev_alloc(pl, &pl->block_sums, sizeof(unsigned long long) * (pl->scan_blocks + 1)));
-    if (precision != FMM_FP64) {
-        FMM_TRY(dev_alloc(pl, &pl->leaf_bstart, sizeof(uint32_t) * (m + 1)));
-        // near-field blocks: at most one partial block per square; the near-field grid has four warps
-        // a CTA and every warp reads its entry, so the map is rounded up to four entries
+    FMM_TRY(dev_alloc(pl, &pl->leaf_bstart, sizeof(uint32_t) * (m + 1)));
+    {
+        // near-field blocks: at most one partial block per square; the mixed near-field grid has four
+        // warps a CTA and every warp reads its entry, so the map is rounded up to four entries
         const size_t nblk = ((size_t)m + (size_t)n / FMM_P2P_BLOCK + 1 + 3) & ~(size_t)3;
         FMM_TRY(dev_alloc(pl, &pl->blk_map, sizeof(uint2) * nblk));
     }
@@ -274,6 +275,13 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
     FMM_TRY(dev_alloc(pl, &pl->T64, sizeof(double2) * T.size()));
     if (cudaMemcpy(pl->T64, T.data(), sizeof(double2) * T.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         FMM_TRY(FMM_ERR_CUDA);
+    if (precision == FMM_FP64) {
+        std::vector<double2> tab(kFmmLogEntries);
+        for (int j = 0; j < kFmmLogEntries; ++j) tab[j] = fmm_log_entry(j);
+        FMM_TRY(dev_alloc(pl, &pl->logtab, sizeof(double2) * tab.size()));
+        if (cudaMemcpy(pl->logtab, tab.data(), sizeof(double2) * tab.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            FMM_TRY(FMM_ERR_CUDA);
+    }
     if (fmm_tc_precision(precision)) {
         std::vector<double> tre(T.size()), tim(T.size());
         for (size_t i = 0; i < T.size(); ++i) {

@@ -92,10 +92,10 @@ struct fmm_plan_s {
     uint32_t* rank;
     uint32_t* counts;
     uint32_t* leaf_start;
-    uint32_t* block_sums;        // scan partials, scan_blocks + 1 entries (64-bit in the mixed path)
+    uint32_t* block_sums;        // scan partials, scan_blocks + 1 entries of 64 bits
     int scan_blocks;
     uint32_t* leaf_bstart;       // near-field target blocks: exclusive scan over the squares, 4^levels + 1
-    uint2* blk_map;              // near-field block -> (square, block inside it), mixed path
+    uint2* blk_map;              // near-field block -> (square, block inside it)
     int clean;                   // mixed path: the square populations are zero (each call's scan
                                  // leaves them so; a call that failed to enqueue does not)
     uint32_t* sorted_key;
@@ -109,6 +109,7 @@ struct fmm_plan_s {
     float2* far_part;                 // mixed path: float-float far field of the coarse levels per particle
 
     double2* T64;       // FP64 operators [49][p+1][p+1]
+    double2* logtab;    // FP64 path: the near field's logarithm table (fp64_math.cuh)
     float2* T32;        // FP32 operators [49][p1b][p1b], zero-padded, [d][0][0] = 0 (mixed SIMT M2L)
     float2* U32;        // mixed path: upward-pass translations [child position][j][m] (p1b each), zero-padded
     int p1b;            // padded coefficient count of the FP32 M2L kernel instance
@@ -182,6 +183,23 @@ __host__ __device__ inline uint32_t fmm_morton(uint32_t ix, uint32_t iy) {
 }
 
 __host__ __device__ inline int fmm_grid_width(int k) { return (1 << k) + 2 * FMM_HALO; }
+
+// Forward neighbour `lane` (< 4: E, NE, N, NW) of finest square `leaf`: its first sorted particle
+// and count (an empty range outside the domain and on the other lanes).
+static __device__ __forceinline__ uint2 fmm_forward_neighbour(const uint32_t* __restrict__ ls, uint32_t leaf, int levels, int lane) {
+    uint32_t first = 0, cnt = 0;
+    if (lane < 4) {
+        const int side = 1 << levels;
+        const int jx = (int)fmm_compact2(leaf) + (lane == 3 ? -1 : (lane == 2 ? 0 : 1));
+        const int jy = (int)fmm_compact2(leaf >> 1) + (lane == 0 ? 0 : 1);
+        if (jx >= 0 && jy >= 0 && jx < side && jy < side) {
+            const uint32_t nl = fmm_morton((uint32_t)jx, (uint32_t)jy);
+            first = ls[nl];
+            cnt = ls[nl + 1] - first;
+        }
+    }
+    return make_uint2(first, cnt);
+}
 
 // Finest-square coordinate floor(fl(x 2^l / box)) clamped to [0, side - 1], the rule the oracle
 // uses, without occupying the narrow FP64 pipe in the common case: an FP32 estimate of the

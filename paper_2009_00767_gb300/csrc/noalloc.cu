@@ -19,11 +19,12 @@
 #include <mutex>
 
 #include "fmm_internal.cuh"
+#include "fp64_math.cuh"
 
 namespace {
 
 // Limits of the no-allocation path and the scratch they need (each sub-buffer 256-byte aligned):
-// particles <= 65536, levels <= 6, p <= 20.  Worst case about 8.0 MB; the array holds 8.5 MB.
+// particles <= 65536, levels <= 6, p <= 20.  Worst case about 8.1 MB; the array holds 8.5 MB.
 constexpr int64_t kMaxN = 65536;
 constexpr int kMaxLevels = 6;
 constexpr int kMaxP = 20;
@@ -78,6 +79,11 @@ __global__ void k_build_ops_f64(int p, double2* __restrict__ T) {
     T[e] = make_double2(c * pr, c * pi);
 }
 
+__global__ void k_build_logtab(double2* __restrict__ tab) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < kFmmLogEntries) tab[j] = fmm_log_entry(j);
+}
+
 // Carve the plan's workspaces out of the scratch block; returns the bytes used.
 size_t carve(fmm_plan_s* pl, unsigned char* base) {
     const int64_t n = pl->n;
@@ -94,7 +100,9 @@ size_t carve(fmm_plan_s* pl, unsigned char* base) {
     pl->counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * m));
     pl->leaf_start = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (m + 1)));
     pl->scan_blocks = fmm_scan_blocks(m);
-    pl->block_sums = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (pl->scan_blocks + 1)));
+    pl->block_sums = reinterpret_cast<uint32_t*>(take(sizeof(unsigned long long) * (pl->scan_blocks + 1)));
+    pl->leaf_bstart = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (m + 1)));
+    pl->blk_map = reinterpret_cast<uint2*>(take(sizeof(uint2) * (m + n / FMM_P2P_BLOCK + 1)));
     pl->sorted_key = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * n));
     pl->sorted64 = reinterpret_cast<fmm_p64*>(take(sizeof(fmm_p64) * n));
     pl->phi_far = reinterpret_cast<double*>(take(sizeof(double) * n));
@@ -105,6 +113,7 @@ size_t carve(fmm_plan_s* pl, unsigned char* base) {
         pl->grids.B[k] = take(((size_t)1 << (2 * k)) * p1 * sizeof(double2));
     }
     pl->T64 = reinterpret_cast<double2*>(take(sizeof(double2) * 49 * p1 * p1));
+    pl->logtab = reinterpret_cast<double2*>(take(sizeof(double2) * kFmmLogEntries));
     pl->d_status = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
     pl->d_counters = reinterpret_cast<unsigned long long*>(take(2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long)));
     return off;
@@ -172,6 +181,7 @@ extern "C" fmm_status fmm_potential_noalloc(int64_t n, int levels, int p, double
     // an error left pending by the caller's own earlier work is not this call's to report or clear
     if (cudaPeekAtLastError() != cudaSuccess) return FMM_ERR_CUDA;
     k_build_ops_f64<<<(nops + 255) / 256, 256, 0, st>>>(p, pl.T64);
+    k_build_logtab<<<(kFmmLogEntries + 127) / 128, 128, 0, st>>>(pl.logtab);
     if (cudaPeekAtLastError() != cudaSuccess) return FMM_ERR_CUDA;
     cudaEventRecord(pl.ev[0], st);
     if (fmm_launch_sort(&pl, xy, q) < 0 || fmm_launch_fp64(&pl, phi) < 0) return FMM_ERR_CUDA;

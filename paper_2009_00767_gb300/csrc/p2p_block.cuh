@@ -233,23 +233,6 @@ __device__ __forceinline__ float2 p2p_near(const float4* __restrict__ sp, const 
 // above) and q_t L to the source, summed over the block's targets in the lane that holds the
 // source and added to the source's accumulator with one FP64 atomic per lane and chunk.
 
-// Forward neighbour `lane` (< 4: E, NE, N, NW) of finest square `leaf`: its first sorted particle
-// and count (an empty range outside the domain and on the other lanes).
-__device__ __forceinline__ uint2 p2p_forward(const uint32_t* __restrict__ ls, uint32_t leaf, int levels, int lane) {
-    uint32_t first = 0, cnt = 0;
-    if (lane < 4) {
-        const int side = 1 << levels;
-        const int jx = (int)fmm_compact2(leaf) + (lane == 3 ? -1 : (lane == 2 ? 0 : 1));
-        const int jy = (int)fmm_compact2(leaf >> 1) + (lane == 0 ? 0 : 1);
-        if (jx >= 0 && jy >= 0 && jx < side && jy < side) {
-            const uint32_t nl = fmm_morton((uint32_t)jx, (uint32_t)jy);
-            first = ls[nl];
-            cnt = ls[nl + 1] - first;
-        }
-    }
-    return make_uint2(first, cnt);
-}
-
 // The block's sources: the own square's particles [t0, t0 + n_own) in nch_own chunks, then the
 // four forward neighbours' in lane order (seg[b]: sorted index minus slot, frame shift; thr:
 // first slot of forward neighbours 1..3).
@@ -345,7 +328,7 @@ __device__ __forceinline__ float2 p2p_near_sym(const float4* __restrict__ sp, co
                                                uint32_t leaf, uint32_t t0, uint32_t t1, uint32_t b0, int T,
                                                int levels, float s_leaf, float4* tgt, float2* tq, int4* seg,
                                                int lane, double* __restrict__ acc, uint32_t* pairs) {
-    const uint2 nb = p2p_forward(ls, leaf, levels, lane);
+    const uint2 nb = fmm_forward_neighbour(ls, leaf, levels, lane);
     const uint32_t n_own = t1 - t0;
     uint32_t incl = nb.y;
 #pragma unroll
@@ -531,7 +514,7 @@ __device__ __forceinline__ NearField p2p_near_sym_field(const float4* __restrict
                                                         float4* tgt, float4* tlo, float2* tq, int4* seg, int lane,
                                                         double* __restrict__ acc, double2* __restrict__ accg,
                                                         uint32_t* pairs) {
-    const uint2 nb = p2p_forward(ls, leaf, levels, lane);
+    const uint2 nb = fmm_forward_neighbour(ls, leaf, levels, lane);
     const uint32_t n_own = t1 - t0;
     uint32_t incl = nb.y;
 #pragma unroll

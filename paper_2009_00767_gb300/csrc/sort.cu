@@ -121,7 +121,7 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, int64_t m, const ui
     if (blockIdx.x == 0 && threadIdx.x == 0) out[m] = (n_total == 0xffffffffu) ? sums[gridDim.x] : n_total;
 }
 
-// Mixed path: one scan of (population, near-field blocks) pairs packed in 64 bits (the low word
+// One scan of (population, near-field blocks) pairs packed in 64 bits (the low word
 // never carries: n < 2^32) gives leaf_start and the block starts at once; the down-sweep also
 // writes the block -> (square, block inside it) map and zeroes the populations it has read.
 __device__ __forceinline__ unsigned long long pop_blocks(uint32_t c) {
@@ -282,12 +282,8 @@ int fmm_launch_sort(fmm_plan_s* pl, const double* xy, const double* q, bool with
         ++launches;
     }
     const int nb = pl->scan_blocks;
-    if (pl->precision == FMM_FP64) {
-        k_scan_reduce<<<nb, kScanThreads, 0, st>>>(pl->counts, m, pl->block_sums);
-        k_scan_top<<<1, kScanThreads, 0, st>>>(pl->block_sums, nb);
-        k_scan_down<<<nb, kScanThreads, 0, st>>>(pl->counts, m, pl->block_sums, pl->leaf_start, (uint32_t)n);
-    } else {
-        // the near-field blocks come with the same scan (block_sums holds 64-bit partials here)
+    {
+        // the near-field blocks come with the same scan (block_sums holds 64-bit partials)
         unsigned long long* sums = reinterpret_cast<unsigned long long*>(pl->block_sums);
         k_scan2_reduce<<<nb, kScanThreads, 0, st>>>(pl->counts, m, sums);
         if (nb <= kLocalTopMax) {

@@ -128,3 +128,36 @@ def test_full_size_uniform_1m(oracle_mod):
     check_parity(phi, ref, TOL, "fp64 N=2^20 levels=8 p=20")
     # near-field pair count: about 9 x 16 sources per particle for a uniform tree
     assert 100 * (1 << 20) < st["p2p_pairs"] < 160 * (1 << 20)
+
+
+@pytest.mark.parametrize("lev", [0, 1, 2])
+@pytest.mark.parametrize("n", [2, 15, 16, 17, 24, 25, 31, 33, 40, 41, 49, 63, 97, 260, 1300])
+def test_near_field_tiles(oracle_mod, n, lev):
+    """Blocks of 1 to 24 targets, source chunks of every remainder, crowded and empty squares: potential and
+    field against the direct sums.  At levels <= 1 there is no far field and both sides add the same terms, each
+    within 2 ulp, so 1e-13 relative (the bound of the other direct comparisons); at level 2 the truncation at
+    p = 40 is below 0.547^40 = 4e-11 of the far field, so the FMM of the same order is the reference."""
+    import torch
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    xy, q = inputs.uniform(n, 8200 + n)
+    txy, tq = to_dev(xy, q)
+    with binding.Plan(n, lev, 40) as plan:
+        phi, field = plan.potential_field(txy, tq)
+        only = plan.potential(txy, tq)
+    rp, rf = ((oracle_mod.direct(xy, q), oracle_mod.direct_field(xy, q)) if lev < 2
+              else oracle_mod.shiftfree_field(xy, q, lev, 40))
+    tol = 1e-13 if lev < 2 else TOL
+    check_parity(only.cpu().numpy(), rp, tol, f"fp64 near n={n} levels={lev}")
+    check_parity(phi.cpu().numpy(), rp, tol, f"fp64 near phi n={n} levels={lev}")
+    check_parity(field.cpu().numpy().ravel(), np.asarray(rf).ravel(), TOL, f"fp64 near field n={n} levels={lev}")
+
+
+def test_near_field_at_extreme_distances(oracle_mod):
+    """r^2 that is zero by underflow, subnormal, one ulp and a power of two: the same as the oracle's log."""
+    from gpu_util import run_fmm
+    x = np.array([0.0, 1e-170, 1e-160, 3e-155, 1e-150, 2.0 ** -30, 2.0 ** -30 + 2.0 ** -82, 1.0, 1.0 + 2.0 ** -52, 2.0, 4.0])
+    xy = np.stack((x, np.zeros_like(x)), 1)
+    q = np.linspace(-1.0, 1.5, x.size)
+    phi, _ = run_fmm(xy, q, 0, 4)
+    check_parity(phi, oracle_mod.direct(xy, q), 1e-13, "fp64 near field, extreme distances")
