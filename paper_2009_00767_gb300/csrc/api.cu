@@ -49,6 +49,35 @@ void build_operators(int p, std::vector<cd>& T) {
         }
 }
 
+// The FP64 path's translations T_d[k][l] = d^-l R[k][l] d^-k (the same entries as above, factored): R, the
+// binomials of M2M and L2L, and d^-k of each orbit's representative (fp64_math.cuh, fp64.cu).
+void build_far_tables(int p, std::vector<double>& tab) {
+    const int p1 = p + 1;
+    tab.assign(fmm_far_table_doubles(p1), 0.0);
+    double* R = tab.data();
+    double* B = R + ((p1 * p1 + 1) & ~1);
+    double* D = B + ((p1 * p1 + 1) & ~1);
+    std::vector<std::vector<double>> C(2 * p + 2, std::vector<double>(2 * p + 2, 0.0));
+    for (int nn = 0; nn < 2 * p + 2; ++nn) {
+        C[nn][0] = 1.0;
+        for (int r = 1; r <= nn; ++r) C[nn][r] = C[nn - 1][r - 1] + (r <= nn - 1 ? C[nn - 1][r] : 0.0);
+    }
+    for (int l = 1; l <= p; ++l) R[l] = -1.0 / (double)l;   // k = 0; the monopole-log term of b'_0 is separate
+    for (int k = 1; k <= p; ++k)
+        for (int l = 0; l <= p; ++l) R[(size_t)k * p1 + l] = ((k & 1) ? 1.0 : -1.0) / (double)k * C[l + k - 1][k - 1];
+    for (int m = 0; m <= p; ++m)
+        for (int j = 0; j <= m; ++j) B[(size_t)m * p1 + j] = C[m][j];
+    for (int o = 0; o < kFmmOrbits; ++o) {
+        const cd inv = 1.0 / cd((double)fmm_orbit_x(o), (double)fmm_orbit_y(o));
+        cd v = 1.0;
+        for (int k = 0; k <= p; ++k) {
+            D[2 * ((size_t)o * p1 + k)] = v.real();
+            D[2 * ((size_t)o * p1 + k) + 1] = v.imag();
+            v *= inv;
+        }
+    }
+}
+
 bool valid_precision(int v) { return v >= FMM_FP64 && v <= FMM_MIXED_BF16X2; }
 
 // fmm_potential_host: inputs of at least kHostChunkMin particles go up in kHostChunks chunks
@@ -91,7 +120,7 @@ void free_plan(fmm_plan_s* pl) {
     void* bufs[] = {pl->keys, pl->rank, pl->counts, pl->leaf_start, pl->block_sums, pl->leaf_bstart,
                     pl->blk_map, pl->sorted_key,
                     pl->sorted64, pl->sorted32, pl->sorted_lo, pl->phi_far, pl->near_grad, pl->far_part,
-                    pl->T64, pl->logtab, pl->T32, pl->U32,
+                    pl->ftab, pl->logtab, pl->T32, pl->U32,
                     pl->d_status,
                     pl->d_counters, pl->d_xy_stage[0], pl->d_q_stage[0], pl->d_phi_stage[0], pl->d_xy_stage[1],
                     pl->d_q_stage[1], pl->d_phi_stage[1]};
@@ -261,8 +290,11 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
     for (int k = 2; k <= levels; ++k) {
         const size_t W = (size_t)fmm_grid_width(k);
         pl->a_bytes[k] = W * W * p1 * sizeof(double2);
-        if (precision == FMM_FP64)   // the mixed path's moments live in the FP32 grids only
+        if (precision == FMM_FP64) {   // the mixed path's moments live in the FP32 grids only
             FMM_TRY(dev_alloc(pl, reinterpret_cast<char**>(&pl->grids.A[k]), pl->a_bytes[k]));
+            // the 3-cell halo stays zero for the plan's lifetime
+            if (cudaMemset(pl->grids.A[k], 0, pl->a_bytes[k]) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
+        }
         FMM_TRY(dev_alloc(pl, reinterpret_cast<char**>(&pl->grids.B[k]), ((size_t)1 << (2 * k)) * p1 * bcplx));
         if (precision != FMM_FP64) {
             // the 3-cell halo of the FP32 grid stays zero for the plan's lifetime
@@ -271,11 +303,13 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         }
     }
     std::vector<cd> T;
-    build_operators(p, T);
-    FMM_TRY(dev_alloc(pl, &pl->T64, sizeof(double2) * T.size()));
-    if (cudaMemcpy(pl->T64, T.data(), sizeof(double2) * T.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-        FMM_TRY(FMM_ERR_CUDA);
+    if (precision != FMM_FP64) build_operators(p, T);
     if (precision == FMM_FP64) {
+        std::vector<double> ftab;
+        build_far_tables(p, ftab);
+        FMM_TRY(dev_alloc(pl, &pl->ftab, sizeof(double) * ftab.size()));
+        if (cudaMemcpy(pl->ftab, ftab.data(), sizeof(double) * ftab.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            FMM_TRY(FMM_ERR_CUDA);
         std::vector<double2> tab(kFmmLogEntries);
         for (int j = 0; j < kFmmLogEntries; ++j) tab[j] = fmm_log_entry(j);
         FMM_TRY(dev_alloc(pl, &pl->logtab, sizeof(double2) * tab.size()));

@@ -13,10 +13,10 @@
 //   A32[k]                   (mixed) FP32 moments of level k, same layout (the mixed path has no
 //                            FP64 A[k]); slot 0 holds M_0 as a float-float pair
 //   (mixed) B[k] slot 0 holds Re b'_0 as a float-float pair
-//   phi_far[n]               FP64 path: far field summed over levels, box-sorted order; mixed
+//   phi_far[n]               FP64 path: far field, then far + near, box-sorted order; mixed
 //                            path: the near field as float-float pairs (log2 r^2 units)
-//   T64                      49 x (p+1) x (p+1) complex FP64 M2L operators, layout [d][k][l],
-//                            d = (dx + 3) + 7 (dy + 3), zero for the 9 adjacent offsets
+//   ftab                     (FP64 path) the translations' real matrices R[k][l] and C(m, j), and the
+//                            powers d^-k of the interaction-list offsets
 // Because keys are Morton-ordered, the particles of every square of every level are one
 // contiguous range of the sorted arrays (square key = finest key >> 2 (levels - k)).
 #pragma once
@@ -108,7 +108,7 @@ struct fmm_plan_s {
     double2* near_grad;               // mixed path: near-field gradient accumulator (fmm_potential_field)
     float2* far_part;                 // mixed path: float-float far field of the coarse levels per particle
 
-    double2* T64;       // FP64 operators [49][p+1][p+1]
+    double* ftab;       // FP64 path: the far field's real matrices and powers (fp64_math.cuh)
     double2* logtab;    // FP64 path: the near field's logarithm table (fp64_math.cuh)
     float2* T32;        // FP32 operators [49][p1b][p1b], zero-padded, [d][0][0] = 0 (mixed SIMT M2L)
     float2* U32;        // mixed path: upward-pass translations [child position][j][m] (p1b each), zero-padded

@@ -61,3 +61,13 @@ __device__ __forceinline__ double fmm_rsqrt(double x) {
     const double e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
+
+// The interaction-list offsets as orbits of quarter turns (fp64.cu): a representative of each.
+constexpr int kFmmOrbits = 10;
+__host__ __device__ constexpr int fmm_orbit_x(int o) { return o < 3 ? 2 : (o == 3 ? 1 : 3); }
+__host__ __device__ constexpr int fmm_orbit_y(int o) { return o < 3 ? o : (o == 3 ? 2 : (o < 9 ? o - 6 : 3)); }
+// Doubles of the far field's tables for p1 = p + 1 coefficients: R[k][l] and C(m, j) (each padded to an
+// even count), then d^-k of every orbit.
+__host__ __device__ inline size_t fmm_far_table_doubles(int p1) {
+    return 2 * (size_t)((p1 * p1 + 1) & ~1) + 2 * (size_t)kFmmOrbits * p1;
+}

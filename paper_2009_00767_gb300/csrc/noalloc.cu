@@ -24,7 +24,7 @@
 namespace {
 
 // Limits of the no-allocation path and the scratch they need (each sub-buffer 256-byte aligned):
-// particles <= 65536, levels <= 6, p <= 20.  Worst case about 8.1 MB; the array holds 8.5 MB.
+// particles <= 65536, levels <= 6, p <= 20.  Worst case about 7.8 MB; the array holds 8.5 MB.
 constexpr int64_t kMaxN = 65536;
 constexpr int kMaxLevels = 6;
 constexpr int kMaxP = 20;
@@ -39,44 +39,34 @@ cudaEvent_t g_events[kMaxDevices][6] = {};
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Scale-free FP64 M2L operators on power-sum moments, built on the device so that the call
-// needs neither a host buffer nor a host-to-device copy; the same formulas as the plan's
-// host-side build (Greengard's 2D conversion, ref. [101] of the paper):
-//   T[d][k][l], d = (dx + 3) + 7 (dy + 3), w0 = dx + i dy:
-//   T[0][0] = log(-w0), T[0][l] = -w0^-l / l, T[k][0] = (-1)^(k+1) w0^-k / k,
-//   T[k][l] = (-1)^(k+1) C(l+k-1, k-1) w0^-(l+k) / k;  zero for the nine adjacent offsets.
-__global__ void k_build_ops_f64(int p, double2* __restrict__ T) {
-    const int p1 = p + 1;
+// The FP64 path's tables (the plan's host-side build_far_tables), built on the device so that the call
+// needs neither a host buffer nor a host-to-device copy: R[k][l] = (-1)^(k+1) C(l+k-1, k-1) / k with
+// R[0][l] = -1 / l, then C(m, j), then d^-k of the interaction lists' orbits.
+__global__ void k_build_far_tables(int p1, double* __restrict__ tab) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= 49 * p1 * p1) return;
-    const int d = e / (p1 * p1), k = (e / p1) % p1, l = e % p1;
-    const int dx = d % 7 - 3, dy = d / 7 - 3;
-    if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) {
-        T[e] = make_double2(0.0, 0.0);
-        return;
+    const int pad = (p1 * p1 + 1) & ~1;
+    const int k = e / p1, l = e % p1;
+    if (e < p1 * p1) {
+        double r = 0.0;
+        if (k == 0) {
+            r = l ? -1.0 / (double)l : 0.0;
+        } else {
+            double b = 1.0;   // C(l+k-1, k-1) by the multiplicative formula (exact for these sizes)
+            for (int i = 1; i <= k - 1; ++i) b = b * (double)(l + i) / (double)i;
+            r = ((k & 1) ? 1.0 : -1.0) / (double)k * b;
+        }
+        tab[e] = r;
+        double c = l <= k ? 1.0 : 0.0;   // C(k, l)
+        for (int i = 1; i <= l && l <= k; ++i) c = c * (double)(k - l + i) / (double)i;
+        tab[pad + e] = c;
     }
-    const double r2 = (double)(dx * dx + dy * dy);
-    const double ivr = (double)dx / r2, ivi = -(double)dy / r2;   // 1 / w0
-    if (k == 0 && l == 0) {
-        T[e] = make_double2(0.5 * log(r2), atan2(-(double)dy, -(double)dx));
-        return;
+    if (e < kFmmOrbits * p1) {
+        const double x = fmm_orbit_x(k), y = fmm_orbit_y(k), r2 = x * x + y * y;
+        double2 v = make_double2(1.0, 0.0);
+        const double ix = x / r2, iy = -y / r2;
+        for (int i = 0; i < l; ++i) v = make_double2(v.x * ix - v.y * iy, v.x * iy + v.y * ix);
+        reinterpret_cast<double2*>(tab + 2 * pad)[e] = v;
     }
-    double pr = 1.0, pi = 0.0;   // w0^-(l+k)
-    for (int m = 0; m < l + k; ++m) {
-        const double nr = pr * ivr - pi * ivi;
-        const double ni = pr * ivi + pi * ivr;
-        pr = nr;
-        pi = ni;
-    }
-    double c;
-    if (k == 0) {
-        c = -1.0 / (double)l;
-    } else {
-        double b = 1.0;   // C(l+k-1, k-1) by the multiplicative formula (exact for these sizes)
-        for (int i = 1; i <= k - 1; ++i) b = b * (double)(l + i) / (double)i;
-        c = ((k & 1) ? 1.0 : -1.0) * b / (double)k;
-    }
-    T[e] = make_double2(c * pr, c * pi);
 }
 
 __global__ void k_build_logtab(double2* __restrict__ tab) {
@@ -112,7 +102,7 @@ size_t carve(fmm_plan_s* pl, unsigned char* base) {
         pl->grids.A[k] = take(pl->a_bytes[k]);
         pl->grids.B[k] = take(((size_t)1 << (2 * k)) * p1 * sizeof(double2));
     }
-    pl->T64 = reinterpret_cast<double2*>(take(sizeof(double2) * 49 * p1 * p1));
+    pl->ftab = reinterpret_cast<double*>(take(sizeof(double) * fmm_far_table_doubles(p1)));
     pl->logtab = reinterpret_cast<double2*>(take(sizeof(double2) * kFmmLogEntries));
     pl->d_status = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
     pl->d_counters = reinterpret_cast<unsigned long long*>(take(2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long)));
@@ -177,10 +167,12 @@ extern "C" fmm_status fmm_potential_noalloc(int64_t n, int levels, int p, double
     if (cudaMemsetAsync(pl.d_status, 0, sizeof(unsigned int), st) != cudaSuccess ||
         cudaMemsetAsync(pl.d_counters, 0, 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long), st) != cudaSuccess)
         return FMM_ERR_CUDA;
-    const int nops = 49 * (p + 1) * (p + 1);
+    for (int k = 2; k <= levels; ++k)   // the halos of the moment grids read as zero
+        if (cudaMemsetAsync(pl.grids.A[k], 0, pl.a_bytes[k], st) != cudaSuccess) return FMM_ERR_CUDA;
+    const int ntab = (p + 1) * (p + 1 > kFmmOrbits ? p + 1 : kFmmOrbits);
     // an error left pending by the caller's own earlier work is not this call's to report or clear
     if (cudaPeekAtLastError() != cudaSuccess) return FMM_ERR_CUDA;
-    k_build_ops_f64<<<(nops + 255) / 256, 256, 0, st>>>(p, pl.T64);
+    k_build_far_tables<<<(ntab + 255) / 256, 256, 0, st>>>(p + 1, pl.ftab);
     k_build_logtab<<<(kFmmLogEntries + 127) / 128, 128, 0, st>>>(pl.logtab);
     if (cudaPeekAtLastError() != cudaSuccess) return FMM_ERR_CUDA;
     cudaEventRecord(pl.ev[0], st);

@@ -161,3 +161,20 @@ def test_near_field_at_extreme_distances(oracle_mod):
     q = np.linspace(-1.0, 1.5, x.size)
     phi, _ = run_fmm(xy, q, 0, 4)
     check_parity(phi, oracle_mod.direct(xy, q), 1e-13, "fp64 near field, extreme distances")
+
+
+@pytest.mark.parametrize("lev", [2, 3, 4, 6])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 8, 15, 20, 31, 32, 39, 40])
+def test_far_field_orders(oracle_mod, p, lev):
+    """Orders that are and are not a multiple of four, rows that do and do not fill a block, parity classes that
+    do and do not fill one: potential and field against the oracle's FMM of the same order, to rounding."""
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    n = 700 + 13 * p
+    xy, q = inputs.uniform(n, 8300 + p)
+    txy, tq = to_dev(xy, q)
+    with binding.Plan(n, lev, p) as plan:
+        phi, field = plan.potential_field(txy, tq)
+    rp, rf = oracle_mod.shiftfree_field(xy, q, lev, p)
+    check_parity(phi.cpu().numpy(), rp, TOL, f"fp64 far p={p} levels={lev}")
+    check_parity(field.cpu().numpy().ravel(), np.asarray(rf).ravel(), TOL, f"fp64 far field p={p} levels={lev}")
