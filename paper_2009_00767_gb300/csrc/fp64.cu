@@ -21,7 +21,7 @@
 // 2 instead of 16 FP64 instructions per (k, l) for four squares.  M2M and L2L, whose four children sit a
 // quarter turn apart, have the same form with binomials for R.
 #include "fmm_internal.cuh"
-#include "fp64_math.cuh"
+#include "p2p64.cuh"
 
 namespace {
 
@@ -356,58 +356,21 @@ __global__ void k_l2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __rest
 }
 
 // -------------------------------------------------------------------------------- P2P + final phi
-// The near field by pair symmetry: log r^2 is the same for both particles of a pair, so each pair of
-// the own and adjacent squares is evaluated once.  One warp per block of up to FMM_P2P_BLOCK targets of
-// a finest square (blk_map, from the sort's scan).  Its pairs are
-//   * the block against itself: lane l (a target) meets target (l + s) mod T at step s = 1 .. T / 2;
-//   * the block against its "later" sources, 32 at a time, one a lane: the rest of the own square after
-//     the block, then the forward neighbours E, NE, N, NW.  At step s lane l meets target (l + s) mod T,
-//     so the lanes' targets differ and their sums can live in shared memory (one row of T sums per T
-//     lanes) while the source's sum stays in a register.
-// A last chunk of at most 16 sources gives each source two lanes that share the steps.  Every result is
-// added to the far field with an FP64 atomic; k_finish_f64 then writes phi in input order.
-//
-// What bounds it: FP64 issue (fp64_math.cuh), 11 instructions a pair: 2 + 2 for r^2, 5 for the logarithm
-// and one FMA for each side.  The rolled loop keeps the code small and needs no sums in registers, so
-// the pipe always has a warp ready.  2^20 uniform particles, levels 8: 1.93 ms against 15.0 ms for a
-// kernel that took every ordered pair with the library's log.
+// The near field, each pair of the own and adjacent squares once (p2p64.cuh): one warp per block of up to
+// FMM_P2P_BLOCK targets of a finest square (blk_map, from the sort's scan), whose later sources are the
+// rest of the own square and the forward neighbours E, NE, N, NW.  Every result is added to the far field
+// with an FP64 atomic; k_finish_f64 then writes phi in input order.
+// 2^20 uniform particles, levels 8: 1.93 ms against 15.0 ms for a kernel that took every ordered pair with
+// the library's log.
 // kField: also grad phi, q (dx, dy) / r^2 to the target and the opposite to the source.
 constexpr int kP2PWarps64 = 8;
 // With fewer blocks than this, CTAs of two warps instead of eight: 152 SMs x 4 schedulers x 8 warps
 // are not filled either way, and the smaller CTAs reach more SMs.
 constexpr int64_t kP2PSmall = 4096;
-// sums per target of a block of T: 32 / T rows of T for whole chunks (at most 31 + T), and for the
-// second lanes of a split chunk 16 / T rows more (at most 15 + T)
-constexpr int kP2PRows = 31 + FMM_P2P_BLOCK + 1, kP2PRows2 = 15 + FMM_P2P_BLOCK + 1;
-
-template <bool kField>
-struct P2PAcc {
-    double phi, gx, gy;
-};
-
-template <bool kField>
-__device__ __forceinline__ void p2p64_pair(P2PAcc<kField>& a, double (*__restrict__ row)[kField ? 3 : 1], double sx,
-                                           double sy, double sq, double tx, double ty, double tq,
-                                           const double2* __restrict__ tab) {
-    const double dx = tx - sx, dy = ty - sy;
-    const double r2 = fma(dx, dx, dy * dy);
-    const double lg = fmm_log(r2, tab);
-    (*row)[0] = fma(sq, lg, (*row)[0]);
-    a.phi = fma(tq, lg, a.phi);
-    if constexpr (kField) {
-        const bool normal = (unsigned)__double2hiint(r2) - 0x00100000u < 0x7fe00000u;
-        const double iv = normal ? fmm_rcp(r2) : (r2 > 0.0 ? 1.0 / r2 : 0.0);
-        const double wx = dx * iv, wy = dy * iv;
-        (*row)[1] = fma(sq, wx, (*row)[1]);
-        (*row)[2] = fma(sq, wy, (*row)[2]);
-        a.gx = fma(-tq, wx, a.gx);
-        a.gy = fma(-tq, wy, a.gy);
-    }
-}
 
 template <bool kField>
 __device__ __forceinline__ void p2p64_add(double* __restrict__ phi, double2* __restrict__ grad, int64_t i,
-                                          const P2PAcc<kField>& a) {
+                                          const P64Acc<kField>& a) {
     atomicAdd(phi + i, 0.5 * a.phi);   // log r = log(r^2) / 2
     if constexpr (kField) {
         atomicAdd(&grad[i].x, a.gx);
@@ -421,10 +384,8 @@ k_p2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __restrict__ leaf_star
           const uint32_t* __restrict__ bstart, const uint2* __restrict__ bmap, uint32_t nleaf, int levels,
           const double2* __restrict__ logtab, double* __restrict__ phi, double2* __restrict__ grad,
           const unsigned int* __restrict__ status, unsigned long long* __restrict__ counters) {
-    constexpr int V = kField ? 3 : 1;
     __shared__ double2 tab[kFmmLogEntries];
-    __shared__ double tgt[kP2PWarps64][3][FMM_P2P_BLOCK];
-    __shared__ double rows[kP2PWarps64][kP2PRows + kP2PRows2][V];
+    __shared__ P64Shared<2, kField, FMM_P2P_BLOCK> sh[kP2PWarps64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kFmmLogEntries; i += blockDim.x) tab[i] = logtab[i];
     __syncthreads();
@@ -435,96 +396,28 @@ k_p2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __restrict__ leaf_star
     const uint32_t leaf = lt.x, t0 = leaf_start[leaf], t1 = leaf_start[leaf + 1];
     const uint32_t b0 = t0 + (uint32_t)FMM_P2P_BLOCK * lt.y;
     const int T = (int)min((uint32_t)FMM_P2P_BLOCK, t1 - b0);
-    // later sources: [b0 + T, t1) of the own square, then the forward neighbours
     const uint2 nb = fmm_forward_neighbour(leaf_start, leaf, levels, lane);
-    const uint32_t n_own = t1 - b0 - (uint32_t)T;
-    uint32_t end[5], first[5];
-    end[0] = n_own;
+    uint32_t end[5], first[5];   // later sources: sorted index minus slot, slots up to the range's end
     first[0] = b0 + (uint32_t)T;
+    end[0] = t1 - first[0];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        first[i + 1] = __shfl_sync(0xffffffffu, nb.x, i) - end[i];   // sorted index minus slot
+        first[i + 1] = __shfl_sync(0xffffffffu, nb.x, i) - end[i];
         end[i + 1] = end[i] + __shfl_sync(0xffffffffu, nb.y, i);
     }
-    const uint32_t nsrc = end[4];
     if (lane == 0) {
         const unsigned slot = leaf % FMM_COUNTER_SLOTS;
-        atomicAdd(&counters[slot], (unsigned long long)T * ((t1 - t0) + 2ull * (nsrc - n_own)) - (unsigned long long)T);
+        atomicAdd(&counters[slot], (unsigned long long)T * ((t1 - t0) + 2ull * (end[4] - end[0])) - (unsigned long long)T);
         atomicMax(&counters[FMM_COUNTER_SLOTS + slot], (unsigned long long)(t1 - t0));
     }
-    double* const X = tgt[warp][0];
-    double* const Y = tgt[warp][1];
-    double* const Q = tgt[warp][2];
-    auto row = rows[warp];
-    fmm_p64 own = fmm_p64{0.0, 0.0, 0.0, 0.0};
-    if (lane < T) {
-        own = sp[b0 + lane];
-        X[lane] = own.x;
-        Y[lane] = own.y;
-        Q[lane] = own.q;
-    }
-    for (int i = lane; i < kP2PRows + kP2PRows2; i += 32)
-#pragma unroll
-        for (int v = 0; v < V; ++v) row[i][v] = 0.0;
-    __syncwarp();
-    // the block against itself: at the last step of an even T the lanes of the lower half cover all pairs
-    P2PAcc<kField> mine = {};
-    for (int s = 1; 2 * s <= T; ++s) {
-        const int lim = 2 * s == T ? s : T;
-        if (lane < lim) {
-            const int t = lane + s < T ? lane + s : lane + s - T;
-            p2p64_pair<kField>(mine, row + t, own.x, own.y, own.q, X[t], Y[t], Q[t], tab);
-        }
-        __syncwarp();
-    }
-    const int lt_row = lane / T;
-    for (uint32_t c = 0; c < nsrc; c += 32u) {
-        const bool split = nsrc - c <= 16u;   // two lanes a source, half of the targets each
-        const int sl = split ? lane & 15 : lane;
-        const int half = (T + 1) >> 1;
-        const int s0 = split && lane >= 16 ? half : 0, s1 = split && lane < 16 ? half : T;
-        const int base = split ? (lane < 16 ? 0 : kP2PRows) + (sl / T) * T : lt_row * T;
-        const uint32_t slot = c + (uint32_t)sl;
-        const bool has = slot < nsrc;
-        P2PAcc<kField> a = {};
-        uint32_t idx = 0;
-        fmm_p64 S = fmm_p64{0.0, 0.0, 0.0, 0.0};
-        if (has) {
-            uint32_t f = first[0];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) f = slot >= end[i] ? first[i + 1] : f;
-            idx = slot + f;
-            S = sp[idx];
-        }
-        int t = (sl + s0) % T;
-        for (int s = 0; s < (split ? half : T); ++s) {
-            if (has && s0 + s < s1) p2p64_pair<kField>(a, row + base + t, S.x, S.y, S.q, X[t], Y[t], Q[t], tab);
-            t = t + 1 == T ? 0 : t + 1;
-            __syncwarp();
-        }
-        if (split) {
-            a.phi += __shfl_xor_sync(0xffffffffu, a.phi, 16);
-            if constexpr (kField) {
-                a.gx += __shfl_xor_sync(0xffffffffu, a.gx, 16);
-                a.gy += __shfl_xor_sync(0xffffffffu, a.gy, 16);
-            }
-        }
-        if (has && (!split || lane < 16)) p2p64_add<kField>(phi, grad, idx, a);
-    }
-    if (lane < T) {
-        auto sum = [&](int i0, int i1) {
-            for (int i = i0 + lane; i < i1; i += T) {
-                mine.phi += row[i][0];
-                if constexpr (kField) {
-                    mine.gx += row[i][1];
-                    mine.gy += row[i][2];
-                }
-            }
-        };
-        sum(0, kP2PRows);
-        sum(kP2PRows, kP2PRows + kP2PRows2);
-        p2p64_add<kField>(phi, grad, b0 + lane, mine);
-    }
+    auto load = [&](uint32_t i) {
+        const fmm_p64 v = sp[i];
+        return P64{v.x, v.y, 0.0, v.q};
+    };
+    p2p64_block<2, kField, FMM_P2P_BLOCK>(
+        lane, T, true, load(b0 + min(lane, T - 1)), first, end, sh[warp], tab, load,
+        [&](uint32_t i, const P64Acc<kField>& a) { p2p64_add<kField>(phi, grad, i, a); },
+        [&](const P64Acc<kField>& a) { p2p64_add<kField>(phi, grad, b0 + lane, a); });
 }
 
 // phi (and E = -grad phi) in input order

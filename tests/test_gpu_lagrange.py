@@ -191,3 +191,14 @@ def test_literal_form_at_its_deepest_level_runs():
         binding.LagPlan(2, 10, 8, 5.0, "literal_f64")
     with pytest.raises(binding.FmmError):
         binding.LagPlan(3, 10, 6, 5.0, "node_f32")
+
+
+@pytest.mark.parametrize("dim,levels", [(2, 0), (2, 1), (2, 3), (3, 0), (3, 1), (3, 2)])
+@pytest.mark.parametrize("n", [1, 2, 16, 17, 31, 32, 33, 48, 63, 65, 97, 500])
+def test_near_field_tiles_f64(oracle_mod, dim, levels, n):
+    """Target chunks of 1 to 32, source chunks of every remainder, empty cells; pair counts included."""
+    pos, q = inputs.paper_cube(n, 9000 + 100 * dim + n, dim)
+    phi, st, cells = run(pos, q, levels, "node_f64")
+    check_parity(phi, oracle_mod.lag_node(pos, q, levels), TOL64, f"node_f64 tiles D={dim} L={levels} n={n}")
+    near = np.abs(cells[:, None, :] - cells[None, :, :]).max(-1) <= 1
+    assert st["p2p_pairs"] == int(near.sum())
