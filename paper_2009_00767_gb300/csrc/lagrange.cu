@@ -29,12 +29,13 @@
 #include "fmm.h"
 #include "fmm_lagrange.h"
 #include "p2p64.cuh"
+#include "p2p_block.cuh"
 
 namespace {
 
 constexpr int kChunk = 128;      // charges per work item
-constexpr int kWarpChunk = 64;   // targets per FP32 near-field warp work item (two per lane)
-constexpr int kWarpChunk64 = 32;   // and per FP64 one (one per lane)
+constexpr int kWarpChunk = 24;     // targets per near-field warp work item, FP32
+constexpr int kWarpChunk64 = 32;   // and FP64
 constexpr int kMaxLevels = 8;
 constexpr double kLn2 = 0.69314718055994530942;
 
@@ -74,21 +75,14 @@ __host__ __device__ inline double kernel64(int D, double r2) {
 
 constexpr unsigned kFlagOutOfBox = 1u, kFlagNonFinite = 2u;
 
-// The MUFU reciprocal square root and base-2 logarithm with subnormal inputs flushed to zero:
-// a near-field r^2 is never subnormal (coincident pairs give exactly 0, which both map to an
-// infinity that the own cell's mask removes), so the subnormal handling of rsqrtf / __log2f is
-// dead weight in the pair loop.
+// The MUFU reciprocal square root with subnormal inputs flushed to zero: a near-field r^2 is never
+// subnormal (coincident pairs give exactly 0, which maps to an infinity that the own cell's mask
+// removes), so the subnormal handling of rsqrtf is dead weight in the pair loop.
 __device__ __forceinline__ float mufu_rsqrt(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float mufu_lg2(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 }  // namespace
 
 // A sorted charge of the FP64 forms: position and charge, one 32-byte load.
@@ -240,51 +234,23 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 
 // ------------------------------------------------------------------------------ near field
 
-// Sec. 2.1 E-2 in FP32, each pair of adjacent cells evaluated once for both sides.  A warp work
-// item is one chunk of up to 64 targets of a finest cell A, two per lane (i and i + 32), against a
-// group of A's "forward" cells: A itself and the neighbours B whose offset is positive in (z, y, x)
-// order (13 in 3D, 4 in 2D), so that every unordered pair of adjacent cells is met once.  For B != A
-// each 1/r (or log r) feeds the target, q_b / r, and the source, q_a / r: the lanes' source terms of
-// a 32-source tile are summed across the warp by a transposing butterfly (31 shuffles leave lane j
-// with source j's sum), then added to the source in FP64.  A itself is evaluated one-sided with the
-// r > 0 mask (only there can a pair sit at distance 0).  The two targets of a lane run in packed
-// FP32x2 against one source, staged negated and duplicated, (-x, -x, -y, -y), so that every
-// difference is one FADD2; differences come from two-word coordinates, (hi_t - hi_s) + (lo_t - lo_s),
-// so a close pair's distance keeps about 48 bits.  Empty slots hold far zero charges.  Sums are FP32
-// within a tile and FP64 across tiles, and meet in FP64 atomics.
-template <int D, bool kMask>
-__device__ __forceinline__ float2 p2p_tile(const float4* __restrict__ s_a, const float4* __restrict__ s_b,
-                                           const float4* __restrict__ s_c, const float2* __restrict__ s_d, int m,
-                                           float2 tx, float2 ty, float2 tz, float2 ux, float2 uy, float2 uz) {
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int j = 0; j < m; ++j) {
-        const float4 A = s_a[j], B = s_b[j], C = s_c[j];
-        const float2 dx = __fadd2_rn(__fadd2_rn(tx, make_float2(A.x, A.y)), __fadd2_rn(ux, make_float2(C.x, C.y)));
-        const float2 dy = __fadd2_rn(__fadd2_rn(ty, make_float2(A.z, A.w)), __fadd2_rn(uy, make_float2(C.z, C.w)));
-        float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
-        if constexpr (D == 3) {
-            const float2 E = s_d[j];
-            const float2 dz = __fadd2_rn(__fadd2_rn(tz, make_float2(B.x, B.y)), __fadd2_rn(uz, E));
-            r2 = __ffma2_rn(dz, dz, r2);
-        }
-        float2 k;
-        if constexpr (D == 3) {
-            k = make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y));
-        } else {
-            k = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-        }
-        if constexpr (kMask) {
-            k.x = r2.x > 0.f ? k.x : 0.f;
-            k.y = r2.y > 0.f ? k.y : 0.f;
-        }
-        acc = __ffma2_rn(make_float2(B.z, B.w), k, acc);
-    }
-    return acc;
-}
-
-constexpr int kSymTile = 32;     // sources per staged tile (one per lane for the butterfly)
-constexpr int kP2PWarps = 8;     // warps per block, each on its own work items
+// Sec. 2.1 E-2 in FP32, each pair of the own and adjacent cells once for both sides.  A work item of a warp
+// is a chunk of up to kWarpChunk targets of a finest cell A and a group of A's "forward" cells: A itself
+// and the neighbours whose offset is positive in (z, y, x) order (13 in 3D, 4 in 2D), so that every
+// unordered pair of adjacent cells is met once.  Lanes over sources, registers over targets: the group's
+// later sources (A's charges after the chunk, then the forward cells') are walked 32 at a time, one a
+// lane; the targets' coordinates and charges are shared-memory broadcasts, and two targets' arithmetic
+// runs in packed FP32x2.  A pair's 1/r (or log r) feeds a register partial of the target and the sum of the
+// source, which stays in its lane and goes out with one FP64 atomic per lane and 32 sources.  The chunk
+// against itself is one-sided.  Pairs inside A are masked at r = 0 (only there can a pair coincide).
+// Differences come from two-word coordinates, (hi_t - hi_s) + (lo_t - lo_s), so a close pair's distance
+// keeps about 48 bits.  After kP2PRun chunks the lanes' partials of a target are summed across the warp
+// (warp_reduce_scatter) and added in FP64.
+// What bounds it: the FMA pipe, 14 packed instructions (two cycles each) for two targets in 3D, 9 of them
+// the two-word differences; MUFU and issue are at about two thirds of that.  200,000 charges in 3D, levels
+// 3: 486 us against 739 us for 64 targets over the lanes and a butterfly over the lanes per source tile
+// (31 shuffles, 62 selects) for the source's side; 2^20 in 2D, levels 7: 256 against 368 us.
+constexpr int kP2PWarps = 4;     // warps per block, each on its own work items
 template <int D>
 __host__ __device__ constexpr int fwd_group() { return D == 3 ? 4 : 5; }   // forward cells per work item
 
@@ -304,34 +270,152 @@ __device__ __forceinline__ void fwd_offset(int f, int* o) {
     }
 }
 
-// v[j] on every lane in, lane j holds the sum over the warp of v[j] out.
-__device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
+// The later sources of a chunk [t0, t0 + T) of cell b and group g: slot s of range i (end[i - 1] <= s <
+// end[i]) is the sorted charge s + first[i].  Returns the ordered pairs the item covers, both directions
+// of the later pairs and, with the own cell, the chunk's own T^2.
+template <int D>
+__device__ __forceinline__ unsigned long long later_sources(const int* __restrict__ start, int b, int b1, int t0, int T,
+                                                            int g, int side, uint32_t (&first)[5], uint32_t (&end)[5]) {
+    constexpr int F = D == 3 ? 14 : 5, FG = fwd_group<D>();
+    int c[3];
+    morton_dec(D, (uint32_t)b, c);
+    uint32_t slots = 0;
 #pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const bool upper = (lane & w) != 0;
+    for (int i = 0; i < 5; ++i) {
+        const int f = g * FG + i;
+        uint32_t from = 0, count = 0;
+        if (i < FG && f < F) {
+            int o[3];
+            fwd_offset<D>(f, o);
+            const int nc[3] = {c[0] + o[0], c[1] + o[1], c[2] + o[2]};
+            bool in = nc[0] >= 0 && nc[0] < side && nc[1] >= 0 && nc[1] < side;
+            if (D == 3) in = in && nc[2] >= 0 && nc[2] < side;
+            if (f == 0) {
+                from = (uint32_t)(t0 + T);
+                count = (uint32_t)(b1 - t0 - T);
+            } else if (in) {
+                const uint32_t nb = morton_enc(D, nc);
+                from = (uint32_t)start[nb];
+                count = (uint32_t)start[nb + 1] - from;
+            }
+        }
+        first[i] = from - slots;
+        slots += count;
+        end[i] = slots;
+    }
+    return 2ull * slots * (unsigned long long)T + (g == 0 ? (unsigned long long)T * (unsigned long long)T : 0ull);
+}
+
+// FP32 to FP64 by integer operations, off the narrow FP64 pipe (subnormals flush to zero; infinities and
+// NaN stay what they are)
+__device__ __forceinline__ double f2d(float f) {
+    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
+    const uint32_t x = e == 0xffu ? 0x7ffu : e + 896u;
+    return e == 0u ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | (x << 20) | (m >> 3)), (int)((m & 7u) << 29));
+}
+
+// a chunk's targets in pairs: {x, x, y, y}, {z, z, q, q} (high words), {x, x, y, y} and {z, z} (low words)
+template <int D>
+struct LagTargets {
+    float4 xy[kWarpChunk / 2], zq[kWarpChunk / 2], lxy[kWarpChunk / 2];
+    float2 lz[D == 3 ? kWarpChunk / 2 : 1];
+};
+
+// the lane's source (h, l) against the chunk's 2 NP targets; returns the source's sum
+template <int D, bool kMask, int NP>
+__device__ __forceinline__ float p2p_lag_chunk(float2 (&part)[NP], const LagTargets<D>& tg, float4 h, float4 l) {
+    const float2 nx = make_float2(-h.x, -h.x), ny = make_float2(-h.y, -h.y), nz = make_float2(-h.z, -h.z);
+    const float2 mx = make_float2(-l.x, -l.x), my = make_float2(-l.y, -l.y), mz = make_float2(-l.z, -l.z);
+    const float2 q2 = make_float2(h.w, h.w);
+    float2 sacc = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < w; ++i) {
-            const float send = upper ? v[i] : v[i + w];
-            const float keep = upper ? v[i + w] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+    for (int t = 0; t < NP; ++t) {
+        const float4 A = tg.xy[t], B = tg.zq[t], C = tg.lxy[t];
+        const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), nx), __fadd2_rn(make_float2(C.x, C.y), mx));
+        const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), ny), __fadd2_rn(make_float2(C.z, C.w), my));
+        float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+        if constexpr (D == 3) {
+            const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), nz), __fadd2_rn(tg.lz[t], mz));
+            r2 = __ffma2_rn(dz, dz, r2);
+        }
+        float2 k = D == 3 ? make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y))
+                          : make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
+        if constexpr (kMask) {
+            k.x = r2.x > 0.f ? k.x : 0.f;
+            k.y = r2.y > 0.f ? k.y : 0.f;
+        }
+        part[t] = __ffma2_rn(q2, k, part[t]);
+        sacc = __ffma2_rn(make_float2(B.z, B.w), k, sacc);
+    }
+    return sacc.x + sacc.y;
+}
+
+// one work item: the sum of target `lane` (units of 1 / r or log2 r^2), the later sources' added to nearf
+template <int D, int NP>
+__device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, const float4* __restrict__ lo, int t0,
+                                               int T, bool self, const uint32_t (&first)[5], const uint32_t (&end)[5],
+                                               uint32_t n_own, const LagTargets<D>& tg, float far, int lane,
+                                               double* __restrict__ nearf) {
+    constexpr int W = NP <= 2 ? 4 : (NP <= 4 ? 8 : (NP <= 8 ? 16 : 32));
+    const float4 far4 = make_float4(far, far, far, 0.f), zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 part[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
+    double acc = 0.0;
+    if (self) {
+        const bool have = lane < T;
+        p2p_lag_chunk<D, true, NP>(part, tg, have ? hi[t0 + lane] : far4, have ? lo[t0 + lane] : zero4);
+    }
+    const uint32_t nsrc = end[4];
+    auto load = [&](uint32_t slot, float4& h, float4& l, uint32_t& idx) {
+        h = far4;
+        l = zero4;
+        idx = 0xffffffffu;
+        if (slot < nsrc) {
+            uint32_t f = first[0];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) f = slot >= end[i] ? first[i + 1] : f;
+            idx = slot + f;
+            h = hi[idx];
+            l = lo[idx];
+        }
+    };
+    float4 h, l;
+    uint32_t idx;
+    load((uint32_t)lane, h, l, idx);
+    int run = 0;
+#pragma unroll 1
+    for (uint32_t c = 0; c < nsrc; c += 32u) {
+        float4 nh, nl;
+        uint32_t nidx;
+        load(c + 32u + (uint32_t)lane, nh, nl, nidx);   // the next chunk's loads are in flight meanwhile
+        const float v = c < n_own ? p2p_lag_chunk<D, true, NP>(part, tg, h, l) : p2p_lag_chunk<D, false, NP>(part, tg, h, l);
+        if (idx != 0xffffffffu) atomicAdd(nearf + idx, f2d(v));
+        h = nh;
+        l = nl;
+        idx = nidx;
+        if (++run == kP2PRun) {
+            acc += f2d(warp_reduce_scatter<W, NP>(part, lane));
+#pragma unroll
+            for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
+            run = 0;
         }
     }
-    return v[0];
+    return acc + f2d(warp_reduce_scatter<W, NP>(part, lane));
 }
 
 template <int D>
-__global__ void __launch_bounds__(kP2PWarps * 32) k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo,
-                                                          const int* __restrict__ start,
-                                                          const int* __restrict__ wchunk_start, int nleaf, int L,
-                                                          double* __restrict__ nearf,
-                                                          unsigned long long* __restrict__ pairs,
-                                                          int* __restrict__ next_item) {
+__global__ void __launch_bounds__(kP2PWarps * 32, D == 3 ? 5 : 6)
+k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int* __restrict__ start,
+        const int* __restrict__ wchunk_start, int nleaf, int L, float box, double* __restrict__ nearf,
+        unsigned long long* __restrict__ pairs, int* __restrict__ next_item) {
     constexpr int F = D == 3 ? 14 : 5, FG = fwd_group<D>(), G = (F + FG - 1) / FG;
-    __shared__ float4 s_a[kP2PWarps][kSymTile], s_b[kP2PWarps][kSymTile], s_c[kP2PWarps][kSymTile];
-    __shared__ float2 s_d[kP2PWarps][kSymTile];
+    __shared__ LagTargets<D> tgts[kP2PWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    LagTargets<D>& tg = tgts[wid];
     const int side = 1 << L;
-    const double scale = D == 2 ? 0.5 * kLn2 : 1.0;
+    // empty source and target slots are zero charges outside the box, away from every charge and each other
+    const float src_far = -0.25f * box, tgt_far = 1.25f * box;
     const int64_t total = (int64_t)wchunk_start[nleaf] * G;
     unsigned long long my_pairs = 0;
     // items are taken from a shared counter, so that the warps finish within one item of each other
@@ -342,76 +426,39 @@ __global__ void __launch_bounds__(kP2PWarps * 32) k_p2p32(const float4* __restri
         if (w >= total) break;
         const int cidx = (int)(w / G), g = (int)(w % G);
         const int b = chunk_leaf(wchunk_start, nleaf, cidx);
-        const int t0 = start[b] + (cidx - wchunk_start[b]) * kWarpChunk, t1 = min(t0 + kWarpChunk, start[b + 1]);
-        const int ia = t0 + lane, ib = ia + 32;
-        const bool va = ia < t1, vb = ib < t1;
-        // an empty target slot is a zero charge far outside the box
-        const float4 far_t = make_float4(-1.0e4f, -1.0e4f, -1.0e4f, 0.f), z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 ha = va ? hi[ia] : far_t, hb = vb ? hi[ib] : far_t;
-        const float4 la = va ? lo[ia] : z4, lb = vb ? lo[ib] : z4;
-        const float2 tx = make_float2(ha.x, hb.x), ty = make_float2(ha.y, hb.y), tz = make_float2(ha.z, hb.z);
-        const float2 ux = make_float2(la.x, lb.x), uy = make_float2(la.y, lb.y), uz = make_float2(la.z, lb.z);
-        const float2 qa = make_float2(ha.w, hb.w);
-        int c[3];
-        morton_dec(D, (uint32_t)b, c);
-        double acc_a = 0.0, acc_b = 0.0;
-#pragma unroll 1
-        for (int f = g * FG; f < min(F, (g + 1) * FG); ++f) {
-            int o[3];
-            fwd_offset<D>(f, o);
-            const int nc[3] = {c[0] + o[0], c[1] + o[1], c[2] + o[2]};
-            if (nc[0] < 0 || nc[0] >= side || nc[1] < 0 || nc[1] >= side) continue;
-            if (D == 3 && (nc[2] < 0 || nc[2] >= side)) continue;
-            const bool own = f == 0;
-            const uint32_t nb = morton_enc(D, nc);
-            const int s0 = start[nb], s1 = start[nb + 1];
-            if (lane == 0) my_pairs += (own ? 1ull : 2ull) * (unsigned long long)(s1 - s0) * (unsigned long long)(t1 - t0);
-            for (int s = s0; s < s1; s += kSymTile) {
-                const int m = min(kSymTile, s1 - s);
-                __syncwarp();
-                {
-                    const bool have = lane < m;
-                    const float4 h = have ? hi[s + lane] : make_float4(1.0e4f, 1.0e4f, 1.0e4f, 0.f);
-                    const float4 l = have ? lo[s + lane] : z4;
-                    s_a[wid][lane] = make_float4(-h.x, -h.x, -h.y, -h.y);
-                    s_b[wid][lane] = make_float4(-h.z, -h.z, h.w, h.w);
-                    s_c[wid][lane] = make_float4(-l.x, -l.x, -l.y, -l.y);
-                    s_d[wid][lane] = make_float2(-l.z, -l.z);
-                }
-                __syncwarp();
-                if (own) {
-                    const float2 a2 = p2p_tile<D, true>(s_a[wid], s_b[wid], s_c[wid], s_d[wid], m, tx, ty, tz, ux, uy, uz);
-                    acc_a += (double)a2.x;
-                    acc_b += (double)a2.y;
-                    continue;
-                }
-                float cs[kSymTile];
-                float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int j = 0; j < kSymTile; ++j) {
-                    const float4 A = s_a[wid][j], B = s_b[wid][j], C = s_c[wid][j];
-                    const float2 dx = __fadd2_rn(__fadd2_rn(tx, make_float2(A.x, A.y)), __fadd2_rn(ux, make_float2(C.x, C.y)));
-                    const float2 dy = __fadd2_rn(__fadd2_rn(ty, make_float2(A.z, A.w)), __fadd2_rn(uy, make_float2(C.z, C.w)));
-                    float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
-                    if constexpr (D == 3) {
-                        const float2 E = s_d[wid][j];
-                        const float2 dz = __fadd2_rn(__fadd2_rn(tz, make_float2(B.x, B.y)), __fadd2_rn(uz, E));
-                        r2 = __ffma2_rn(dz, dz, r2);
-                    }
-                    const float2 k = D == 3 ? make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y))
-                                            : make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-                    acc = __ffma2_rn(make_float2(B.z, B.w), k, acc);
-                    const float2 t = __fmul2_rn(qa, k);
-                    cs[j] = t.x + t.y;
-                }
-                acc_a += (double)acc.x;
-                acc_b += (double)acc.y;
-                const float v = warp_transpose_sum(cs, lane);
-                if (lane < m) atomicAdd(nearf + s + lane, (double)v * scale);
-            }
+        const int b1 = start[b + 1], t0 = start[b] + (cidx - wchunk_start[b]) * kWarpChunk, T = min(kWarpChunk, b1 - t0);
+        uint32_t first[5], end[5];
+        my_pairs += later_sources<D>(start, b, b1, t0, T, g, side, first, end);
+        const uint32_t n_own = g == 0 ? end[0] : 0u;
+        __syncwarp();
+        if (lane < kWarpChunk) {
+            const bool have = lane < T;
+            const float4 h = have ? hi[t0 + lane] : make_float4(tgt_far, tgt_far, tgt_far, 0.f);
+            const float4 l = have ? lo[t0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const int o = lane & 1;
+            float* A = reinterpret_cast<float*>(&tg.xy[lane >> 1]);
+            float* B = reinterpret_cast<float*>(&tg.zq[lane >> 1]);
+            float* C = reinterpret_cast<float*>(&tg.lxy[lane >> 1]);
+            A[o] = h.x;
+            A[2 + o] = h.y;
+            B[o] = h.z;
+            B[2 + o] = h.w;
+            C[o] = l.x;
+            C[2 + o] = l.y;
+            if constexpr (D == 3) reinterpret_cast<float*>(&tg.lz[lane >> 1])[o] = l.z;
         }
-        if (va) atomicAdd(nearf + ia, acc_a * scale);
-        if (vb) atomicAdd(nearf + ib, acc_b * scale);
+        __syncwarp();
+        double acc;
+        const bool self = g == 0;
+        switch ((T + 3) >> 2) {   // the chunk's target pairs, rounded up to an even count
+            case 1: acc = p2p_lag_item<D, 2>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+            case 2: acc = p2p_lag_item<D, 4>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+            case 3: acc = p2p_lag_item<D, 6>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+            case 4: acc = p2p_lag_item<D, 8>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+            case 5: acc = p2p_lag_item<D, 10>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+            default: acc = p2p_lag_item<D, 12>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+        }
+        if (lane < T) atomicAdd(nearf + t0 + lane, acc);
     }
     if (lane == 0 && my_pairs) atomicAdd(pairs, my_pairs);
 }
@@ -449,35 +496,8 @@ k_p2p64(const Pos64* __restrict__ p, const int* __restrict__ start, const int* _
         const int b = chunk_leaf(wchunk_start, nleaf, cidx);
         const int b1 = start[b + 1], t0 = start[b] + (cidx - wchunk_start[b]) * kWarpChunk64;
         const int T = min(kWarpChunk64, b1 - t0);
-        int c[3];
-        morton_dec(D, (uint32_t)b, c);
-        // the group's ranges of later sources: for the own cell (f = 0) its charges after the chunk
-        uint32_t first[5], end[5], slots = 0;
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            const int f = g * FG + i;
-            uint32_t from = 0, count = 0;
-            if (i < FG && f < F) {
-                int o[3];
-                fwd_offset<D>(f, o);
-                const int nc[3] = {c[0] + o[0], c[1] + o[1], c[2] + o[2]};
-                bool in = nc[0] >= 0 && nc[0] < side && nc[1] >= 0 && nc[1] < side;
-                if (D == 3) in = in && nc[2] >= 0 && nc[2] < side;
-                if (f == 0) {
-                    from = (uint32_t)(t0 + T);
-                    count = (uint32_t)(b1 - t0 - T);
-                    my_pairs += (unsigned long long)(b1 - start[b]) * (unsigned long long)T;
-                } else if (in) {
-                    const uint32_t nb = morton_enc(D, nc);
-                    from = (uint32_t)start[nb];
-                    count = (uint32_t)start[nb + 1] - from;
-                    my_pairs += 2ull * count * (unsigned long long)T;
-                }
-            }
-            first[i] = from - slots;
-            slots += count;
-            end[i] = slots;
-        }
+        uint32_t first[5], end[5];
+        my_pairs += later_sources<D>(start, b, b1, t0, T, g, side, first, end);
         auto load = [&](uint32_t i) {
             const Pos64 v = p[i];
             return P64{v.x, v.y, v.z, v.w};
@@ -669,11 +689,12 @@ __global__ void __launch_bounds__(256) k_m2l(const T* __restrict__ K, const T* _
 // ------------------------------------------------------------------------------ evaluation
 
 // Node forms: phi_far(c) = sum_{k=2..L} h_{m_k}(c) . psi_{m_k}, the tensor-product contraction
-// done axis by axis; phi in input order = far + near, written only if the inputs passed.
+// done axis by axis; phi in input order = far + near (nearf in units of near_unit), written only if the
+// inputs passed.
 template <int D, typename T>
 __global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_t n, int L, double box,
-                      LevelPtrs psi, const double* __restrict__ nearf, const int* __restrict__ order,
-                      const unsigned* __restrict__ status, double* __restrict__ phi) {
+                      LevelPtrs psi, const double* __restrict__ nearf, double near_unit,
+                      const int* __restrict__ order, const unsigned* __restrict__ status, double* __restrict__ phi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint32_t key = skey[i];
@@ -712,7 +733,7 @@ __global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_
         far += (double)v;
     }
     if (*(volatile const unsigned*)status != 0u) return;
-    phi[order[i]] = far + nearf[i];
+    phi[order[i]] = fma(near_unit, nearf[i], far);
 }
 
 // ------------------------------------------------------------------------------ literal form
@@ -993,7 +1014,8 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
             pl->p64, pl->start, pl->wchunk_start, (int)pl->nleaf, L, pl->logtab, pl->nearf, pl->pairs, pl->next_item);
     } else {
         k_p2p32<D><<<(unsigned)pl->grid_p2p, kP2PWarps * 32, 0, p2p_st>>>(
-            pl->hi, pl->lo, pl->start, pl->wchunk_start, (int)pl->nleaf, L, pl->nearf, pl->pairs, pl->next_item);
+            pl->hi, pl->lo, pl->start, pl->wchunk_start, (int)pl->nleaf, L, (float)pl->box, pl->nearf, pl->pairs,
+            pl->next_item);
     }
     ++launches;
     cudaEventRecord(pl->ev[6], p2p_st);
@@ -1036,10 +1058,10 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
         cudaStreamWaitEvent(st, pl->ev_join, 0);
         if (f64)
             k_l2p<D, double><<<gb, 256, 0, st>>>(PosReader<double>{pl->p64}, pl->skey, n, L, pl->box, pots, pl->nearf,
-                                                 pl->order, pl->status, phi);
-        else
+                                                 1.0, pl->order, pl->status, phi);
+        else   // the FP32 near field is in units of 1 / r, or log2 r^2
             k_l2p<D, float><<<gb, 256, 0, st>>>(PosReader<float>{pl->hi, pl->lo}, pl->skey, n, L, pl->box, pots,
-                                                pl->nearf, pl->order, pl->status, phi);
+                                                pl->nearf, D == 2 ? 0.5 * kLn2 : 1.0, pl->order, pl->status, phi);
         ++launches;
     } else if (L < 2) {
         // no interaction lists: phi is the near field (the node evaluation over no levels)
@@ -1047,7 +1069,7 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
         cudaEventRecord(pl->ev[3], st);
         cudaStreamWaitEvent(st, pl->ev_join, 0);
         k_l2p<D, double><<<gb, 256, 0, st>>>(PosReader<double>{pl->p64}, pl->skey, n, L, pl->box, pots, pl->nearf,
-                                             pl->order, pl->status, phi);
+                                             1.0, pl->order, pl->status, phi);
         ++launches;
     } else {
         // U-bar-1: v of every finest cell from the charges' root-node images

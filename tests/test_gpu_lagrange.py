@@ -202,3 +202,22 @@ def test_near_field_tiles_f64(oracle_mod, dim, levels, n):
     check_parity(phi, oracle_mod.lag_node(pos, q, levels), TOL64, f"node_f64 tiles D={dim} L={levels} n={n}")
     near = np.abs(cells[:, None, :] - cells[None, :, :]).max(-1) <= 1
     assert st["p2p_pairs"] == int(near.sum())
+
+
+@pytest.mark.parametrize("dim,levels", [(2, 0), (2, 1), (3, 0), (3, 1)])
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 23, 24, 25, 31, 32, 33, 49, 56, 57, 90, 700, 1500])
+def test_near_field_tiles_f32(oracle_mod, dim, levels, n):
+    """Target chunks of 1 to 24, source chunks of every remainder, more than one run of chunks, a coincident pair;
+    no far field at these levels.  A term's error: MUFU lg2 (2^-22 absolute) or rsqrt (2^-22.4 relative), r^2 to
+    2^-22 relative, and the FP32 sums of at most 16 x 12 terms below that of one term each: together within 2^-20
+    of |q_j| (|K_ij| + 1) summed over the sources."""
+    pos, q = inputs.paper_cube(n, 9500 + 100 * dim + n, dim)
+    if n > 8:
+        pos[n - 1] = pos[0]
+    phi, st, cells = run(pos, q, levels, "node_f32")
+    d = np.linalg.norm(pos[:, None, :] - pos[None, :, :], axis=-1)
+    apart = d > 0.0
+    k = np.where(apart, np.log(np.where(apart, d, 1.0)) if dim == 2 else 1.0 / np.where(apart, d, 1.0), 0.0)
+    bound = 2.0 ** -20 * ((np.abs(k) + 1.0) * np.abs(q)[None, :]).sum(1)
+    assert np.all(np.abs(phi - (k * q[None, :]).sum(1)) <= bound)
+    assert st["p2p_pairs"] == int((np.abs(cells[:, None, :] - cells[None, :, :]).max(-1) <= 1).sum())
