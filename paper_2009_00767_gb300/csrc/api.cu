@@ -80,6 +80,9 @@ void build_far_tables(int p, std::vector<double>& tab) {
 
 bool valid_precision(int v) { return v >= FMM_FP64 && v <= FMM_MIXED_BF16X2; }
 
+// what fmm_sync copies: the counters and the status word after them
+constexpr size_t kSyncBytes = (2 * FMM_COUNTER_SLOTS + 1) * sizeof(unsigned long long);
+
 // fmm_potential_host: inputs of at least kHostChunkMin particles go up in kHostChunks chunks
 constexpr size_t kHostChunkMin = 1 << 16;
 constexpr int kHostChunks = 4;
@@ -121,7 +124,6 @@ void free_plan(fmm_plan_s* pl) {
                     pl->blk_map, pl->sorted_key,
                     pl->sorted64, pl->sorted32, pl->sorted_lo, pl->phi_far, pl->near_grad, pl->far_part,
                     pl->ftab, pl->logtab, pl->T32, pl->U32,
-                    pl->d_status,
                     pl->d_counters, pl->d_xy_stage[0], pl->d_q_stage[0], pl->d_phi_stage[0], pl->d_xy_stage[1],
                     pl->d_q_stage[1], pl->d_phi_stage[1]};
     for (void* b : bufs)
@@ -132,11 +134,11 @@ void free_plan(fmm_plan_s* pl) {
         if (pl->grids.A32[k]) cudaFree(pl->grids.A32[k]);
     }
     fmm_tc_destroy(pl);
-    if (pl->h_status) cudaFreeHost(pl->h_status);
     if (pl->h_counters) cudaFreeHost(pl->h_counters);
     if (pl->crowd_hint_h) cudaFreeHost(pl->crowd_hint_h);
-    for (int e = 0; e < fmm_plan_s::kEvents; ++e)
-        if (pl->ev[e]) cudaEventDestroy(pl->ev[e]);
+    for (auto& set : pl->ev_sets)
+        for (cudaEvent_t e : set)
+            if (e) cudaEventDestroy(e);
     if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
     if (pl->ev_join) cudaEventDestroy(pl->ev_join);
     if (pl->ev_join3) cudaEventDestroy(pl->ev_join3);
@@ -198,10 +200,10 @@ fmm_status enqueue(fmm_plan_s* pl, const double* xy, const double* q, double* ph
     }
     int launches = fmm_launch_sort(pl, xy, q, field != nullptr && pl->precision != FMM_FP64, binned);
     if (launches < 0) return FMM_ERR_CUDA;
-    if (pl->ev_sorted) {
-        // the inputs, keys, ranks and populations are free for the next host call's uploads
+    if (binned || pl->host_used) {
+        // the keys, ranks and populations (and a host call's inputs) are free for the next host call's uploads
         if (cudaEventRecord(pl->ev_sorted, pl->stream) != cudaSuccess ||
-            cudaEventRecord(pl->ev_stage_free[pl->stage_next], pl->stream) != cudaSuccess)
+            (binned && cudaEventRecord(pl->ev_stage_free[pl->stage_next], pl->stream) != cudaSuccess))
             return FMM_ERR_CUDA;
     }
     if (binned) launches += pl->host_chunks;   // the binning kernels of the chunks
@@ -212,6 +214,39 @@ fmm_status enqueue(fmm_plan_s* pl, const double* xy, const double* q, double* ph
     pl->events_recorded = 1;
     if (pl->precision != FMM_FP64) pl->clean = 1;
     return FMM_OK;
+}
+
+// the stage times of the last synced call into plan->last
+void read_times(fmm_plan_s* plan) {
+    DeviceGuard g(plan->device);
+    auto span = [&](int a, int b) -> double {
+        float t = 0.f;
+        return cudaEventElapsedTime(&t, plan->last_ev[a], plan->last_ev[b]) == cudaSuccess ? (double)t : 0.0;
+    };
+    const int kb = plan->last_kernels;
+    plan->last.ms_total = span(0, 5);
+    plan->last.ms_sort = span(0, 1);
+    plan->last.ms_m2l_tc = (kb & 1) ? span(6, 7) : 0.0;
+    plan->last.ms_p2p_kernel = (kb & 2) ? span(8, 9) : 0.0;
+    if (plan->precision == FMM_FP64) {
+        plan->last.ms_p2m = span(1, 2);
+        plan->last.ms_m2l = span(2, 3);
+        plan->last.ms_l2p = span(3, 4);
+        plan->last.ms_p2p = span(4, 5);
+        plan->last.ms_p2m_fine = plan->last.ms_p2m_coarse = plan->last.ms_m2l_coarse = 0.0;
+        plan->last.ms_m2l_fine = plan->last.ms_m2l;
+    } else {
+        // three streams overlap: each stage is the sum of its kernels' own spans
+        plan->last.ms_p2m_fine = span(1, 2);
+        plan->last.ms_p2m_coarse = (kb & 4) ? span(10, 11) : 0.0;
+        plan->last.ms_m2l_fine = span(14, 3);
+        plan->last.ms_m2l_coarse = (kb & 8) ? span(11, 13) : 0.0;
+        plan->last.ms_p2m = plan->last.ms_p2m_fine + plan->last.ms_p2m_coarse;
+        plan->last.ms_m2l = plan->last.ms_m2l_fine + plan->last.ms_m2l_coarse;
+        plan->last.ms_l2p = span(4, 5) + ((kb & 16) ? span(15, 16) : 0.0);
+        plan->last.ms_p2p = plan->last.ms_p2p_kernel;
+    }
+    plan->last_ev = nullptr;
 }
 
 }  // namespace
@@ -362,25 +397,23 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         if (cudaMemcpy(pl->U32, U.data(), sizeof(float2) * U.size(), cudaMemcpyHostToDevice) != cudaSuccess)
             FMM_TRY(FMM_ERR_CUDA);
     }
-    FMM_TRY(dev_alloc(pl, &pl->d_status, sizeof(unsigned int)));
-    FMM_TRY(dev_alloc(pl, &pl->d_counters, 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long)));
-    if (cudaMemset(pl->d_status, 0, sizeof(unsigned int)) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
+    FMM_TRY(dev_alloc(pl, &pl->d_counters, kSyncBytes));
+    pl->d_status = reinterpret_cast<unsigned int*>(pl->d_counters + 2 * FMM_COUNTER_SLOTS);
+    if (cudaMemset(pl->d_counters, 0, kSyncBytes) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
     if (cudaHostAlloc(reinterpret_cast<void**>(&pl->crowd_hint_h), sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void**>(&pl->crowd_hint_d), pl->crowd_hint_h, 0) != cudaSuccess)
         FMM_TRY(FMM_ERR_CUDA);
     *pl->crowd_hint_h = 0;
-    if (cudaMallocHost(reinterpret_cast<void**>(&pl->h_status), sizeof(unsigned int)) != cudaSuccess)
-        FMM_TRY(FMM_ERR_OOM);
-    if (cudaMallocHost(reinterpret_cast<void**>(&pl->h_counters), 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long)) !=
-        cudaSuccess)
-        FMM_TRY(FMM_ERR_OOM);
+    if (cudaMallocHost(reinterpret_cast<void**>(&pl->h_counters), kSyncBytes) != cudaSuccess) FMM_TRY(FMM_ERR_OOM);
     for (int b = 0; b < 2; ++b) {
         FMM_TRY(dev_alloc(pl, &pl->d_xy_stage[b], sizeof(double) * 2 * n));
         FMM_TRY(dev_alloc(pl, &pl->d_q_stage[b], sizeof(double) * n));
         FMM_TRY(dev_alloc(pl, &pl->d_phi_stage[b], sizeof(double) * n));
     }
-    for (int e = 0; e < fmm_plan_s::kEvents; ++e)
-        if (cudaEventCreate(&pl->ev[e]) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
+    for (auto& set : pl->ev_sets)
+        for (cudaEvent_t& e : set)
+            if (cudaEventCreate(&e) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
+    pl->ev = pl->ev_sets[0];
     if (precision != FMM_FP64) {
         // the mixed path's near field and coarse levels run on streams of the plan's own
         if (cudaStreamCreateWithFlags(&pl->stream2, cudaStreamNonBlocking) != cudaSuccess ||
@@ -461,6 +494,9 @@ fmm_status fmm_potential_host_async(fmm_plan_t plan, const double* xy_host, cons
         // Plan's stream: the rest of the method once the uploads are in (and, before L2P writes this
         // set's phi, once the call two back has downloaded it).  Download stream: phi, after L2P.
         cudaStream_t up = plan->s_up, down = plan->s_down;
+        // the plan's first host call waits for all of the device-array calls before it, not for their sorts
+        if (!plan->host_used && cudaEventRecord(plan->ev_sorted, st) != cudaSuccess) return FMM_ERR_CUDA;
+        plan->host_used = 1;
         if (cudaStreamWaitEvent(up, plan->ev_stage_free[b], 0) != cudaSuccess ||
             cudaStreamWaitEvent(up, plan->ev_sorted, 0) != cudaSuccess)
             return FMM_ERR_CUDA;
@@ -494,6 +530,7 @@ fmm_status fmm_potential_host_async(fmm_plan_t plan, const double* xy_host, cons
             return FMM_ERR_CUDA;
     }
     plan->stage_next = b ^ 1;
+    plan->host_pending = 1;
     return FMM_OK;
 }
 
@@ -507,42 +544,15 @@ fmm_status fmm_sync(fmm_plan_t plan) {
     if (!plan) return FMM_ERR_INVALID_ARG;
     DeviceGuard g(plan->device);
     cudaStream_t st = plan->stream;
-    if (cudaMemcpyAsync(plan->h_status, plan->d_status, sizeof(unsigned int), cudaMemcpyDeviceToHost, st) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(plan->h_counters, plan->d_counters, 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long),
-                        cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemsetAsync(plan->d_status, 0, sizeof(unsigned int), st) != cudaSuccess)
+    if (cudaMemcpyAsync(plan->h_counters, plan->d_counters, kSyncBytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return FMM_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return FMM_ERR_CUDA;
-    if (plan->s_down && cudaStreamSynchronize(plan->s_down) != cudaSuccess) return FMM_ERR_CUDA;
+    if (plan->host_pending && plan->s_down && cudaStreamSynchronize(plan->s_down) != cudaSuccess) return FMM_ERR_CUDA;
+    plan->host_pending = 0;
     if (plan->events_recorded) {
-        auto span = [&](int a, int b) -> double {
-            float t = 0.f;
-            return cudaEventElapsedTime(&t, plan->ev[a], plan->ev[b]) == cudaSuccess ? (double)t : 0.0;
-        };
-        const int kb = plan->ev_kernels;
-        plan->last.ms_total = span(0, 5);
-        plan->last.ms_sort = span(0, 1);
-        plan->last.ms_m2l_tc = (kb & 1) ? span(6, 7) : 0.0;
-        plan->last.ms_p2p_kernel = (kb & 2) ? span(8, 9) : 0.0;
-        if (plan->precision == FMM_FP64) {
-            plan->last.ms_p2m = span(1, 2);
-            plan->last.ms_m2l = span(2, 3);
-            plan->last.ms_l2p = span(3, 4);
-            plan->last.ms_p2p = span(4, 5);
-            plan->last.ms_p2m_fine = plan->last.ms_p2m_coarse = plan->last.ms_m2l_coarse = 0.0;
-            plan->last.ms_m2l_fine = plan->last.ms_m2l;
-        } else {
-            // three streams overlap: each stage is the sum of its kernels' own spans
-            plan->last.ms_p2m_fine = span(1, 2);
-            plan->last.ms_p2m_coarse = (kb & 4) ? span(10, 11) : 0.0;
-            plan->last.ms_m2l_fine = span(14, 3);
-            plan->last.ms_m2l_coarse = (kb & 8) ? span(12, 13) : 0.0;
-            plan->last.ms_p2m = plan->last.ms_p2m_fine + plan->last.ms_p2m_coarse;
-            plan->last.ms_m2l = plan->last.ms_m2l_fine + plan->last.ms_m2l_coarse;
-            plan->last.ms_l2p = span(4, 5) + ((kb & 16) ? span(15, 16) : 0.0);
-            plan->last.ms_p2p = plan->last.ms_p2p_kernel;
-        }
+        plan->last_ev = plan->ev;   // read by fmm_plan_stats; the next calls record the other set
+        plan->last_kernels = plan->ev_kernels;
+        plan->ev = plan->ev_sets[plan->ev == plan->ev_sets[0]];
         plan->ev_kernels = 0;
         unsigned long long pairs = 0, mx = 0;
         for (int c = 0; c < FMM_COUNTER_SLOTS; ++c) {
@@ -554,7 +564,10 @@ fmm_status fmm_sync(fmm_plan_t plan) {
         plan->last.kernel_launches = plan->launches;
         plan->events_recorded = 0;
     }
-    const unsigned int f = *plan->h_status;
+    const unsigned int f = *reinterpret_cast<const unsigned int*>(plan->h_counters + 2 * FMM_COUNTER_SLOTS);
+    if (f != 0u && (cudaMemsetAsync(plan->d_status, 0, sizeof(unsigned int), st) != cudaSuccess ||
+                    cudaStreamSynchronize(st) != cudaSuccess))
+        return FMM_ERR_CUDA;
     if (f & FMM_FLAG_NONFINITE) return FMM_ERR_NONFINITE;
     if (f & FMM_FLAG_OUT_OF_BOX) return FMM_ERR_OUT_OF_BOX;
     if (f & FMM_FLAG_TIMEOUT) return FMM_ERR_TIMEOUT;
@@ -577,6 +590,7 @@ fmm_status fmm_inject_timeout(fmm_plan_t plan, int enable) {
 
 fmm_status fmm_plan_stats(fmm_plan_t plan, fmm_stats* out) {
     if (!plan || !out) return FMM_ERR_INVALID_ARG;
+    if (plan->last_ev) read_times(plan);
     *out = plan->last;
     return FMM_OK;
 }

@@ -116,9 +116,9 @@ struct fmm_plan_s {
     FmmTc* tc;          // tensor-core M2L state (TF32 modes), or null
 
     unsigned int* d_status;
-    unsigned long long* d_counters;   // [0..63] near-field pair partials, [64..127] max leaf population
-    unsigned int* h_status;           // pinned
-    unsigned long long* h_counters;   // pinned [128]
+    unsigned long long* d_counters;   // [0..63] near-field pair partials, [64..127] max leaf population; a plan's
+                                      // d_status is the word after them, so that fmm_sync copies both at once
+    unsigned long long* h_counters;   // pinned copy of the counters and the status
     // mixed path: set to 1 by the scan of a call that finds a finest square above FMM_LANE_MAX
     // particles (mapped host memory, read without a sync by the next call's enqueue, which then
     // sums crowded squares' fine-level moments with k_p2m_crowded instead of one warp each)
@@ -133,6 +133,8 @@ struct fmm_plan_s {
     int host_chunks;                         // chunks the current host call binned itself
     cudaStream_t s_up, s_down;               // mixed path: uploads + binning, result downloads
     cudaEvent_t ev_sorted;                   // the sort no longer needs keys, ranks or populations
+    int host_used;                           // a host call has been made: calls record ev_sorted from then on
+    int host_pending;                        // host calls since the last sync (their downloads are waited for)
     cudaEvent_t ev_stage_free[2];            // the set's inputs were consumed (scatter done)
     cudaEvent_t ev_up_done, ev_l2p_done;     // a host call's uploads / compute are complete
     cudaEvent_t ev_down_done[2];             // the set's result was downloaded
@@ -148,11 +150,16 @@ struct fmm_plan_s {
     // Timing events.  FP64 path: stage boundaries [0..5] (sort, P2M, M2L, L2P, P2P).  Mixed path:
     // [0] start, [1] sort done, [2] fine P2M done, [14] fine M2L start, [3] fine M2L done, [4] L2P
     // start (after the joins), [5] end, all on the plan's stream; [6, 7] the tensor-core M2L
-    // kernel; [8, 9] the near-field kernel (stream2); [10, 11] the coarse P2M and its conversion,
-    // [12, 13] the coarse M2L, [15, 16] the coarse levels' L2P (stream3).
+    // kernel; [8, 9] the near-field kernel (stream2); [10, 11] the upward pass, [11, 13] the coarse
+    // M2L, [15, 16] the coarse levels' L2P (stream3).
+    // The calls between two syncs record the set `ev`; fmm_sync then turns to the other one, so that the
+    // times of the last synced call can be read when fmm_plan_stats asks for them.
     static constexpr int kEvents = 17;
-    cudaEvent_t ev[kEvents];
-    int ev_kernels;       // bits: 1 [6, 7], 2 [8, 9], 4 [10, 11], 8 [12, 13], 16 [15, 16] recorded this call
+    cudaEvent_t ev_sets[2][kEvents];
+    cudaEvent_t* ev;
+    int ev_kernels;       // bits: 1 [6, 7], 2 [8, 9], 4 [10, 11], 8 [11, 13], 16 [15, 16] recorded this call
+    cudaEvent_t* last_ev;   // the last synced call's set while its times are unread, else null
+    int last_kernels;       // its ev_kernels
     int serial;           // fmm_set_concurrency(plan, 1): every stage on the plan's stream
     int events_recorded;
     int launches;

@@ -110,6 +110,7 @@ struct fmm_lag_plan_s {
     Pos64* p64 = nullptr;        // FP64 forms
     double* nearf = nullptr;       // [n_max] near field, sorted order
     unsigned* status = nullptr;
+    unsigned* h_status = nullptr;  // pinned
     unsigned long long* pairs = nullptr;   // near-field pair counter
     int* next_item = nullptr;              // near-field work counter
     void* node[kMaxLevels + 1] = {};       // Q_k (node) or v_k (literal), d values per cell
@@ -123,6 +124,7 @@ struct fmm_lag_plan_s {
     uint64_t bytes = 0;
     int launches = 0;
     int grid_particles = 0;
+    cudaStream_t last_st = nullptr;   // the stream of the last call, for comparison only
     bool serial = false;   // every kernel in turn on the plan's stream (per-kernel timing)
     int grid_p2p = 0;      // resident blocks of the form's near-field kernel, all SMs
     double2* logtab = nullptr;   // 2D FP64 forms: the logarithm's table (fp64_math.cuh)
@@ -941,6 +943,7 @@ void plan_free(fmm_lag_plan_s* pl) {
     if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
     if (pl->ev_join) cudaEventDestroy(pl->ev_join);
     if (pl->st2) cudaStreamDestroy(pl->st2);
+    if (pl->h_status) cudaFreeHost(pl->h_status);
     delete pl;
 }
 
@@ -1102,6 +1105,7 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
     cudaEventRecord(pl->ev[4], st);
     pl->launches = launches;
     pl->last_n = n;
+    pl->last_st = st;
     return cuda_status(cudaGetLastError());
 }
 
@@ -1179,6 +1183,7 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
         }
     }
     if (rc == FMM_OK) rc = cuda_status(cudaMemset(pl->status, 0, sizeof(unsigned)));
+    if (rc == FMM_OK) rc = cuda_status(cudaMallocHost(reinterpret_cast<void**>(&pl->h_status), sizeof(unsigned)));
     if (rc == FMM_OK && dim == 3 && f64 && !lit)
         rc = cuda_status(cudaFuncSetAttribute(k_m2l<3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)m2l_smem_bytes<3, double>()));
@@ -1269,12 +1274,14 @@ fmm_status fmm_lag_potential(fmm_lag_plan_t pl, const double* pos, const double*
 
 fmm_status fmm_lag_sync(fmm_lag_plan_t pl) {
     if (!pl) return FMM_ERR_INVALID_ARG;
-    fmm_status rc = cuda_status(cudaStreamSynchronize(pl->st));
-    if (rc == FMM_OK) rc = cuda_status(cudaStreamSynchronize(pl->st2));
+    // a call joins its near field's stream back before the final sum, so its stream is all there is to wait
+    // for; after a change of stream the last call's is waited for as well
+    fmm_status rc = FMM_OK;
+    if (pl->st != pl->last_st) rc = cuda_status(cudaEventSynchronize(pl->ev[4]));
+    if (rc == FMM_OK) rc = cuda_status(cudaMemcpyAsync(pl->h_status, pl->status, sizeof(unsigned), cudaMemcpyDeviceToHost, pl->st));
+    if (rc == FMM_OK) rc = cuda_status(cudaStreamSynchronize(pl->st));
     if (rc != FMM_OK) return rc;
-    unsigned flags = 0;
-    rc = cuda_status(cudaMemcpy(&flags, pl->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (rc != FMM_OK) return rc;
+    const unsigned flags = *pl->h_status;
     if (flags) {
         cudaMemset(pl->status, 0, sizeof(unsigned));
         return (flags & kFlagNonFinite) ? FMM_ERR_NONFINITE : FMM_ERR_OUT_OF_BOX;

@@ -964,7 +964,6 @@ int fmm_launch_mixed(fmm_plan_s* pl, double* phi, double* field) {
         // M2L on the plan's stream reads
         if (kc_max > kw && cudaEventRecord(pl->ev_a32, s3) != cudaSuccess) return -1;
         cudaEventRecord(pl->ev[11], s3);
-        cudaEventRecord(pl->ev[12], s3);
         // coarse levels: a CTA per 4 x kM2LWarpTargets targets of one class
         M2LWarpArgs wa;
         wa.g = pl->grids;

@@ -160,7 +160,7 @@ extern "C" fmm_status fmm_potential_noalloc(int64_t n, int levels, int p, double
     pl.stream = static_cast<cudaStream_t>(stream);
     if (carve(&pl, nullptr) > kScratchBytes) return FMM_ERR_INVALID_ARG;   // cannot happen within the limits
     carve(&pl, static_cast<unsigned char*>(scratch));
-    for (int e = 0; e < 6; ++e) pl.ev[e] = events[e];
+    pl.ev = events;   // the FP64 stages record the first six
 
     // The array keeps the previous call's contents: clear what must start at zero.
     cudaStream_t st = pl.stream;
