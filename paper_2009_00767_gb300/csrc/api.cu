@@ -81,7 +81,7 @@ void build_far_tables(int p, std::vector<double>& tab) {
 bool valid_precision(int v) { return v >= FMM_FP64 && v <= FMM_MIXED_BF16X2; }
 
 // what fmm_sync copies: the counters and the status word after them
-constexpr size_t kSyncBytes = (2 * FMM_COUNTER_SLOTS + 1) * sizeof(unsigned long long);
+constexpr size_t kSyncBytes = (FMM_COUNTERS + 1) * sizeof(unsigned long long);
 
 // fmm_potential_host: inputs of at least kHostChunkMin particles go up in kHostChunks chunks
 constexpr size_t kHostChunkMin = 1 << 16;
@@ -121,7 +121,7 @@ void free_plan(fmm_plan_s* pl) {
     cudaGetDevice(&prev);
     cudaSetDevice(pl->device);
     void* bufs[] = {pl->keys, pl->rank, pl->counts, pl->leaf_start, pl->block_sums, pl->leaf_bstart,
-                    pl->blk_map, pl->sorted_key,
+                    pl->blk_map, pl->crowd_list, pl->sorted_key,
                     pl->sorted64, pl->sorted32, pl->sorted_lo, pl->phi_far, pl->near_grad, pl->far_part,
                     pl->ftab, pl->logtab, pl->T32, pl->U32,
                     pl->d_counters, pl->d_xy_stage[0], pl->d_q_stage[0], pl->d_phi_stage[0], pl->d_xy_stage[1],
@@ -180,7 +180,7 @@ fmm_status reset_accumulators(fmm_plan_s* pl, cudaStream_t st) {
 // the mixed path's accumulators back to zero.
 fmm_status enqueue_prologue(fmm_plan_s* pl) {
     cudaStream_t st = pl->stream;
-    if (cudaMemsetAsync(pl->d_counters, 0, 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long), st) != cudaSuccess)
+    if (cudaMemsetAsync(pl->d_counters, 0, FMM_COUNTERS * sizeof(unsigned long long), st) != cudaSuccess)
         return FMM_ERR_CUDA;
     if (pl->precision != FMM_FP64) {
         if (!pl->clean && reset_accumulators(pl, st) != FMM_OK) return FMM_ERR_CUDA;
@@ -278,6 +278,10 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         delete pl;
         return FMM_ERR_CUDA;
     }
+    if (cudaDeviceGetAttribute(&pl->sms, cudaDevAttrMultiProcessorCount, pl->device) != cudaSuccess) {
+        delete pl;
+        return FMM_ERR_CUDA;
+    }
     pl->n = n;
     pl->levels = levels;
     pl->p = p;
@@ -308,6 +312,7 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         // warps a CTA and every warp reads its entry, so the map is rounded up to four entries
         const size_t nblk = ((size_t)m + (size_t)n / FMM_P2P_BLOCK + 1 + 3) & ~(size_t)3;
         FMM_TRY(dev_alloc(pl, &pl->blk_map, sizeof(uint2) * nblk));
+        if (precision != FMM_FP64) FMM_TRY(dev_alloc(pl, &pl->crowd_list, sizeof(uint2) * fmm_crowd_items(n)));
     }
     FMM_TRY(dev_alloc(pl, &pl->sorted_key, sizeof(uint32_t) * n));
     if (precision == FMM_FP64)
@@ -398,7 +403,7 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
             FMM_TRY(FMM_ERR_CUDA);
     }
     FMM_TRY(dev_alloc(pl, &pl->d_counters, kSyncBytes));
-    pl->d_status = reinterpret_cast<unsigned int*>(pl->d_counters + 2 * FMM_COUNTER_SLOTS);
+    pl->d_status = reinterpret_cast<unsigned int*>(pl->d_counters + FMM_COUNTERS);
     if (cudaMemset(pl->d_counters, 0, kSyncBytes) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
     if (cudaHostAlloc(reinterpret_cast<void**>(&pl->crowd_hint_h), sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void**>(&pl->crowd_hint_d), pl->crowd_hint_h, 0) != cudaSuccess)
@@ -564,7 +569,7 @@ fmm_status fmm_sync(fmm_plan_t plan) {
         plan->last.kernel_launches = plan->launches;
         plan->events_recorded = 0;
     }
-    const unsigned int f = *reinterpret_cast<const unsigned int*>(plan->h_counters + 2 * FMM_COUNTER_SLOTS);
+    const unsigned int f = *reinterpret_cast<const unsigned int*>(plan->h_counters + FMM_COUNTERS);
     if (f != 0u && (cudaMemsetAsync(plan->d_status, 0, sizeof(unsigned int), st) != cudaSuccess ||
                     cudaStreamSynchronize(st) != cudaSuccess))
         return FMM_ERR_CUDA;

@@ -75,6 +75,7 @@ struct BatchArgs {
     unsigned int* status;
     int m2l_kmax;    // levels 2..m2l_kmax of each system run in kb_m2l_f32 (the tensor cores take the rest)
     int p2p_block;   // near-field targets per block (16 or 24)
+    P2PCrowd crowd;  // the near-field blocks with many sources
 };
 
 // largest s with pre[s] <= w, for pre[0] = 0 <= w < pre[nsys]
@@ -476,6 +477,7 @@ __global__ void __launch_bounds__(kT, 8) kb_p2p(BatchArgs a, MixedLevels lv) {
         const uint32_t leaf = (uint32_t)((long long)lt.x - pre[s]);
         const uint32_t* ls = a.leaf_start + S.leaf_off;
         const uint32_t t0 = ls[leaf], t1 = ls[leaf + 1];
+        if (t1 - t0 > (uint32_t)FMM_CROWD_POP) continue;   // in the crowd list: kb_p2p_crowd takes it
         const uint32_t b0 = t0 + (uint32_t)a.p2p_block * lt.y;
         const int T = (int)min((uint32_t)a.p2p_block, t1 - b0);
         const float s_leaf = a.box_ff.x * __int_as_float((127 - S.levels) << 23);
@@ -484,6 +486,30 @@ __global__ void __launch_bounds__(kT, 8) kb_p2p(BatchArgs a, MixedLevels lv) {
                                          seg[warp], lane, a.acc, &pairs);
         if (lane < T) atomicAdd(a.acc + b0 + lane, fmm_f2d_bits(near.x) + fmm_f2d_bits(near.y));
         __syncwarp();   // tgt, tq and seg are rewritten by the next block
+    }
+}
+
+// The squares in the crowd list (p2p_near_crowd), their items taken from a counter by
+// resident warps.
+__global__ void __launch_bounds__(kT, kCrowdBlocksPerSm) kb_p2p_crowd(BatchArgs a) {
+    extern __shared__ long long pre[];
+    __shared__ __align__(16) P2PCrowdShared sh[kT / 32];
+    load_prefix(pre, a.wp_leaf, a.nsys);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned long long total = *a.crowd.count;
+    if (*(volatile const unsigned int*)a.status != 0u) return;   // inputs failed the device checks
+    for (;;) {
+        unsigned long long w = 0;
+        if (lane == 0) w = atomicAdd(a.crowd.count + 1, 1ull);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= total) return;
+        const uint2 it = a.crowd.list[w];
+        const int s = find_sys(pre, a.nsys, (long long)it.x);
+        const BatchSys& S = a.sys[s];
+        const uint32_t leaf = (uint32_t)((long long)it.x - pre[s]);
+        const uint32_t* ls = a.leaf_start + S.leaf_off;
+        const float s_leaf = a.box_ff.x * __int_as_float((127 - S.levels) << 23);
+        p2p_near_crowd(a.sorted32, ls, leaf, ls[leaf], ls[leaf + 1], it.y, S.levels, s_leaf, sh[warp], lane, a.acc);
     }
 }
 
@@ -509,6 +535,8 @@ struct fmm_batch_s {
     BatchCall* h_call;                // pinned
     uint32_t *keys, *rank, *counts, *leaf_start, *block_sums, *sorted_key, *leaf_nb, *bstart;
     uint2* bmap;
+    uint2* crowd_list;
+    unsigned long long* crowd_count;
     float4* sorted32;
     float2 *a32, *b32;
     double* acc;                      // near field per sorted particle
@@ -532,7 +560,7 @@ void batch_free(fmm_batch_s* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     void* bufs[] = {b->d_sys, b->d_pre, b->d_call, b->keys, b->rank, b->counts, b->leaf_start, b->block_sums,
-                    b->leaf_nb, b->bstart, b->bmap,
+                    b->leaf_nb, b->bstart, b->bmap, b->crowd_list, b->crowd_count,
                     b->sorted_key, b->sorted32, b->a32, b->b32, b->acc, b->T32, b->U32, b->d_status};
     fmm_tc_free(b->tc);
     for (void* p : bufs)
@@ -567,7 +595,8 @@ int enqueue_batch_kernels(fmm_batch_s* b, const BatchArgs& a, const MixedLevels&
     const size_t pre_bytes = sizeof(long long) * (b->nsys + 1);
     int launches = 0;
     if (cudaMemsetAsync(b->counts, 0, sizeof(uint32_t) * b->nl, st) != cudaSuccess ||
-        cudaMemsetAsync(b->acc, 0, sizeof(double) * b->nt, st) != cudaSuccess)
+        cudaMemsetAsync(b->acc, 0, sizeof(double) * b->nt, st) != cudaSuccess ||
+        cudaMemsetAsync(b->crowd_count, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess)
         return -1;
     kb_bin<<<grid, kT, pre_bytes, st>>>(a, lv);
     ++launches;
@@ -580,10 +609,11 @@ int enqueue_batch_kernels(fmm_batch_s* b, const BatchArgs& a, const MixedLevels&
     if (st2 != st && (cudaEventRecord(ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(st2, ev_fork, 0) != cudaSuccess))
         return -1;
     const int lb = fmm_launch_leaf_blocks(b->leaf_start, b->nl, (uint32_t)b->p2p_block, b->leaf_nb, b->block_sums,
-                                          b->bstart, b->bmap, st2);
+                                          b->bstart, b->bmap, a.crowd, st2);
     if (lb < 0) return -1;
     kb_p2p<<<grid, kT, pre_bytes, st2>>>(a, lv);
-    launches += lb + 1;
+    kb_p2p_crowd<<<(unsigned)(sms * kCrowdBlocksPerSm), kT, pre_bytes, st2>>>(a);
+    launches += lb + 2;
     if (st2 != st && cudaEventRecord(ev_join, st2) != cudaSuccess) return -1;
     kb_p2m_fine<P1B><<<grid, kT, pre_bytes, st>>>(a, lv);
     ++launches;
@@ -637,6 +667,7 @@ int enqueue_all(fmm_batch_s* b, cudaStream_t st, cudaStream_t st2, cudaEvent_t e
     a.status = b->d_status;
     a.m2l_kmax = b->tc ? fmm_tc_kmin() - 1 : FMM_MAX_LEVELS;
     a.p2p_block = b->p2p_block;
+    a.crowd = {b->crowd_count, b->crowd_list};
     fmm_plan_s shim{};
     shim.box = b->box;
     shim.levels = 0;
@@ -853,7 +884,8 @@ fmm_status fmm_batch_plan(fmm_batch_t* out, int nsys, const int64_t* n, const in
               balloc(b, &b->block_sums, 4 * ((size_t)fmm_scan_blocks(nl) + 1)) && balloc(b, &b->sorted_key, 4 * nt) &&
               balloc(b, &b->leaf_nb, 4 * nl) && balloc(b, &b->bstart, 4 * (nl + 1)) &&
               balloc(b, &b->bmap, sizeof(uint2) * ((size_t)nl + (size_t)nt / kP2PBlockMin + 1)) &&
-              balloc(b, &b->sorted32, 16 * nt) &&
+              balloc(b, &b->crowd_list, sizeof(uint2) * fmm_crowd_items(nt)) &&
+              balloc(b, &b->crowd_count, 2 * sizeof(unsigned long long)) && balloc(b, &b->sorted32, 16 * nt) &&
               balloc(b, &b->a32, sizeof(float2) * b->a_cells * p1) && balloc(b, &b->b32, sizeof(float2) * bcells * p1) &&
               balloc(b, &b->acc, sizeof(double) * nt) && balloc(b, &b->d_status, sizeof(unsigned int));
     if (!ok) {

@@ -43,6 +43,7 @@ struct __align__(32) fmm_p64 {
 // Near-field statistics are spread over this many counter slots (one update per CTA each) so
 // that no single L2 address serialises the updates.
 #define FMM_COUNTER_SLOTS 64
+#define FMM_COUNTERS (2 * FMM_COUNTER_SLOTS + 2)
 #define FMM_LANE_MAX 128   // finest squares above this many particles are "crowded" in the fine P2M
 
 // Conversions between FP32 and FP64 by integer bit operations, so that they do not occupy
@@ -96,6 +97,8 @@ struct fmm_plan_s {
     int scan_blocks;
     uint32_t* leaf_bstart;       // near-field target blocks: exclusive scan over the squares, 4^levels + 1
     uint2* blk_map;              // near-field block -> (square, block inside it)
+    uint2* crowd_list;           // mixed path: near-field items of squares with many sources (p2p_block.cuh)
+    int sms;                     // multiprocessors of the device
     int clean;                   // mixed path: the square populations are zero (each call's scan
                                  // leaves them so; a call that failed to enqueue does not)
     uint32_t* sorted_key;
@@ -116,7 +119,8 @@ struct fmm_plan_s {
     FmmTc* tc;          // tensor-core M2L state (TF32 modes), or null
 
     unsigned int* d_status;
-    unsigned long long* d_counters;   // [0..63] near-field pair partials, [64..127] max leaf population; a plan's
+    unsigned long long* d_counters;   // [0..63] near-field pair partials, [64..127] max leaf population,
+                                      // [128] items in crowd_list, [129] items taken from it; a plan's
                                       // d_status is the word after them, so that fmm_sync copies both at once
     unsigned long long* h_counters;   // pinned copy of the counters and the status
     // mixed path: set to 1 by the scan of a call that finds a finest square above FMM_LANE_MAX
@@ -253,6 +257,32 @@ static __device__ __forceinline__ float2 scatter_mul(float a, float2 s) {
 }
 
 
+// Near field of crowded squares (p2p_near_crowd): squares above FMM_CROWD_POP particles go to a list, and
+// the kernels over the block map skip them.  At 16 particles a square none does; above 64 the block of 32
+// targets and steps of 64 sources fill.  A square's work items are its blocks of up to kCrowdTargets targets
+// of (almost) equal size, each split by its sources into the same number of parts (one per kCrowdPart
+// particles of the square, about a fifth of the block's sources); item i is part i % parts of block i / parts.
+#define FMM_CROWD_POP 64
+constexpr int kCrowdTargets = 32, kCrowdParts = 4;
+constexpr uint32_t kCrowdPart = 1024;
+struct P2PCrowd {
+    unsigned long long* count;   // items in the list; the next word counts the items taken from it
+    uint2* list;                 // (square, item of the square)
+};
+__host__ __device__ inline uint32_t fmm_crowd_blocks(uint32_t n) { return (n + kCrowdTargets - 1) / kCrowdTargets; }
+__host__ __device__ inline uint32_t fmm_crowd_parts(uint32_t n) {
+    const uint32_t p = (n + kCrowdPart - 1) / kCrowdPart;
+    return p < (uint32_t)kCrowdParts ? p : (uint32_t)kCrowdParts;
+}
+// square `id` of n particles into the list
+static __device__ __forceinline__ void fmm_crowd_add(P2PCrowd c, uint32_t id, uint32_t n) {
+    const uint32_t items = fmm_crowd_blocks(n) * fmm_crowd_parts(n);
+    const unsigned long long at = atomicAdd(c.count, (unsigned long long)items);
+    for (uint32_t i = 0; i < items; ++i) c.list[at + i] = make_uint2(id, i);
+}
+// items of n particles at most: the blocks of crowded squares hold at least half of kCrowdTargets
+inline size_t fmm_crowd_items(int64_t n) { return (size_t)kCrowdParts * ((size_t)n / (kCrowdTargets / 2) + 1); }
+
 // --- launchers (each returns the number of kernels it launched, or -1 on a launch error) ---------
 // with_lo: also the rounding residues of the mixed path's local coordinates (sorted_lo); binned: the
 // particles were already binned (fmm_launch_bin_range over all of them)
@@ -262,9 +292,10 @@ int fmm_scan_blocks(int64_t m);
 int fmm_launch_scan(const uint32_t* counts, int64_t m, uint32_t* block_sums, uint32_t* leaf_start, uint32_t n_total,
                     cudaStream_t st);
 // Near-field target blocks: nb[i] = ceil(population of square i / block), bstart = their exclusive
-// scan (m + 1 entries), and, if map is not null, map[b] = (square, index of b inside it).
+// scan (m + 1 entries), and, if map is not null, map[b] = (square, index of b inside it) and the crowded
+// squares' items in the crowd list.
 int fmm_launch_leaf_blocks(const uint32_t* leaf_start, int64_t m, uint32_t block, uint32_t* nb, uint32_t* block_sums,
-                           uint32_t* bstart, uint2* map, cudaStream_t st);
+                           uint32_t* bstart, uint2* map, P2PCrowd crowd, cudaStream_t st);
 // targets per near-field block of the mixed path (the batched form uses 32)
 #define FMM_P2P_BLOCK 24
 

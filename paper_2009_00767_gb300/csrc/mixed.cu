@@ -757,6 +757,7 @@ k_p2p_mixed(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
     if (*(volatile const unsigned int*)status != 0u) return;   // inputs failed the device checks
     const uint32_t leaf = lt.x;
     const uint32_t t0 = leaf_start[leaf], t1 = leaf_start[leaf + 1];
+    if (t1 - t0 > (uint32_t)FMM_CROWD_POP) return;   // in the crowd list: k_p2p_crowd takes it
     const uint32_t b0 = t0 + (uint32_t)FMM_P2P_BLOCK * lt.y;
     const int T = (int)min((uint32_t)FMM_P2P_BLOCK, t1 - b0);
     uint32_t pairs;
@@ -768,6 +769,33 @@ k_p2p_mixed(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
         atomicMax(&counters[FMM_COUNTER_SLOTS + slot], (unsigned long long)(t1 - t0));
     }
     if (lane < T) atomicAdd(acc + b0 + lane, fmm_f2d_bits(near.x) + fmm_f2d_bits(near.y));
+}
+
+// The squares that the sort put into the crowd list (p2p_near_crowd): resident warps take their items from
+// a counter, so that they finish within one item of each other whatever the squares' sizes.
+__global__ void __launch_bounds__(kP2PWarps * 32, kCrowdBlocksPerSm)
+k_p2p_crowd(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_start, int levels, float s_leaf,
+            double* __restrict__ acc, P2PCrowd crowd, const unsigned int* __restrict__ status,
+            unsigned long long* __restrict__ counters) {
+    __shared__ __align__(16) P2PCrowdShared sh[kP2PWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned long long total = *crowd.count;
+    if (total == 0ull || *(volatile const unsigned int*)status != 0u) return;   // none, or the inputs failed the checks
+    for (;;) {
+        unsigned long long w = 0;
+        if (lane == 0) w = atomicAdd(crowd.count + 1, 1ull);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (w >= total) return;
+        const uint2 it = crowd.list[w];
+        const uint32_t t0 = leaf_start[it.x], t1 = leaf_start[it.x + 1];
+        const unsigned long long pairs =
+            p2p_near_crowd(sp, leaf_start, it.x, t0, t1, it.y, levels, s_leaf, sh[warp], lane, acc);
+        if (lane == 0) {
+            const unsigned slot = it.x % FMM_COUNTER_SLOTS;
+            atomicAdd(&counters[slot], pairs);
+            atomicMax(&counters[FMM_COUNTER_SLOTS + slot], (unsigned long long)(t1 - t0));
+        }
+    }
 }
 
 // The near field with the gradient (fmm_potential_field): p2p_near_sym_field, the gradient sums
@@ -832,13 +860,17 @@ int fmm_launch_p2p_concurrent(fmm_plan_s* pl, const MixedLevels& lv, bool with_f
         k_p2p_field<<<blocks, kP2PWarps * 32, 0, s2>>>(pl->sorted32, pl->leaf_start, pl->leaf_bstart, pl->blk_map,
                                                       nleaf, L, lv.s_leaf, pl->sorted_lo, pl->phi_far, pl->near_grad,
                                                       pl->d_status, pl->d_counters);
-    else
+    else {
+        const P2PCrowd crowd = {pl->d_counters + 2 * FMM_COUNTER_SLOTS, pl->crowd_list};
         k_p2p_mixed<<<blocks, kP2PWarps * 32, 0, s2>>>(pl->sorted32, pl->leaf_start, pl->leaf_bstart, pl->blk_map,
                                                       nleaf, L, lv.s_leaf, pl->phi_far, pl->d_status, pl->d_counters);
+        k_p2p_crowd<<<(unsigned)(pl->sms * kCrowdBlocksPerSm), kP2PWarps * 32, 0, s2>>>(
+            pl->sorted32, pl->leaf_start, L, lv.s_leaf, pl->phi_far, crowd, pl->d_status, pl->d_counters);
+    }
     cudaEventRecord(pl->ev[9], s2);
     pl->ev_kernels |= 2;
     if (cudaEventRecord(pl->ev_join, s2) != cudaSuccess) return -1;
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    return cudaGetLastError() == cudaSuccess ? (with_field ? 1 : 2) : -1;
 }
 
 namespace {

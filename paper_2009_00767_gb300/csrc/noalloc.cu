@@ -105,7 +105,7 @@ size_t carve(fmm_plan_s* pl, unsigned char* base) {
     pl->ftab = reinterpret_cast<double*>(take(sizeof(double) * fmm_far_table_doubles(p1)));
     pl->logtab = reinterpret_cast<double2*>(take(sizeof(double2) * kFmmLogEntries));
     pl->d_status = reinterpret_cast<unsigned int*>(take(sizeof(unsigned int)));
-    pl->d_counters = reinterpret_cast<unsigned long long*>(take(2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long)));
+    pl->d_counters = reinterpret_cast<unsigned long long*>(take(FMM_COUNTERS * sizeof(unsigned long long)));
     return off;
 }
 
@@ -165,7 +165,7 @@ extern "C" fmm_status fmm_potential_noalloc(int64_t n, int levels, int p, double
     // The array keeps the previous call's contents: clear what must start at zero.
     cudaStream_t st = pl.stream;
     if (cudaMemsetAsync(pl.d_status, 0, sizeof(unsigned int), st) != cudaSuccess ||
-        cudaMemsetAsync(pl.d_counters, 0, 2 * FMM_COUNTER_SLOTS * sizeof(unsigned long long), st) != cudaSuccess)
+        cudaMemsetAsync(pl.d_counters, 0, FMM_COUNTERS * sizeof(unsigned long long), st) != cudaSuccess)
         return FMM_ERR_CUDA;
     for (int k = 2; k <= levels; ++k)   // the halos of the moment grids read as zero
         if (cudaMemsetAsync(pl.grids.A[k], 0, pl.a_bytes[k], st) != cudaSuccess) return FMM_ERR_CUDA;

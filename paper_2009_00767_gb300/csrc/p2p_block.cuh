@@ -86,144 +86,6 @@ __device__ __forceinline__ void p2p_chunk(float2 (&part)[NP], const float4* __re
     }
 }
 
-// The block's sources: the own square's particles [t0, t0 + n_own) in nch_own chunks, then the
-// eight neighbours' in slot order (seg: sorted index minus slot and the frame shift per
-// neighbour, thr: first slot of neighbours 1..7).
-struct P2PSources {
-    const float4* sp;
-    const int4* seg;
-    uint32_t thr[7];
-    uint32_t t0, n_own, nch_own, n_nb;
-
-    // source of chunk c for this lane, in the target square's frame; slots past a part's end
-    // carry q = 0
-    __device__ __forceinline__ float4 load(uint32_t c, int lane) const {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < nch_own) {
-            const uint32_t s = 32u * c + (uint32_t)lane;
-            if (s < n_own) v = sp[t0 + s];
-        } else {
-            const uint32_t s = 32u * (c - nch_own) + (uint32_t)lane;
-            if (s < n_nb) {
-                int b = 0;
-#pragma unroll
-                for (int i = 0; i < 7; ++i) b += s >= thr[i] ? 1 : 0;
-                const int4 g = seg[b];
-                v = sp[s + (uint32_t)g.x];
-                v.x += __int_as_float(g.y);
-                v.y += __int_as_float(g.z);
-            }
-        }
-        return v;
-    }
-};
-
-// the near-field sum (log2 r^2 units, float-float) of target `lane` of a block of at most 2 NP
-// targets
-template <int NP>
-__device__ __forceinline__ float2 p2p_block(const P2PSources& S, const float4* __restrict__ tg, int lane) {
-    constexpr int W = NP <= 2 ? 4 : (NP <= 4 ? 8 : (NP <= 8 ? 16 : 32));
-    const uint32_t nch = S.nch_own + (S.n_nb + 31u) / 32u;
-    float2 near = make_float2(0.f, 0.f);
-    for (uint32_t r0 = 0; r0 < nch; r0 += kP2PRun) {
-        const uint32_t r1 = min(nch, r0 + (uint32_t)kP2PRun);
-        float2 part[NP];
-#pragma unroll
-        for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
-        // the next chunk's loads are in flight while one is summed (a deeper ring, unrolled, made
-        // the kernel's code outgrow the instruction cache)
-        float4 cur = S.load(r0, lane);
-        for (uint32_t c = r0; c < r1; ++c) {
-            const float4 nxt = (c + 1 < r1) ? S.load(c + 1, lane) : cur;
-            if (c < S.nch_own)
-                p2p_chunk<true, NP>(part, tg, cur);
-            else
-                p2p_chunk<false, NP>(part, tg, cur);
-            cur = nxt;
-        }
-        near = ff_add_f(near, warp_reduce_scatter<W, NP>(part, lane));
-    }
-    return near;
-}
-
-// Neighbour b = (dx + 1) + 3 (dy + 1) of finest square `leaf` (lane b < 9, b != 4; other lanes
-// and squares outside the domain give an empty range): its first sorted particle and count.
-__device__ __forceinline__ uint2 p2p_neighbour(const uint32_t* __restrict__ ls, uint32_t leaf, int levels, int lane) {
-    uint32_t first = 0, cnt = 0;
-    if (lane < 9 && lane != 4) {
-        const int side = 1 << levels;
-        const int jx = (int)fmm_compact2(leaf) + lane % 3 - 1, jy = (int)fmm_compact2(leaf >> 1) + lane / 3 - 1;
-        if (jx >= 0 && jy >= 0 && jx < side && jy < side) {
-            const uint32_t nl = fmm_morton((uint32_t)jx, (uint32_t)jy);
-            first = ls[nl];
-            cnt = ls[nl + 1] - first;
-        }
-    }
-    return make_uint2(first, cnt);
-}
-
-// The near field of the targets [b0, b0 + T) (T <= 24) of a finest square with particles
-// [t0, t1), whose neighbours' ranges nb came from p2p_neighbour; s_leaf is the square's side.
-// Returns target `lane`'s sum in log2 r^2 units as a float-float pair and the block's source
-// count in *nsrc.  tgt (16 float4) and seg (8 int4) are the warp's shared memory.
-__device__ __forceinline__ float2 p2p_near_nb(const float4* __restrict__ sp, uint32_t t0, uint32_t t1, uint32_t b0,
-                                              int T, uint2 nb, float s_leaf, float4* tgt, int4* seg, int lane,
-                                              uint32_t* nsrc) {
-    const uint32_t n_own = t1 - t0;
-    // the eight neighbours' sources take consecutive slots of the neighbour chunks
-    const uint32_t first = nb.x, cnt = nb.y;
-    uint32_t incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const uint32_t excl = incl - cnt;
-    const uint32_t n_nb = __shfl_sync(0xffffffffu, incl, 8);
-    if (lane < 9 && lane != 4)
-        seg[lane - (lane > 4)] = make_int4((int)(first - excl), __float_as_int((float)(lane % 3 - 1) * s_leaf),
-                                           __float_as_int((float)(lane / 3 - 1) * s_leaf), 0);
-    P2PSources S;
-    S.sp = sp;
-    S.seg = seg;
-#pragma unroll
-    for (int i = 1; i < 8; ++i) S.thr[i - 1] = __shfl_sync(0xffffffffu, excl, i + (i >= 4));
-    S.t0 = t0;
-    S.n_own = n_own;
-    S.nch_own = (n_own + 31u) / 32u;
-    S.n_nb = n_nb;
-    *nsrc = n_own + n_nb;
-    {
-        float x = 0.f, y = 0.f;
-        if (lane < T) {
-            const float4 P = sp[b0 + lane];
-            x = P.x;
-            y = P.y;
-        }
-        float* t = reinterpret_cast<float*>(&tgt[lane >> 1]);
-        t[lane & 1] = x;
-        t[2 + (lane & 1)] = y;
-    }
-    __syncwarp();
-    // the block's target pairs, rounded up to an even count, fix the unrolled width
-    switch ((T + 3) >> 2) {
-        case 1: return p2p_block<2>(S, tgt, lane);
-        case 2: return p2p_block<4>(S, tgt, lane);
-        case 3: return p2p_block<6>(S, tgt, lane);
-        case 4: return p2p_block<8>(S, tgt, lane);
-        case 5: return p2p_block<10>(S, tgt, lane);
-        default: return p2p_block<12>(S, tgt, lane);
-    }
-}
-
-// p2p_near_nb with the neighbours looked up first (square `leaf` of a quadtree of depth `levels`
-// whose CSR over the sorted array is ls)
-__device__ __forceinline__ float2 p2p_near(const float4* __restrict__ sp, const uint32_t* __restrict__ ls,
-                                           uint32_t leaf, uint32_t t0, uint32_t t1, uint32_t b0, int T, int levels,
-                                           float s_leaf, float4* tgt, int4* seg, int lane, uint32_t* nsrc) {
-    return p2p_near_nb(sp, t0, t1, b0, T, p2p_neighbour(ls, leaf, levels, lane), s_leaf, tgt, seg, lane, nsrc);
-}
-
 // ---------------------------------------------------------------- symmetric near field
 // The pair term log r^2 is symmetric, so each pair of adjacent squares is evaluated once: the
 // block's targets take their own square in full (both orders, as above) and only the four
@@ -375,6 +237,154 @@ __device__ __forceinline__ float2 p2p_near_sym(const float4* __restrict__ sp, co
         case 5: return p2p_block_sym<10>(S, tgt, tq, lane, acc);
         default: return p2p_block_sym<12>(S, tgt, tq, lane, acc);
     }
+}
+
+// ---------------------------------------------------------------- crowded squares
+// The symmetric near field of squares above FMM_CROWD_POP particles (listed by the sort).  Each lane holds two sources, so that a target pair
+// read from shared memory serves four pairs and the independent work covers the latencies of the MUFU and
+// of the source loads; and the own square is taken once for both sides too: a block of up to kCrowdTargets
+// targets against itself one-sided, then its "later" sources -- the rest of the own square after the block,
+// masked at r^2 = 0, and the forward neighbours.  The sources of a large square's blocks are split into up
+// to kCrowdParts work items, so that a square of ten thousand particles does not end as one long tail.
+// What bounds it: the MUFU, one lg2 a pair (16 a clock and SM), with the FMA pipe (6 packed instructions
+// of two cycles for two pairs) and issue close behind.
+// 2^24 clustered particles (32 Gaussians, levels 10, 2.1e11 ordered pairs): 28.5 ms against 33.5 ms for blocks
+// of 24 targets, one source a lane and the own square in full; of the difference 3 ms are the own square's
+// second half.  24 targets 30.7 ms, 48 targets with one source a lane 29.0 ms, the targets in registers
+// instead of shared memory (one source a lane, 16 warps an SM) 41.7 ms, waiting for source loads.
+constexpr int kCrowdBlocksPerSm = 4;
+struct P2PCrowdShared {
+    float4 tg[kCrowdTargets / 2];
+    float2 tq[kCrowdTargets / 2];
+    int4 seg[5];   // ranges of later sources: {sorted index minus slot, frame shift x, y, first slot past it}
+};
+
+// two sources of the lane against the NP target pairs, both sides; pairs at r^2 = 0 give 0 with kMask.
+// Returns the sources' sums.
+template <bool kMask, int NP>
+__device__ __forceinline__ float2 p2p_chunk_sym2(float2 (&part)[NP], const float4* __restrict__ tg,
+                                                 const float2* __restrict__ tq, float4 a, float4 b) {
+    const float2 ax = make_float2(-a.x, -a.x), ay = make_float2(-a.y, -a.y), aq = make_float2(a.z, a.z);
+    const float2 bx = make_float2(-b.x, -b.x), by = make_float2(-b.y, -b.y), bq = make_float2(b.z, b.z);
+    const float2 tiny = make_float2(0x1p-100f, 0x1p-100f);
+    float2 sa = make_float2(0.f, 0.f), sb = make_float2(0.f, 0.f);
+    auto log2_r2 = [&](float2 dx, float2 dy) {
+        const float2 r2 = __ffma2_rn(dx, dx, kMask ? __fmul2_rn(dy, dy) : __ffma2_rn(dy, dy, tiny));
+        float2 lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
+        if (kMask) {
+            lg.x = r2.x > 0.f ? lg.x : 0.f;
+            lg.y = r2.y > 0.f ? lg.y : 0.f;
+        }
+        return lg;
+    };
+#pragma unroll
+    for (int tp = 0; tp < NP; ++tp) {
+        const float4 t = tg[tp];
+        const float2 q = tq[tp], tx = make_float2(t.x, t.y), ty = make_float2(t.z, t.w);
+        const float2 la = log2_r2(__fadd2_rn(tx, ax), __fadd2_rn(ty, ay));
+        const float2 lb = log2_r2(__fadd2_rn(tx, bx), __fadd2_rn(ty, by));
+        part[tp] = __ffma2_rn(bq, lb, __ffma2_rn(aq, la, part[tp]));
+        sa = __ffma2_rn(q, la, sa);
+        sb = __ffma2_rn(q, lb, sb);
+    }
+    return make_float2(sa.x + sa.y, sb.x + sb.y);
+}
+
+// The block's targets [b0, b0 + T) against the slots [c0, c1) of its later sources and, with part 0,
+// against themselves; slots below n_own belong to the own square.
+__device__ __forceinline__ void p2p_crowd_item(const float4* __restrict__ sp, uint32_t b0, int T, bool self,
+                                               uint32_t c0, uint32_t c1, uint32_t n_own, const P2PCrowdShared& sh,
+                                               int lane, double* __restrict__ acc) {
+    constexpr int NP = kCrowdTargets / 2;
+    float2 part[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
+    if (self) p2p_chunk<true, NP>(part, sh.tg, lane < T ? sp[b0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f));
+    const uint32_t e0 = (uint32_t)sh.seg[0].w, e1 = (uint32_t)sh.seg[1].w, e2 = (uint32_t)sh.seg[2].w,
+                   e3 = (uint32_t)sh.seg[3].w;
+    auto load = [&](uint32_t s, uint32_t* idx) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        *idx = 0xffffffffu;
+        if (s < c1) {
+            const int4 g = sh.seg[(s >= e0 ? 1 : 0) + (s >= e1 ? 1 : 0) + (s >= e2 ? 1 : 0) + (s >= e3 ? 1 : 0)];
+            *idx = s + (uint32_t)g.x;
+            v = sp[*idx];
+            v.x += __int_as_float(g.y);
+            v.y += __int_as_float(g.z);
+        }
+        return v;
+    };
+    float2 near = make_float2(0.f, 0.f);
+    uint32_t ia, ib;
+    float4 a = load(c0 + (uint32_t)lane, &ia), b = load(c0 + 32u + (uint32_t)lane, &ib);
+    int run = 1;
+#pragma unroll 1
+    for (uint32_t c = c0; c < c1; c += 64u) {
+        uint32_t na, nb;   // the next sources' loads are in flight meanwhile
+        const float4 xa = load(c + 64u + (uint32_t)lane, &na), xb = load(c + 96u + (uint32_t)lane, &nb);
+        const float2 v = c < n_own ? p2p_chunk_sym2<true, NP>(part, sh.tg, sh.tq, a, b)
+                                   : p2p_chunk_sym2<false, NP>(part, sh.tg, sh.tq, a, b);
+        if (ia != 0xffffffffu) atomicAdd(acc + ia, fmm_f2d_bits(v.x));
+        if (ib != 0xffffffffu) atomicAdd(acc + ib, fmm_f2d_bits(v.y));
+        a = xa;
+        b = xb;
+        ia = na;
+        ib = nb;
+        run += 2;
+        if (run >= kP2PRun) {
+            near = ff_add_f(near, warp_reduce_scatter<32>(part, lane));
+#pragma unroll
+            for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
+            run = 0;
+        }
+    }
+    near = ff_add_f(near, warp_reduce_scatter<32>(part, lane));
+    if (lane < T) atomicAdd(acc + b0 + lane, fmm_f2d_bits(near.x) + fmm_f2d_bits(near.y));
+}
+
+// Item `item` of the crowded square `leaf` with particles [t0, t1).  Returns the ordered pairs covered (both
+// directions of every later pair); sh is the warp's shared memory.
+__device__ __forceinline__ unsigned long long p2p_near_crowd(const float4* __restrict__ sp,
+                                                             const uint32_t* __restrict__ ls, uint32_t leaf,
+                                                             uint32_t t0, uint32_t t1, uint32_t item, int levels,
+                                                             float s_leaf, P2PCrowdShared& sh, int lane,
+                                                             double* __restrict__ acc) {
+    const uint2 nb = fmm_forward_neighbour(ls, leaf, levels, lane);
+    uint32_t n_fw = nb.y;
+    n_fw += __shfl_xor_sync(0xffffffffu, n_fw, 1);
+    n_fw += __shfl_xor_sync(0xffffffffu, n_fw, 2);
+    n_fw = __shfl_sync(0xffffffffu, n_fw, 0);
+    const uint32_t n = t1 - t0, nblk = fmm_crowd_blocks(n), parts = fmm_crowd_parts(n);
+    const uint32_t blk = item / parts, prt = item % parts;
+    const uint32_t b0 = t0 + (uint32_t)((unsigned long long)n * blk / nblk);
+    const int T = (int)(t0 + (uint32_t)((unsigned long long)n * (blk + 1) / nblk) - b0);
+    const uint32_t n_own = t1 - b0 - (uint32_t)T, n_src = n_own + n_fw;
+    // parts of whole 64-source chunks
+    const uint32_t chunks = (n_src + 63u) / 64u;
+    const uint32_t c0 = 64u * (uint32_t)((unsigned long long)chunks * prt / parts);
+    const uint32_t c1 = min(n_src, 64u * (uint32_t)((unsigned long long)chunks * (prt + 1) / parts));
+    __syncwarp();
+    uint32_t slots = n_own;
+    if (lane == 0) sh.seg[0] = make_int4((int)(b0 + (uint32_t)T), 0, 0, (int)n_own);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t first = __shfl_sync(0xffffffffu, nb.x, i), cnt = __shfl_sync(0xffffffffu, nb.y, i);
+        const float ox = (float)(i == 3 ? -1 : (i == 2 ? 0 : 1)) * s_leaf, oy = (float)(i == 0 ? 0 : 1) * s_leaf;
+        if (lane == i)
+            sh.seg[1 + i] = make_int4((int)(first - slots), __float_as_int(ox), __float_as_int(oy), (int)(slots + cnt));
+        slots += cnt;
+    }
+    for (int i = lane; i < kCrowdTargets; i += 32) {
+        const float4 own = i < T ? sp[b0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float* t = reinterpret_cast<float*>(&sh.tg[i >> 1]);
+        t[i & 1] = own.x;
+        t[2 + (i & 1)] = own.y;
+        reinterpret_cast<float*>(&sh.tq[i >> 1])[i & 1] = own.z;
+    }
+    __syncwarp();
+    const bool self = prt == 0u;
+    p2p_crowd_item(sp, b0, T, self, c0, c1, n_own, sh, lane, acc);
+    return 2ull * (unsigned long long)T * (c1 > c0 ? c1 - c0 : 0u) + (self ? (unsigned long long)T * (T - 1) : 0ull);
 }
 
 // ---------------------------------------------------------------- near field with the field

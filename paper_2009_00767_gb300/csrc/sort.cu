@@ -177,7 +177,7 @@ constexpr int kLocalTopMax = 1024;
 template <bool kLocalTop>
 __global__ void k_scan2_down(uint32_t* __restrict__ in, int64_t m, const unsigned long long* __restrict__ sums,
                              uint32_t* __restrict__ leaf_start, uint32_t* __restrict__ bstart,
-                             uint2* __restrict__ map, int* __restrict__ crowd_hint) {
+                             uint2* __restrict__ map, int* __restrict__ crowd_hint, P2PCrowd crowd) {
     __shared__ unsigned long long wt[kScanThreads / 32 + 1];
     unsigned long long v[kScanItems];
     uint32_t nbk[kScanItems];
@@ -188,6 +188,7 @@ __global__ void k_scan2_down(uint32_t* __restrict__ in, int64_t m, const unsigne
         v[j] = (base + j < m) ? pop_blocks(in[base + j]) : 0ull;
         nbk[j] = (uint32_t)(v[j] >> 32);
         crowded |= (uint32_t)v[j] > (uint32_t)FMM_LANE_MAX;
+        if ((uint32_t)v[j] > (uint32_t)FMM_CROWD_POP && crowd.list) fmm_crowd_add(crowd, (uint32_t)(base + j), (uint32_t)v[j]);
         if (base + j < m) in[base + j] = 0u;   // the populations start the next call at zero
     }
     if (crowded && crowd_hint) *(volatile int*)crowd_hint = 1;
@@ -283,17 +284,19 @@ int fmm_launch_sort(fmm_plan_s* pl, const double* xy, const double* q, bool with
     }
     const int nb = pl->scan_blocks;
     {
-        // the near-field blocks come with the same scan (block_sums holds 64-bit partials)
+        // the near-field blocks come with the same scan (block_sums holds 64-bit partials), and in the mixed
+        // path the crowded squares' items
+        const P2PCrowd crowd = {pl->d_counters + 2 * FMM_COUNTER_SLOTS, pl->crowd_list};
         unsigned long long* sums = reinterpret_cast<unsigned long long*>(pl->block_sums);
         k_scan2_reduce<<<nb, kScanThreads, 0, st>>>(pl->counts, m, sums);
         if (nb <= kLocalTopMax) {
             k_scan2_down<true><<<nb, kScanThreads, 0, st>>>(pl->counts, m, sums, pl->leaf_start, pl->leaf_bstart,
-                                                            pl->blk_map, pl->crowd_hint_d);
+                                                            pl->blk_map, pl->crowd_hint_d, crowd);
             launches -= 1;
         } else {
             k_scan2_top<<<1, kScanThreads, 0, st>>>(sums, nb);
             k_scan2_down<false><<<nb, kScanThreads, 0, st>>>(pl->counts, m, sums, pl->leaf_start, pl->leaf_bstart,
-                                                             pl->blk_map, pl->crowd_hint_d);
+                                                             pl->blk_map, pl->crowd_hint_d, crowd);
         }
     }
     launches += 3;
@@ -322,10 +325,13 @@ __global__ void k_leaf_blocks(const uint32_t* __restrict__ leaf_start, int64_t m
     if (i < m) nb[i] = (leaf_start[i + 1] - leaf_start[i] + block - 1u) / block;
 }
 
-// block -> (square, block index inside the square), one thread per square
-__global__ void k_block_map(const uint32_t* __restrict__ bstart, int64_t m, uint2* __restrict__ map) {
+// block -> (square, block index inside the square), one thread per square; crowded squares' items
+__global__ void k_block_map(const uint32_t* __restrict__ bstart, const uint32_t* __restrict__ leaf_start, int64_t m,
+                            uint2* __restrict__ map, P2PCrowd crowd) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
+    const uint32_t n = leaf_start[i + 1] - leaf_start[i];
+    if (n > (uint32_t)FMM_CROWD_POP) fmm_crowd_add(crowd, (uint32_t)i, n);
     const uint32_t b0 = bstart[i], b1 = bstart[i + 1];
     for (uint32_t b = b0; b < b1; ++b) map[b] = make_uint2((uint32_t)i, b - b0);
 }
@@ -340,12 +346,12 @@ int fmm_launch_scan(const uint32_t* counts, int64_t m, uint32_t* block_sums, uin
 }
 
 int fmm_launch_leaf_blocks(const uint32_t* leaf_start, int64_t m, uint32_t block, uint32_t* nb, uint32_t* block_sums,
-                           uint32_t* bstart, uint2* map, cudaStream_t st) {
+                           uint32_t* bstart, uint2* map, P2PCrowd crowd, cudaStream_t st) {
     const unsigned g = (unsigned)((m + 255) / 256);
     k_leaf_blocks<<<g, 256, 0, st>>>(leaf_start, m, block, nb);
     const int r = fmm_launch_scan(nb, m, block_sums, bstart, 0xffffffffu, st);
     if (r < 0) return -1;
     if (map == nullptr) return r + 1;
-    k_block_map<<<g, 256, 0, st>>>(bstart, m, map);
+    k_block_map<<<g, 256, 0, st>>>(bstart, leaf_start, m, map, crowd);
     return cudaGetLastError() == cudaSuccess ? r + 2 : -1;
 }

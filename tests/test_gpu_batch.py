@@ -142,3 +142,19 @@ def test_batch_autotune_cache(tmp_path):
         assert t2["ms"] == pytest.approx(t1["ms"], abs=1e-5)
     assert len(cache.read_text().splitlines()) == 1
     check_parity(tuned, first, MIXED_TOL, "batch after the autotuner vs before")
+
+
+def test_crowded_squares_in_a_batch():
+    """Systems with crowded squares (a kernel of their own) beside small ones: the same sums as single-system
+    plans of the same form, to the rounding of FP32 sums in another order (MIXED_TOL)."""
+    from gpu_util import run_fmm, to_dev
+    from paper_2009_00767_gb300 import binding
+    sizes, levels = [350, 5000, 40, 9001, 1200], [0, 1, 1, 2, 2]
+    systems = [inputs.gmm(n, 8500 + n, k=2, sigma_lo=0.05, sigma_hi=0.2) for n in sizes]
+    txy, tq = to_dev(np.concatenate([s[0] for s in systems]), np.concatenate([s[1] for s in systems]))
+    with binding.Batch(sizes, levels, 20, 5.0, "fp32") as b:
+        phi = b.potential(txy, tq).cpu().numpy()
+    at = 0
+    for (xy, q), n, lev in zip(systems, sizes, levels):
+        check_parity(phi[at:at + n], run_fmm(xy, q, lev, 20, "fp32")[0], MIXED_TOL, f"batch crowded n={n} levels={lev}")
+        at += n

@@ -308,3 +308,27 @@ def test_host_calls_in_flight(oracle_mod):
     refs = [oracle_mod.shiftfree(xy, q, 7, 16) for xy, q in sets]
     for i in range(3):
         check_parity(outs[i].numpy(), refs[i % 2], MIXED_TOL, f"host call {i} in flight")
+
+
+@pytest.mark.parametrize("lev", [0, 1])
+@pytest.mark.parametrize("n", [40, 63, 64, 65, 66, 96, 97, 129, 353, 1000, 1025, 4500, 9000])
+def test_crowded_squares(n, lev):
+    """Squares either side of the population from which a kernel of their own takes them, blocks of 1 to 32
+    targets, source chunks of every remainder, sources in one and in several parts, coincident particles; no far
+    field at these levels.  In a box of side 4 positions on a grid of 2^-20 are exact in FP32 whatever the
+    square, so a term's error is that of r^2 (2^-22 relative), of the MUFU's lg2 (2^-22) and of FP32 sums of at
+    most 16 terms of it: together within 2^-20 of |q_j| (|log r_ij| + 1) summed over the sources."""
+    from gpu_util import run_fmm
+    xy, q = inputs.gmm(n, 8400 + n, k=3, sigma_lo=0.05, sigma_hi=0.2, box=4.0, centre_hi=3.5)
+    xy = np.round(xy * 2.0 ** 20) / 2.0 ** 20
+    q = q.astype(np.float32).astype(np.float64)
+    xy[n - 1] = xy[0]
+    phi, st = run_fmm(xy, q, lev, 8, "fp32", box=4.0)
+    for i0 in range(0, n, 500):
+        d = np.hypot(xy[i0:i0 + 500, None, 0] - xy[None, :, 0], xy[i0:i0 + 500, None, 1] - xy[None, :, 1])
+        k = np.where(d > 0.0, np.log(np.where(d > 0.0, d, 1.0)), 0.0)
+        bound = 2.0 ** -20 * ((np.abs(k) + 1.0) * np.abs(q)[None, :]).sum(1)
+        assert np.all(np.abs(phi[i0:i0 + 500] - (k * q[None, :]).sum(1)) <= bound)
+    cell = np.minimum((xy * 2 ** lev / 4.0).astype(int), 2 ** lev - 1)
+    cnt = np.bincount(cell[:, 0] + 2 ** lev * cell[:, 1])
+    assert st["p2p_pairs"] == n * (n - 1) and st["max_leaf"] == int(cnt.max())
