@@ -34,10 +34,12 @@
  *                        to the method's own error only to about level 4 (2D) and 3 (3D).
  *   FMM_LAG_NODE_F64     the same bilinear forms with the change of basis applied on the
  *                        particle side (STEP4: M_m h_{m^0}(c) = h_m(c) exactly): node charges
- *                        of every cell at every level straight from its charges, the node-to-
- *                        node matrix M_b over each interaction list, the node potentials
- *                        interpolated back at the charges; equal to the literal form in exact
- *                        arithmetic and free of its cancellation.  FP64 throughout.
+ *                        of the finest cells straight from their charges and of the coarser
+ *                        ones from their children's (U-bar-2; a cubic is its own interpolant,
+ *                        so this is exact), the node-to-node matrix M_b over each interaction
+ *                        list, the node potentials summed down to the finest cells (D-bar-2)
+ *                        and interpolated back at the charges; equal to the literal form in
+ *                        exact arithmetic and free of its cancellation.  FP64 throughout.
  *   FMM_LAG_NODE_F32     the node form in FP32 arithmetic with FP64 accumulation across
  *                        levels and source tiles; near-field differences from two-word (hi, lo)
  *                        FP32 coordinates.  About 1e-7 relative to the FP64 node form.
@@ -78,7 +80,7 @@ typedef struct {
     double ms_up;              /* node charges of levels 2..levels (literal: U-bar sums) */
     double ms_down;            /* node potentials over the interaction lists (literal: D-bar) */
     double ms_eval;            /* interpolation at the charges + far/near sum in input order */
-    double ms_p2p;             /* near field (on a second stream, overlapping the far field) */
+    double ms_p2p;             /* near field (the far field overlaps it on a second stream) */
     int64_t p2p_pairs;         /* ordered pairs of the near field, self pairs included */
     int64_t m2l_pairs;         /* interaction-list pairs of levels 2..levels */
     uint64_t workspace_bytes;  /* device memory the plan owns (the literal form's B included) */
@@ -109,7 +111,7 @@ fmm_status fmm_lag_stats_get(fmm_lag_plan_t plan, fmm_lag_stats* out);
 /* Change the stream later calls enqueue on. */
 fmm_status fmm_lag_set_stream(fmm_lag_plan_t plan, void* stream);
 
-/* 2 (the default): the near field runs on a stream of the plan's own beside the far field, joined
+/* 2 (the default): the far field runs on a stream of the plan's own beside the near field, joined
  * back before the final sum.  1: every kernel in turn on the plan's stream, so that the stage
  * times of fmm_lag_stats_get are those of each stage alone.  Same results either way.
  * FMM_ERR_INVALID_ARG for another count or a NULL plan. */

@@ -6,17 +6,17 @@
 //     level are one contiguous range: FP32 forms keep (x, y, z, q) as a float4 "hi" and the
 //     residues x - hi as a float4 "lo"; FP64 forms keep (x, y, z, q) as a Pos64;
 //   * per level k, the cells in Morton order with d = 4^D node values each (node index
-//     i + 4j + 16k): node charges Q_k and node potentials psi_k (node forms), or the vectors
-//     v_k and dual vectors u_k (literal form);
+//     i + 4j + 16k): node charges Q_k and node potentials psi_k (node forms; psi_k in FP64), or
+//     the vectors v_k and dual vectors u_k (literal form);
 //   * node forms: per level a 7^D table of d x d node-to-node matrices, indexed by the offset
 //     between source and target cell, laid out [offset][source node i][target node j];
 //   * literal form: per level the interaction-list pairs in CSR order by target cell, and one
 //     d x d FP64 matrix B = M_{m_i}^T M_b M_m per pair (row a: the root-node coordinate of the
 //     source's vector, column l: that of the target's).
 //
-// Work items of the particle kernels are chunks of up to 128 consecutive sorted charges within
-// one finest cell; a persistent grid walks the chunk list, so crowded cells are split over
-// blocks and any distribution keeps every SM busy.
+// Work items of the particle kernels are chunks of consecutive sorted charges within one finest
+// cell (up to kChunk, or the near field's kWarpChunk), so crowded cells are split over warps and any
+// distribution keeps every SM busy.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,6 +35,7 @@ namespace {
 
 constexpr int kChunk = 128;      // charges per work item
 constexpr int kWarpChunk = 24;     // targets per near-field warp work item, FP32
+constexpr int kPairSlots = 64;     // the near field's pair counter is spread over this many words
 constexpr int kWarpChunk64 = 32;   // and FP64
 constexpr int kMaxLevels = 8;
 constexpr double kLn2 = 0.69314718055994530942;
@@ -90,6 +91,11 @@ struct __align__(32) Pos64 {
     double x, y, z, w;
 };
 
+// Sums over finest cells: charges, particle-kernel chunks, near-field chunks.
+struct Scan3 {
+    int n, c, w;
+};
+
 struct fmm_lag_plan_s {
     int dev = 0, dim = 2, levels = 0, form = 0, d = 16;
     double box = 5.0;
@@ -105,6 +111,7 @@ struct fmm_lag_plan_s {
     int* chunk_start = nullptr;    // [nleaf + 1]
     int* wchunk_start = nullptr;   // [nleaf + 1] near-field warp chunks
     int* order = nullptr;          // [n_max] sorted -> input index
+    Scan3* scan = nullptr;  // per tile of the scan
     float4* hi = nullptr;          // FP32 forms
     float4* lo = nullptr;
     Pos64* p64 = nullptr;        // FP64 forms
@@ -114,7 +121,10 @@ struct fmm_lag_plan_s {
     unsigned long long* pairs = nullptr;   // near-field pair counter
     int* next_item = nullptr;              // near-field work counter
     void* node[kMaxLevels + 1] = {};       // Q_k (node) or v_k (literal), d values per cell
-    void* pot[kMaxLevels + 1] = {};        // psi_k (node) or u_k (literal)
+    void* pot[kMaxLevels + 1] = {};        // psi_k (node) or u_k (literal), one allocation at pot[2]
+    size_t pot_bytes = 0;
+    double* psi0 = nullptr;                // FP32 form: the finest cells' potentials as one FP64 value a cell
+    float* dpsi = nullptr;                 // and FP32 differences from it
     void* K = nullptr;                     // node forms: operators of levels 2..levels
     int* pair_start[kMaxLevels + 1] = {};  // literal: CSR by target cell
     int* pair_src[kMaxLevels + 1] = {};
@@ -126,7 +136,7 @@ struct fmm_lag_plan_s {
     int grid_particles = 0;
     cudaStream_t last_st = nullptr;   // the stream of the last call, for comparison only
     bool serial = false;   // every kernel in turn on the plan's stream (per-kernel timing)
-    int grid_p2p = 0;      // resident blocks of the form's near-field kernel, all SMs
+    int grid_p2p = 0;      // resident blocks of the FP64 near-field kernel, all SMs
     double2* logtab = nullptr;   // 2D FP64 forms: the logarithm's table (fp64_math.cuh)
 };
 
@@ -134,24 +144,27 @@ namespace {
 
 // ------------------------------------------------------------------------------ binning
 
-// Finest cell per charge with the FP64 floor/clamp rule, its Morton key and its rank within
+// Finest cell per charge with the FP64 floor/clamp rule (finest_coord), its Morton key and its rank within
 // the cell (atomic), plus the input checks.
 template <int D>
 __global__ void k_bin(const double* __restrict__ pos, const double* __restrict__ q, int64_t n, int L,
-                      double box, uint32_t* __restrict__ key, uint32_t* __restrict__ rank, int* __restrict__ count,
-                      unsigned* __restrict__ status) {
+                      double box, float side_over_box, uint32_t* __restrict__ key, uint32_t* __restrict__ rank,
+                      int* __restrict__ count, unsigned* __restrict__ status) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int side = 1 << L;
+    const long long bb = __double_as_longlong(box);
     int c[3] = {0, 0, 0};
-    unsigned bad = 0;
-    if (!isfinite(q[i])) bad |= kFlagNonFinite;
+    unsigned bad = finite_bits(q[i]) ? 0u : kFlagNonFinite;
+#pragma unroll
     for (int a = 0; a < D; ++a) {
         const double x = pos[i * D + a];
-        if (!isfinite(x)) bad |= kFlagNonFinite;
-        else if (!(x >= 0.0 && x <= box)) bad |= kFlagOutOfBox;
-        const double f = floor(x * (double)side / box);
-        c[a] = f < 0.0 ? 0 : (f > (double)(side - 1) ? side - 1 : (int)f);
+        if (!finite_bits(x)) {
+            bad |= kFlagNonFinite;
+        } else {
+            if (!in_box_bits(x, bb)) bad |= kFlagOutOfBox;
+            c[a] = finest_coord(x, (double)side, side_over_box, box, side);
+        }
     }
     if (bad) atomicOr(status, bad);
     const uint32_t k = morton_enc(D, c);
@@ -159,46 +172,64 @@ __global__ void k_bin(const double* __restrict__ pos, const double* __restrict__
     rank[i] = (uint32_t)atomicAdd(count + k, 1);
 }
 
-// Exclusive scans of the populations and of the chunk counts, one block.
-// (chunks of kChunk, and of wchunk for the near field's warps)
-__global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ count, int nleaf, int wchunk, int* __restrict__ start,
-                                               int* __restrict__ chunk_start, int* __restrict__ wchunk_start) {
-    __shared__ int s_n[1024], s_c[1024], s_w[1024];
-    const int t = threadIdx.x;
-    const int per = (nleaf + 1023) / 1024;
-    const int b0 = min(nleaf, t * per), b1 = min(nleaf, b0 + per);
-    int sn = 0, sc = 0, sw = 0;
-    for (int b = b0; b < b1; ++b) {
-        sn += count[b];
-        sc += (count[b] + kChunk - 1) / kChunk;
-        sw += (count[b] + wchunk - 1) / wchunk;
+// Exclusive scans of the populations and of the chunk counts (chunks of kChunk, and of wchunk for the near
+// field's warps) over the finest cells, in tiles of kScanTile cells: each tile's sums, then each tile's scan
+// behind the sums of the tiles before it (at most 65,536 cells, 128 tiles).
+constexpr int kScanTile = 512;
+
+__device__ __forceinline__ Scan3 scan_add(Scan3 a, Scan3 b) { return Scan3{a.n + b.n, a.c + b.c, a.w + b.w}; }
+__device__ __forceinline__ Scan3 scan_cell(const int* __restrict__ count, int b, int nleaf, int wchunk) {
+    const int n = b < nleaf ? count[b] : 0;
+    return Scan3{n, (n + kChunk - 1) / kChunk, (n + wchunk - 1) / wchunk};
+}
+// exclusive scan of one value a thread over the block; *total receives the block's sum
+__device__ __forceinline__ Scan3 scan_block(Scan3 v, Scan3* total) {
+    __shared__ Scan3 warps[kScanTile / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Scan3 inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const Scan3 y = Scan3{__shfl_up_sync(0xffffffffu, inc.n, o), __shfl_up_sync(0xffffffffu, inc.c, o),
+                              __shfl_up_sync(0xffffffffu, inc.w, o)};
+        if (lane >= o) inc = scan_add(inc, y);
     }
-    s_n[t] = sn;
-    s_c[t] = sc;
-    s_w[t] = sw;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {   // Hillis-Steele inclusive scan
-        const int vn = t >= off ? s_n[t - off] : 0, vc = t >= off ? s_c[t - off] : 0;
-        const int vw = t >= off ? s_w[t - off] : 0;
-        __syncthreads();
-        s_n[t] += vn;
-        s_c[t] += vc;
-        s_w[t] += vw;
-        __syncthreads();
+    if (lane == 31) warps[warp] = inc;
+    __syncthreads();
+    Scan3 before = {0, 0, 0}, all = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < kScanTile / 32; ++i) {
+        if (i < warp) before = scan_add(before, warps[i]);
+        all = scan_add(all, warps[i]);
     }
-    int rn = s_n[t] - sn, rc = s_c[t] - sc, rw = s_w[t] - sw;
-    for (int b = b0; b < b1; ++b) {
-        start[b] = rn;
-        chunk_start[b] = rc;
-        wchunk_start[b] = rw;
-        rn += count[b];
-        rc += (count[b] + kChunk - 1) / kChunk;
-        rw += (count[b] + wchunk - 1) / wchunk;
+    *total = all;
+    return Scan3{before.n + inc.n - v.n, before.c + inc.c - v.c, before.w + inc.w - v.w};
+}
+
+__global__ void __launch_bounds__(kScanTile) k_scan_sums(const int* __restrict__ count, int nleaf, int wchunk,
+                                                         Scan3* __restrict__ sums) {
+    Scan3 total;
+    scan_block(scan_cell(count, blockIdx.x * kScanTile + threadIdx.x, nleaf, wchunk), &total);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kScanTile) k_scan(const int* __restrict__ count, int nleaf, int wchunk,
+                                                    const Scan3* __restrict__ sums, int* __restrict__ start,
+                                                    int* __restrict__ chunk_start, int* __restrict__ wchunk_start) {
+    Scan3 before = {0, 0, 0}, total;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += kScanTile) before = scan_add(before, sums[t]);
+    scan_block(before, &before);
+    const int b = blockIdx.x * kScanTile + threadIdx.x;
+    const Scan3 v = scan_add(before, scan_block(scan_cell(count, b, nleaf, wchunk), &total));
+    if (b < nleaf) {
+        start[b] = v.n;
+        chunk_start[b] = v.c;
+        wchunk_start[b] = v.w;
     }
-    if (t == 1023) {
-        start[nleaf] = s_n[1023];
-        chunk_start[nleaf] = s_c[1023];
-        wchunk_start[nleaf] = s_w[1023];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        start[nleaf] = before.n + total.n;
+        chunk_start[nleaf] = before.c + total.c;
+        wchunk_start[nleaf] = before.w + total.w;
     }
 }
 
@@ -240,18 +271,19 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 // is a chunk of up to kWarpChunk targets of a finest cell A and a group of A's "forward" cells: A itself
 // and the neighbours whose offset is positive in (z, y, x) order (13 in 3D, 4 in 2D), so that every
 // unordered pair of adjacent cells is met once.  Lanes over sources, registers over targets: the group's
-// later sources (A's charges after the chunk, then the forward cells') are walked 32 at a time, one a
+// later sources (A's charges after the chunk, then the forward cells') are walked 64 at a time, two a
 // lane; the targets' coordinates and charges are shared-memory broadcasts, and two targets' arithmetic
 // runs in packed FP32x2.  A pair's 1/r (or log r) feeds a register partial of the target and the sum of the
-// source, which stays in its lane and goes out with one FP64 atomic per lane and 32 sources.  The chunk
+// source, which stays in its lane and goes out with one FP64 atomic.  The chunk
 // against itself is one-sided.  Pairs inside A are masked at r = 0 (only there can a pair coincide).
 // Differences come from two-word coordinates, (hi_t - hi_s) + (lo_t - lo_s), so a close pair's distance
 // keeps about 48 bits.  After kP2PRun chunks the lanes' partials of a target are summed across the warp
 // (warp_reduce_scatter) and added in FP64.
 // What bounds it: the FMA pipe, 14 packed instructions (two cycles each) for two targets in 3D, 9 of them
-// the two-word differences; MUFU and issue are at about two thirds of that.  200,000 charges in 3D, levels
-// 3: 486 us against 739 us for 64 targets over the lanes and a butterfly over the lanes per source tile
-// (31 shuffles, 62 selects) for the source's side; 2^20 in 2D, levels 7: 256 against 368 us.
+// the two-word differences.  A lane holds two sources, so that the targets' shared-memory broadcasts (8
+// wavefronts for two targets) serve four pairs.  200,000 charges in 3D, levels 3: 467 us against 739 us for
+// 64 targets over the lanes and a butterfly over the lanes per source tile (31 shuffles, 62 selects) for the
+// source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us.
 constexpr int kP2PWarps = 4;     // warps per block, each on its own work items
 template <int D>
 __host__ __device__ constexpr int fwd_group() { return D == 3 ? 4 : 5; }   // forward cells per work item
@@ -323,33 +355,61 @@ struct LagTargets {
     float2 lz[D == 3 ? kWarpChunk / 2 : 1];
 };
 
-// the lane's source (h, l) against the chunk's 2 NP targets; returns the source's sum
-template <int D, bool kMask, int NP>
-__device__ __forceinline__ float p2p_lag_chunk(float2 (&part)[NP], const LagTargets<D>& tg, float4 h, float4 l) {
-    const float2 nx = make_float2(-h.x, -h.x), ny = make_float2(-h.y, -h.y), nz = make_float2(-h.z, -h.z);
-    const float2 mx = make_float2(-l.x, -l.x), my = make_float2(-l.y, -l.y), mz = make_float2(-l.z, -l.z);
-    const float2 q2 = make_float2(h.w, h.w);
-    float2 sacc = make_float2(0.f, 0.f);
+// A lane's source, its coordinates negated and duplicated: {-x, -x} (high and low words), {q, q}.
+template <int D>
+struct LagSource {
+    float2 x[D], l[D], q;
+    __device__ LagSource(float4 h, float4 lo) {
+        x[0] = make_float2(-h.x, -h.x);
+        x[1] = make_float2(-h.y, -h.y);
+        l[0] = make_float2(-lo.x, -lo.x);
+        l[1] = make_float2(-lo.y, -lo.y);
+        if constexpr (D == 3) {
+            x[2] = make_float2(-h.z, -h.z);
+            l[2] = make_float2(-lo.z, -lo.z);
+        }
+        q = make_float2(h.w, h.w);
+    }
+};
+
+// 1 / r (3D) or log2 r^2 (2D) of the lane's source and target pair t; kMask: 0 for a coincident pair
+template <int D, bool kMask>
+__device__ __forceinline__ float2 p2p_lag_pair(const LagSource<D>& s, float4 A, float4 B, float4 C, float2 lz) {
+    const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), s.x[0]), __fadd2_rn(make_float2(C.x, C.y), s.l[0]));
+    const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), s.x[1]), __fadd2_rn(make_float2(C.z, C.w), s.l[1]));
+    float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+    if constexpr (D == 3) {
+        const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), s.x[2]), __fadd2_rn(lz, s.l[2]));
+        r2 = __ffma2_rn(dz, dz, r2);
+    }
+    float2 k = D == 3 ? make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y)) : make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
+    if constexpr (kMask) {
+        k.x = r2.x > 0.f ? k.x : 0.f;
+        k.y = r2.y > 0.f ? k.y : 0.f;
+    }
+    return k;
+}
+
+// the lane's kS sources (1 or 2) against the chunk's 2 NP targets; returns the sources' sums
+template <int D, bool kMask, int NP, int kS>
+__device__ __forceinline__ float2 p2p_lag_chunk(float2 (&part)[NP], const LagTargets<D>& tg, float4 ha, float4 la,
+                                                float4 hb, float4 lb) {
+    const LagSource<D> a(ha, la), b(hb, lb);
+    float2 sa = make_float2(0.f, 0.f), sb = make_float2(0.f, 0.f);
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
         const float4 A = tg.xy[t], B = tg.zq[t], C = tg.lxy[t];
-        const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), nx), __fadd2_rn(make_float2(C.x, C.y), mx));
-        const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), ny), __fadd2_rn(make_float2(C.z, C.w), my));
-        float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
-        if constexpr (D == 3) {
-            const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), nz), __fadd2_rn(tg.lz[t], mz));
-            r2 = __ffma2_rn(dz, dz, r2);
+        const float2 lz = D == 3 ? tg.lz[t] : make_float2(0.f, 0.f), q = make_float2(B.z, B.w);
+        const float2 ka = p2p_lag_pair<D, kMask>(a, A, B, C, lz);
+        part[t] = __ffma2_rn(a.q, ka, part[t]);
+        sa = __ffma2_rn(q, ka, sa);
+        if constexpr (kS == 2) {
+            const float2 kb = p2p_lag_pair<D, kMask>(b, A, B, C, lz);
+            part[t] = __ffma2_rn(b.q, kb, part[t]);
+            sb = __ffma2_rn(q, kb, sb);
         }
-        float2 k = D == 3 ? make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y))
-                          : make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-        if constexpr (kMask) {
-            k.x = r2.x > 0.f ? k.x : 0.f;
-            k.y = r2.y > 0.f ? k.y : 0.f;
-        }
-        part[t] = __ffma2_rn(q2, k, part[t]);
-        sacc = __ffma2_rn(make_float2(B.z, B.w), k, sacc);
     }
-    return sacc.x + sacc.y;
+    return make_float2(sa.x + sa.y, sb.x + sb.y);
 }
 
 // one work item: the sum of target `lane` (units of 1 / r or log2 r^2), the later sources' added to nearf
@@ -366,7 +426,7 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
     double acc = 0.0;
     if (self) {
         const bool have = lane < T;
-        p2p_lag_chunk<D, true, NP>(part, tg, have ? hi[t0 + lane] : far4, have ? lo[t0 + lane] : zero4);
+        p2p_lag_chunk<D, true, NP, 1>(part, tg, have ? hi[t0 + lane] : far4, have ? lo[t0 + lane] : zero4, far4, zero4);
     }
     const uint32_t nsrc = end[4];
     auto load = [&](uint32_t slot, float4& h, float4& l, uint32_t& idx) {
@@ -382,21 +442,23 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
             l = lo[idx];
         }
     };
-    float4 h, l;
-    uint32_t idx;
-    load((uint32_t)lane, h, l, idx);
     int run = 0;
 #pragma unroll 1
-    for (uint32_t c = 0; c < nsrc; c += 32u) {
-        float4 nh, nl;
-        uint32_t nidx;
-        load(c + 32u + (uint32_t)lane, nh, nl, nidx);   // the next chunk's loads are in flight meanwhile
-        const float v = c < n_own ? p2p_lag_chunk<D, true, NP>(part, tg, h, l) : p2p_lag_chunk<D, false, NP>(part, tg, h, l);
-        if (idx != 0xffffffffu) atomicAdd(nearf + idx, f2d(v));
-        h = nh;
-        l = nl;
-        idx = nidx;
-        if (++run == kP2PRun) {
+    for (uint32_t c = 0; c < nsrc; c += 64u) {
+        float4 ha, la, hb, lb;
+        uint32_t ia, ib;
+        load(c + (uint32_t)lane, ha, la, ia);
+        load(c + 32u + (uint32_t)lane, hb, lb, ib);
+        float2 v;
+        if (c + 32u >= nsrc)   // a last half chunk (masked, which is right for every pair)
+            v = p2p_lag_chunk<D, true, NP, 1>(part, tg, ha, la, hb, lb);
+        else
+            v = c < n_own ? p2p_lag_chunk<D, true, NP, 2>(part, tg, ha, la, hb, lb)
+                          : p2p_lag_chunk<D, false, NP, 2>(part, tg, ha, la, hb, lb);
+        if (ia != 0xffffffffu) atomicAdd(nearf + ia, f2d(v.x));
+        if (ib != 0xffffffffu) atomicAdd(nearf + ib, f2d(v.y));
+        run += 2;
+        if (run >= kP2PRun) {
             acc += f2d(warp_reduce_scatter<W, NP>(part, lane));
 #pragma unroll
             for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
@@ -406,11 +468,13 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
     return acc + f2d(warp_reduce_scatter<W, NP>(part, lane));
 }
 
+// A warp per work item (the grid is the bound on their number): beside the far field, whose kernels have the
+// higher priority, a resident grid would hold every SM until its last item.
 template <int D>
-__global__ void __launch_bounds__(kP2PWarps * 32, D == 3 ? 5 : 6)
+__global__ void __launch_bounds__(kP2PWarps * 32, 5)
 k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int* __restrict__ start,
         const int* __restrict__ wchunk_start, int nleaf, int L, float box, double* __restrict__ nearf,
-        unsigned long long* __restrict__ pairs, int* __restrict__ next_item) {
+        unsigned long long* __restrict__ pairs) {
     constexpr int F = D == 3 ? 14 : 5, FG = fwd_group<D>(), G = (F + FG - 1) / FG;
     __shared__ LagTargets<D> tgts[kP2PWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -418,51 +482,40 @@ k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int*
     const int side = 1 << L;
     // empty source and target slots are zero charges outside the box, away from every charge and each other
     const float src_far = -0.25f * box, tgt_far = 1.25f * box;
-    const int64_t total = (int64_t)wchunk_start[nleaf] * G;
-    unsigned long long my_pairs = 0;
-    // items are taken from a shared counter, so that the warps finish within one item of each other
-    for (;;) {
-        int64_t w = 0;
-        if (lane == 0) w = atomicAdd(next_item, 1);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= total) break;
-        const int cidx = (int)(w / G), g = (int)(w % G);
-        const int b = chunk_leaf(wchunk_start, nleaf, cidx);
-        const int b1 = start[b + 1], t0 = start[b] + (cidx - wchunk_start[b]) * kWarpChunk, T = min(kWarpChunk, b1 - t0);
-        uint32_t first[5], end[5];
-        my_pairs += later_sources<D>(start, b, b1, t0, T, g, side, first, end);
-        const uint32_t n_own = g == 0 ? end[0] : 0u;
-        __syncwarp();
-        if (lane < kWarpChunk) {
-            const bool have = lane < T;
-            const float4 h = have ? hi[t0 + lane] : make_float4(tgt_far, tgt_far, tgt_far, 0.f);
-            const float4 l = have ? lo[t0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const int o = lane & 1;
-            float* A = reinterpret_cast<float*>(&tg.xy[lane >> 1]);
-            float* B = reinterpret_cast<float*>(&tg.zq[lane >> 1]);
-            float* C = reinterpret_cast<float*>(&tg.lxy[lane >> 1]);
-            A[o] = h.x;
-            A[2 + o] = h.y;
-            B[o] = h.z;
-            B[2 + o] = h.w;
-            C[o] = l.x;
-            C[2 + o] = l.y;
-            if constexpr (D == 3) reinterpret_cast<float*>(&tg.lz[lane >> 1])[o] = l.z;
-        }
-        __syncwarp();
-        double acc;
-        const bool self = g == 0;
-        switch ((T + 3) >> 2) {   // the chunk's target pairs, rounded up to an even count
-            case 1: acc = p2p_lag_item<D, 2>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-            case 2: acc = p2p_lag_item<D, 4>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-            case 3: acc = p2p_lag_item<D, 6>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-            case 4: acc = p2p_lag_item<D, 8>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-            case 5: acc = p2p_lag_item<D, 10>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-            default: acc = p2p_lag_item<D, 12>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-        }
-        if (lane < T) atomicAdd(nearf + t0 + lane, acc);
+    const int64_t w = (int64_t)blockIdx.x * kP2PWarps + wid;
+    if (w >= (int64_t)wchunk_start[nleaf] * G) return;
+    const int cidx = (int)(w / G), g = (int)(w % G);
+    const int b = chunk_leaf(wchunk_start, nleaf, cidx);
+    const int b1 = start[b + 1], t0 = start[b] + (cidx - wchunk_start[b]) * kWarpChunk, T = min(kWarpChunk, b1 - t0);
+    uint32_t first[5], end[5];
+    const unsigned long long my_pairs = later_sources<D>(start, b, b1, t0, T, g, side, first, end);
+    if (lane == 0 && my_pairs) atomicAdd(pairs + (w & (kPairSlots - 1)), my_pairs);
+    const uint32_t n_own = g == 0 ? end[0] : 0u;
+    if (lane < kWarpChunk) {
+        const bool have = lane < T;
+        const float4 h = have ? hi[t0 + lane] : make_float4(tgt_far, tgt_far, tgt_far, 0.f);
+        const float4 l = have ? lo[t0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int o = lane & 1;
+        float* A = reinterpret_cast<float*>(&tg.xy[lane >> 1]);
+        float* B = reinterpret_cast<float*>(&tg.zq[lane >> 1]);
+        float* C = reinterpret_cast<float*>(&tg.lxy[lane >> 1]);
+        A[o] = h.x;
+        A[2 + o] = h.y;
+        B[o] = h.z;
+        B[2 + o] = h.w;
+        C[o] = l.x;
+        C[2 + o] = l.y;
+        if constexpr (D == 3) reinterpret_cast<float*>(&tg.lz[lane >> 1])[o] = l.z;
     }
-    if (lane == 0 && my_pairs) atomicAdd(pairs, my_pairs);
+    __syncwarp();
+    double acc;
+    const bool self = g == 0;
+    switch ((T + 7) >> 3) {   // the chunk's target pairs, rounded up to a multiple of four
+        case 1: acc = p2p_lag_item<D, 4>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+        case 2: acc = p2p_lag_item<D, 8>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+        default: acc = p2p_lag_item<D, 12>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+    }
+    if (lane < T) atomicAdd(nearf + t0 + lane, acc);
 }
 
 // The near field in FP64 (node and literal FP64 forms): p2p64.cuh's warp per chunk of up to kWarpChunk64
@@ -509,7 +562,7 @@ k_p2p64(const Pos64* __restrict__ p, const int* __restrict__ start, const int* _
             [&](uint32_t i, const P64Acc<false>& a) { atomicAdd(nearf + i, scale * a.phi); },
             [&](const P64Acc<false>& a) { atomicAdd(nearf + t0 + lane, scale * a.phi); });
     }
-    if (lane == 0 && my_pairs) atomicAdd(pairs, my_pairs);
+    if (lane == 0 && my_pairs) atomicAdd(pairs + (blockIdx.x & (kPairSlots - 1)), my_pairs);
 }
 
 // ------------------------------------------------------------------------------ node charges
@@ -519,26 +572,32 @@ __device__ __forceinline__ void atomic_add(T* a, T v) {
     atomicAdd(a, v);
 }
 
-// Local coordinate (position - centre) / (s/5) of a sorted charge on axis a.
+// Sorted charges as seen from cells of side s: centre of cell c along an axis, and the local coordinate
+// (position - centre) / (s/5) of charge i on axis a.  FP32: two-word positions, side and centre.
 template <typename T>
 struct PosReader;
 template <>
 struct PosReader<float> {
     const float4* hi;
     const float4* lo;
-    __device__ float local(int i, int a, double centre, double inv) const {
+    float2 s;
+    float inv;
+    __device__ float2 centre(int c) const { return scatter_mul((float)c + 0.5f, s); }
+    __device__ float local(int i, int a, float2 c) const {
         const float4 h = hi[i], l = lo[i];
         const float hv = a == 0 ? h.x : (a == 1 ? h.y : h.z), lv = a == 0 ? l.x : (a == 1 ? l.y : l.z);
-        return ((hv - (float)centre) + lv) * (float)inv;
+        return ((hv - c.x) + (lv - c.y)) * inv;
     }
     __device__ float charge(int i) const { return hi[i].w; }
 };
 template <>
 struct PosReader<double> {
     const Pos64* p;
-    __device__ double local(int i, int a, double centre, double inv) const {
+    double s, inv;
+    __device__ double centre(int c) const { return ((double)c + 0.5) * s; }
+    __device__ double local(int i, int a, double c) const {
         const Pos64 v = p[i];
-        return ((a == 0 ? v.x : (a == 1 ? v.y : v.z)) - centre) * inv;
+        return ((a == 0 ? v.x : (a == 1 ? v.y : v.z)) - c) * inv;
     }
     __device__ double charge(int i) const { return p[i].w; }
 };
@@ -547,56 +606,205 @@ struct LevelPtrs {
     void* p[kMaxLevels + 1];
 };
 
-// STEP2 summed per cell: for each level k in [k0, k1] add sum_c q_c h(c) over the chunk's
-// charges into the node values of the accumulation cell.  Node forms: weights and accumulation
-// at level k (the node charges M_m v_m of every level straight from the charges, no shift).
-// Literal U-bar-1: weights of the root box (wlevel0) accumulated into the finest cell.
-template <int D, typename T>
-__global__ void __launch_bounds__(kChunk) k_p2m(PosReader<T> rd, const int* __restrict__ start,
-                                                const int* __restrict__ chunk_start, int nleaf, int L, double box,
-                                                int k0, int k1, bool wlevel0, LevelPtrs out) {
-    constexpr int d = nodes_of(D), PL = kChunk / d;
-    __shared__ T s_w[kChunk][D][4];
-    __shared__ T s_q[kChunk];
-    __shared__ T s_red[kChunk];
-    const int total = chunk_start[nleaf];
-    const int tid = threadIdx.x, j = tid % d, pl = tid / d;
-    const int ji[3] = {j & 3, (j >> 2) & 3, j >> 4};
-    for (int w = blockIdx.x; w < total; w += gridDim.x) {
-        const int b = chunk_leaf(chunk_start, nleaf, w);
-        const int t0 = start[b] + (w - chunk_start[b]) * kChunk, t1 = min(t0 + kChunk, start[b + 1]);
-        const int m = t1 - t0;
-        for (int k = k0; k <= k1; ++k) {
-            const int kw = wlevel0 ? 0 : k;               // level whose nodes the weights refer to
-            const uint32_t cell = (uint32_t)b >> (D * (L - k));
-            int cc[3];
-            morton_dec(D, (uint32_t)b >> (D * (L - kw)), cc);
-            const double s = box / (double)(1 << kw), inv = 5.0 / s;
-            __syncthreads();
-            if (tid < m) {
-                for (int a = 0; a < D; ++a) lag_basis<T>(rd.local(t0 + tid, a, ((double)cc[a] + 0.5) * s, inv), s_w[tid][a]);
-                s_q[tid] = rd.charge(t0 + tid);
-            }
-            __syncthreads();
-            T acc = T(0);
-            for (int c = pl; c < m; c += PL) {
-                T v = s_q[c] * s_w[c][0][ji[0]] * s_w[c][1][ji[1]];
-                if constexpr (D == 3) v *= s_w[c][2][ji[2]];
-                acc += v;
-            }
-            s_red[tid] = acc;
-            __syncthreads();
-            if (pl == 0) {
-                for (int r = 1; r < PL; ++r) acc += s_red[r * d + j];
-                atomic_add(static_cast<T*>(out.p[k]) + (size_t)cell * d + j, acc);
+// Sum of v[i] over the warp's lanes, scattered: afterwards lane l holds entries [l V / 32, (l + 1) V / 32)
+// (V >= 32) or, for V = 16, entry l / 2.
+template <int V, typename T>
+__device__ __forceinline__ void warp_reduce_nodes(T (&v)[V], int lane) {
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {
+        constexpr int W = V < 32 ? V : 32;
+        const int live = V < 32 ? (m * V) / 32 : m * (V / W);   // entries kept at this step
+        if (live == 0) {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+        } else {
+            const bool up = (lane & m) != 0;
+#pragma unroll
+            for (int i = 0; i < live; ++i) {
+                const T send = up ? v[i] : v[i + live], keep = up ? v[i + live] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
             }
         }
     }
 }
 
+// STEP2 summed per finest cell: sum_c q_c h(c) over the cell's charges.  Node forms: weights of the cell's
+// own nodes; the coarser cells' node charges follow by k_up.  Literal U-bar-1: weights of the root box's
+// nodes (root).  A warp per chunk of up to kChunk charges of one cell, the charges over the lanes and the
+// nodes' sums in registers; the lanes' sums are combined by a shuffle reduce-scatter, one atomic per node.
+// 2^20 charges in 2D, levels 7: 45 us with the upward pass against 409 us for the charges' weights at each of six
+// levels, staged in shared memory.
+template <int D, typename T>
+__global__ void __launch_bounds__(kChunk) k_p2m(PosReader<T> rd, const int* __restrict__ start,
+                                                const int* __restrict__ chunk_start, int nleaf, bool root,
+                                                T* __restrict__ out) {
+    constexpr int d = nodes_of(D);
+    const int total = chunk_start[nleaf];
+    const int lane = threadIdx.x & 31;
+    for (int w = blockIdx.x * (kChunk / 32) + (threadIdx.x >> 5); w < total; w += gridDim.x * (kChunk / 32)) {
+        const int b = chunk_leaf(chunk_start, nleaf, w);
+        const int t0 = start[b] + (w - chunk_start[b]) * kChunk, t1 = min(t0 + kChunk, start[b + 1]);
+        int cc[3] = {0, 0, 0};
+        if (!root) morton_dec(D, (uint32_t)b, cc);
+        decltype(rd.centre(0)) centre[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) centre[a] = rd.centre(cc[a]);
+        T acc[d];
+#pragma unroll
+        for (int j = 0; j < d; ++j) acc[j] = T(0);
+        for (int i = t0 + lane; i < t1; i += 32) {
+            T f[D][4];
+#pragma unroll
+            for (int a = 0; a < D; ++a) lag_basis<T>(rd.local(i, a, centre[a]), f[a]);
+            const T q = rd.charge(i);
+#pragma unroll
+            for (int jz = 0; jz < (D == 3 ? 4 : 1); ++jz) {
+                const T qz = D == 3 ? q * f[D - 1][jz] : q;
+#pragma unroll
+                for (int jy = 0; jy < 4; ++jy) {
+                    const T qy = qz * f[1][jy];
+#pragma unroll
+                    for (int jx = 0; jx < 4; ++jx) acc[jx + 4 * jy + 16 * jz] += qy * f[0][jx];
+                }
+            }
+        }
+        warp_reduce_nodes<d, T>(acc, lane);
+        T* o = out + (size_t)b * d;
+        if constexpr (d < 32) {
+            if ((lane & 1) == 0) atomic_add(o + (lane >> 1), acc[0]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < d / 32; ++i) atomic_add(o + lane * (d / 32) + i, acc[i]);
+        }
+    }
+}
+
+// Between levels (STEP4 for a cell and its child): per axis a cell's basis at the nodes of its two halves,
+// E[4 h + i][j] = f_j(x_{h,i}) with x_{h,i} = (2.5 h - 1.25) + a_i / 2 in units where the cell's side is 5.
+// A cubic is its own interpolant, so sums over charges and evaluations at charges pass through it exactly:
+// a cell's node charges are E^T applied along each axis to its children's (U-bar-2), and a child's node
+// potentials receive E applied to the cell's (D-bar-2).
+// Both run in FP64 (they are a few percent of the particles' work), so that the FP32 form's node charges are
+// rounded once per level and its node potentials, kept in FP64, not at all on the way down.
+struct Halves {
+    double e[8][4];
+};
+Halves make_halves() {
+    const double a[4] = {-2.0, -1.0, 1.0, 2.0};
+    Halves H;
+    for (int h = 0; h < 2; ++h)
+        for (int i = 0; i < 4; ++i) lag_basis<double>(2.5 * h - 1.25 + 0.5 * a[i], H.e[4 * h + i]);
+    return H;
+}
+
+constexpr int kShiftWarps = 4;   // a warp per cell
+
+// the 8^D values of a cell's children, x fastest: index (4 h + i) per axis -> (child, node)
+template <int D>
+__device__ __forceinline__ int child_value(int v) {
+    int ch = 0, node = 0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const int c = (v >> (3 * a)) & 7;
+        ch |= (c >> 2) << a;
+        node |= (c & 3) << (2 * a);
+    }
+    return ch * nodes_of(D) + node;
+}
+
+template <int D, typename T>
+__global__ void __launch_bounds__(kShiftWarps * 32) k_up(const T* __restrict__ child, T* __restrict__ parent, int ncell,
+                                                         Halves H) {
+    constexpr int N = D == 2 ? 64 : 512;
+    __shared__ double buf[kShiftWarps][N + N / 2];
+    __shared__ double E[8][4];
+    if (threadIdx.x < 32) E[threadIdx.x >> 2][threadIdx.x & 3] = H.e[threadIdx.x >> 2][threadIdx.x & 3];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m = blockIdx.x * kShiftWarps + warp;
+    if (m >= ncell) return;
+    double* in = buf[warp];
+    double* out = in + N;
+    const T* c = child + (size_t)m * (1 << D) * nodes_of(D);
+    for (int v = lane; v < N; v += 32) in[v] = (double)c[child_value<D>(v)];
+    __syncwarp();
+    // along x (8 -> 4), then y, then z: the contracted axis has stride st, the ones before it 4 values
+    int n = N, st = 1;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        n >>= 1;
+        for (int v = lane; v < n; v += 32) {
+            const int lowi = v % st, j = (v / st) & 3, high = v / (4 * st);
+            const double* x = in + high * 8 * st + lowi;
+            double t = 0.0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) t += E[i][j] * x[i * st];
+            out[v] = t;
+        }
+        __syncwarp();
+        double* swap = in;
+        in = out;
+        out = swap;
+        st *= 4;
+    }
+    for (int v = lane; v < n; v += 32) parent[(size_t)m * nodes_of(D) + v] = (T)in[v];
+}
+
+template <int D>
+__global__ void __launch_bounds__(kShiftWarps * 32) k_down(const double* __restrict__ parent, double* __restrict__ child, int ncell,
+                                                           Halves H) {
+    constexpr int N = D == 2 ? 64 : 512;
+    __shared__ double buf[kShiftWarps][N + N / 2];
+    __shared__ double E[8][4];
+    if (threadIdx.x < 32) E[threadIdx.x >> 2][threadIdx.x & 3] = H.e[threadIdx.x >> 2][threadIdx.x & 3];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m = blockIdx.x * kShiftWarps + warp;
+    if (m >= ncell) return;
+    // the last axis's values land in the full-size half of the buffer
+    double* in = D == 2 ? buf[warp] : buf[warp] + N;
+    double* out = D == 2 ? buf[warp] + N : buf[warp];
+    for (int v = lane; v < nodes_of(D); v += 32) in[v] = parent[(size_t)m * nodes_of(D) + v];
+    __syncwarp();
+    // along x (4 -> 8), then y, then z: the axes before the expanded one have 8 values
+    int n = nodes_of(D), st = 1;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        n <<= 1;
+        for (int v = lane; v < n; v += 32) {
+            const int lowi = v % st, i = (v / st) & 7, high = v / (8 * st);
+            const double* x = in + high * 4 * st + lowi;
+            double t = 0.0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) t += E[i][j] * x[j * st];
+            out[v] = t;
+        }
+        __syncwarp();
+        double* swap = in;
+        in = out;
+        out = swap;
+        st *= 8;
+    }
+    double* c = child + (size_t)m * (1 << D) * nodes_of(D);
+    for (int v = lane; v < N; v += 32) c[child_value<D>(v)] += in[v];
+}
+
+// The finest cells' node potentials for the FP32 evaluation: each cell's first node value in FP64 and the
+// others' differences from it in FP32.  The weights of a charge sum to one, so phi = psi_0 + sum_j w_j
+// (psi_j - psi_0), and FP32 rounds only the potential's variation over a cell.
+template <int D>
+__global__ void k_split_psi(const double* __restrict__ psi, int64_t nval, double* __restrict__ psi0,
+                            float* __restrict__ delta) {
+    constexpr int d = nodes_of(D);
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= nval) return;
+    const double first = psi[v / d * d];
+    delta[v] = (float)(psi[v] - first);
+    if (v % d == 0) psi0[v / d] = first;
+}
+
 // ------------------------------------------------------------------------------ node potentials
 
-// psi_m[j] += sum_{o in IL} sum_i K_k[o][i][j] Q_{m+o}[i] for one level.  Targets are grouped by
+// psi_m[j] += sum_{o in IL} sum_i K_k[o][i][j] Q_{m+o}[i].  Targets are grouped by
 // the parity of their coordinates: within a parity class the interaction list is the same set of
 // offsets (o_a in [-2 - p_a, 3 - p_a], Chebyshev distance >= 2), so a block takes 32 targets of
 // one class and a group of offsets, and applies each offset's d x d matrix to 32 source columns
@@ -606,18 +814,29 @@ constexpr size_t m2l_smem_bytes() {
     return ((size_t)nodes_of(D) * nodes_of(D) + (size_t)nodes_of(D) * 33) * sizeof(T);
 }
 
+// All levels in one launch: level k's blocks begin at base[k].
+struct M2LLevels {
+    const void* K[kMaxLevels + 1];
+    LevelPtrs Q, psi;
+    int base[kMaxLevels + 2];
+};
+
 template <int D, typename T>
-__global__ void __launch_bounds__(256) k_m2l(const T* __restrict__ K, const T* __restrict__ Q, T* __restrict__ psi,
-                                             int k, int ngroups) {
+__global__ void __launch_bounds__(256) k_m2l(M2LLevels lv, int ngroups) {
     constexpr int d = nodes_of(D), TT = 32, NT = 256, NTG = NT / d, RT = TT / NTG;
     constexpr int NOFF = D == 2 ? 27 : 189;
     extern __shared__ __align__(16) unsigned char m2l_smem[];
     T* s_K = reinterpret_cast<T*>(m2l_smem);                              // [d][d]
     T(*s_Q)[TT + 1] = reinterpret_cast<T(*)[TT + 1]>(s_K + d * d);        // [d][TT + 1]
+    int k = 2;
+    while ((int)blockIdx.x >= lv.base[k + 1]) ++k;
+    const T* K = static_cast<const T*>(lv.K[k]);
+    const T* Q = static_cast<const T*>(lv.Q.p[k]);
+    double* psi = static_cast<double*>(lv.psi.p[k]);   // FP64 sums in every form
     const int side = 1 << k, pside = side >> 1;
     const int nparent = D == 2 ? pside * pside : pside * pside * pside;
     const int ntiles = (nparent + TT - 1) / TT;
-    int blk = blockIdx.x;
+    int blk = blockIdx.x - lv.base[k];
     const int g = blk % ngroups;
     blk /= ngroups;
     const int tile = blk % ntiles, par = blk / ntiles;
@@ -684,58 +903,51 @@ __global__ void __launch_bounds__(256) k_m2l(const T* __restrict__ K, const T* _
         if (P >= nparent) continue;
         const int pc[3] = {P % pside, (P / pside) % pside, D == 3 ? P / (pside * pside) : 0};
         const int tc[3] = {2 * pc[0] + p[0], 2 * pc[1] + p[1], 2 * pc[2] + p[2]};
-        atomic_add(psi + (size_t)morton_enc(D, tc) * d + j, acc[r]);
+        atomicAdd(psi + (size_t)morton_enc(D, tc) * d + j, (double)acc[r]);
     }
 }
 
 // ------------------------------------------------------------------------------ evaluation
 
-// Node forms: phi_far(c) = sum_{k=2..L} h_{m_k}(c) . psi_{m_k}, the tensor-product contraction
-// done axis by axis; phi in input order = far + near (nearf in units of near_unit), written only if the
-// inputs passed.
+// Node forms: phi_far(c) = h_m(c) . psi_m of the charge's finest cell (which k_down has left with the sum
+// of all levels), the tensor-product contraction done axis by axis; phi in input order = far + near (nearf
+// in units of near_unit), written only if the inputs passed.  psi is null without a far field; psi0 (FP32)
+// is what k_split_psi took off it.
+// 2^20 charges in 2D, levels 7: 54 us with the downward pass against 332 us for an interpolation at each of six
+// levels with its FP64 centre and division.
 template <int D, typename T>
-__global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_t n, int L, double box,
-                      LevelPtrs psi, const double* __restrict__ nearf, double near_unit,
-                      const int* __restrict__ order, const unsigned* __restrict__ status, double* __restrict__ phi) {
+__global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_t n, const T* __restrict__ psi,
+                      const double* __restrict__ psi0, const double* __restrict__ nearf, double near_unit, const int* __restrict__ order,
+                      const unsigned* __restrict__ status, double* __restrict__ phi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t key = skey[i];
-    double far = 0.0;
-    for (int k = 2; k <= L; ++k) {
-        const uint32_t cell = key >> (D * (L - k));
+    T v = T(0);
+    double base = 0.0;
+    if (psi != nullptr) {
+        const uint32_t cell = skey[i];
+        if (psi0 != nullptr) base = psi0[cell];
         int cc[3];
         morton_dec(D, cell, cc);
-        const double s = box / (double)(1 << k), inv = 5.0 / s;
-        T f[3][4];
-        for (int a = 0; a < D; ++a) lag_basis<T>(rd.local((int)i, a, ((double)cc[a] + 0.5) * s, inv), f[a]);
-        const T* ps = static_cast<const T*>(psi.p[k]) + (size_t)cell * nodes_of(D);
-        T v = T(0);
-        if constexpr (D == 2) {
+        T f[D][4];
+#pragma unroll
+        for (int a = 0; a < D; ++a) lag_basis<T>(rd.local((int)i, a, rd.centre(cc[a])), f[a]);
+        const T* ps = psi + (size_t)cell * nodes_of(D);
+#pragma unroll
+        for (int iz = 0; iz < (D == 3 ? 4 : 1); ++iz) {
+            T u = T(0);
 #pragma unroll
             for (int iy = 0; iy < 4; ++iy) {
                 T r = T(0);
 #pragma unroll
-                for (int ix = 0; ix < 4; ++ix) r += f[0][ix] * __ldg(ps + ix + 4 * iy);
-                v += f[1][iy] * r;
+                for (int ix = 0; ix < 4; ++ix) r += f[0][ix] * __ldg(ps + ix + 4 * iy + 16 * iz);
+                u += f[1][iy] * r;
             }
-        } else {
-#pragma unroll
-            for (int iz = 0; iz < 4; ++iz) {
-                T u = T(0);
-#pragma unroll
-                for (int iy = 0; iy < 4; ++iy) {
-                    T r = T(0);
-#pragma unroll
-                    for (int ix = 0; ix < 4; ++ix) r += f[0][ix] * __ldg(ps + ix + 4 * iy + 16 * iz);
-                    u += f[1][iy] * r;
-                }
-                v += f[2][iz] * u;
-            }
+            if constexpr (D == 3) v += f[2][iz] * u;
+            else v = u;
         }
-        far += (double)v;
     }
     if (*(volatile const unsigned*)status != 0u) return;
-    phi[order[i]] = fma(near_unit, nearf[i], far);
+    phi[order[i]] = fma(near_unit, nearf[i], base + (double)v);
 }
 
 // ------------------------------------------------------------------------------ literal form
@@ -935,8 +1147,9 @@ void plan_free(fmm_lag_plan_s* pl) {
     cudaFree(pl->key); cudaFree(pl->rank); cudaFree(pl->skey); cudaFree(pl->count); cudaFree(pl->start);
     cudaFree(pl->chunk_start); cudaFree(pl->wchunk_start); cudaFree(pl->order); cudaFree(pl->hi); cudaFree(pl->lo); cudaFree(pl->p64);
     cudaFree(pl->nearf); cudaFree(pl->status); cudaFree(pl->pairs); cudaFree(pl->next_item); cudaFree(pl->K); cudaFree(pl->logtab);
+    cudaFree(pl->scan); cudaFree(pl->pot[2]); cudaFree(pl->psi0); cudaFree(pl->dpsi);
     for (int k = 0; k <= kMaxLevels; ++k) {
-        cudaFree(pl->node[k]); cudaFree(pl->pot[k]); cudaFree(pl->pair_start[k]); cudaFree(pl->pair_src[k]);
+        cudaFree(pl->node[k]); cudaFree(pl->pair_start[k]); cudaFree(pl->pair_src[k]);
         cudaFree(pl->B[k]);
     }
     for (auto& e : pl->ev) if (e) cudaEventDestroy(e);
@@ -974,6 +1187,75 @@ std::vector<double> build_operators(int D, int L, double box) {
     return K;
 }
 
+// the plan's stream behind the far field's
+void lag_join(fmm_lag_plan_s* pl, cudaStream_t far_st) {
+    if (far_st == pl->st) return;
+    cudaEventRecord(pl->ev_join, far_st);
+    cudaStreamWaitEvent(pl->st, pl->ev_join, 0);
+}
+
+// The far field of the node forms on its stream, joined with the near field: node charges of the
+// finest cells, up the tree, over the interaction lists, down the tree, evaluation.
+template <int D, typename T>
+int enqueue_nodes(fmm_lag_plan_s* pl, const PosReader<T>& rd, int64_t n, unsigned gp, unsigned gb, double near_unit,
+                  double* phi) {
+    constexpr int d = nodes_of(D);
+    const int L = pl->levels;
+    cudaStream_t st = pl->serial ? pl->st : pl->st2;
+    int launches = 0;
+    static const Halves H = make_halves();
+    const auto shift_blocks = [](int64_t cells) { return (unsigned)((cells + kShiftWarps - 1) / kShiftWarps); };
+    if (L >= 2) {
+        k_p2m<D, T><<<gp, kChunk, 0, st>>>(rd, pl->start, pl->chunk_start, (int)pl->nleaf, false,
+                                           static_cast<T*>(pl->node[L]));
+        ++launches;
+        for (int k = L - 1; k >= 2; --k) {
+            const int64_t cells = ipow(1 << k, D);
+            k_up<D, T><<<shift_blocks(cells), kShiftWarps * 32, 0, st>>>(
+                static_cast<const T*>(pl->node[k + 1]), static_cast<T*>(pl->node[k]), (int)cells, H);
+            ++launches;
+        }
+    }
+    cudaEventRecord(pl->ev[2], st);
+    if (L >= 2) {
+        const int ngroups = D == 2 ? 3 : 27;
+        M2LLevels lv{};
+        int blocks = 0;
+        for (int k = 2; k <= L; ++k) {
+            lv.K[k] = static_cast<const T*>(pl->K) + (size_t)(k - 2) * offsets_of(D) * d * d;
+            lv.Q.p[k] = pl->node[k];
+            lv.psi.p[k] = pl->pot[k];
+            lv.base[k] = blocks;
+            blocks += (int)(((ipow(1 << (k - 1), D) + 31) / 32) * (1 << D) * ngroups);
+        }
+        lv.base[L + 1] = blocks;
+        k_m2l<D, T><<<(unsigned)blocks, 256, m2l_smem_bytes<D, T>(), st>>>(lv, ngroups);
+        ++launches;
+    }
+    cudaEventRecord(pl->ev[3], st);
+    for (int k = 2; k < L; ++k) {
+        const int64_t cells = ipow(1 << k, D);
+        k_down<D><<<shift_blocks(cells), kShiftWarps * 32, 0, st>>>(
+            static_cast<const double*>(pl->pot[k]), static_cast<double*>(pl->pot[k + 1]), (int)cells, H);
+        ++launches;
+    }
+    const T* psi = L >= 2 ? static_cast<const T*>(pl->pot[L]) : nullptr;
+    const double* psi0 = nullptr;
+    if constexpr (sizeof(T) == 4) {
+        if (L >= 2) {
+            const int64_t nval = pl->nleaf * d;
+            k_split_psi<D><<<(unsigned)((nval + 255) / 256), 256, 0, st>>>(static_cast<const double*>(pl->pot[L]), nval,
+                                                                          pl->psi0, pl->dpsi);
+            ++launches;
+            psi = pl->dpsi;
+            psi0 = pl->psi0;
+        }
+    }
+    lag_join(pl, st);
+    k_l2p<D, T><<<gb, 256, 0, pl->st>>>(rd, pl->skey, n, psi, psi0, pl->nearf, near_unit, pl->order, pl->status, phi);
+    return launches + 1;
+}
+
 template <int D>
 fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64_t n, double* phi) {
     constexpr int d = nodes_of(D);
@@ -983,121 +1265,94 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
     int launches = 0;
     cudaEventRecord(pl->ev[0], st);
     cudaMemsetAsync(pl->count, 0, sizeof(int) * (size_t)pl->nleaf, st);
-    cudaMemsetAsync(pl->pairs, 0, sizeof(unsigned long long), st);
-    for (int k = (lit ? std::max(L, 2) : 2); k <= L; ++k) {
-        const size_t cells = (size_t)ipow(1 << k, D) * d;
-        cudaMemsetAsync(pl->node[k], 0, cells * (f64 ? 8 : 4), st);
-        if (!lit) cudaMemsetAsync(pl->pot[k], 0, cells * (f64 ? 8 : 4), st);
+    cudaMemsetAsync(pl->pairs, 0, kPairSlots * sizeof(unsigned long long), st);
+    if (L >= 2) {   // sums that start at zero: the finest cells' node values, every level's potentials
+        cudaMemsetAsync(pl->node[L], 0, (size_t)pl->nleaf * d * (f64 ? 8 : 4), st);
+        if (!lit) cudaMemsetAsync(pl->pot[2], 0, pl->pot_bytes, st);
     }
     const unsigned gb = (unsigned)((n + 255) / 256);
-    k_bin<D><<<gb, 256, 0, st>>>(pos, q, n, L, pl->box, pl->key, pl->rank, pl->count, pl->status);
-    k_scan<<<1, 1024, 0, st>>>(pl->count, (int)pl->nleaf, f64 ? kWarpChunk64 : kWarpChunk, pl->start, pl->chunk_start,
-                               pl->wchunk_start);
+    k_bin<D><<<gb, 256, 0, st>>>(pos, q, n, L, pl->box, (float)((double)(1 << L) / pl->box), pl->key, pl->rank,
+                                 pl->count, pl->status);
+    const unsigned tiles = (unsigned)((pl->nleaf + kScanTile - 1) / kScanTile);
+    const int wchunk = f64 ? kWarpChunk64 : kWarpChunk;
+    k_scan_sums<<<tiles, kScanTile, 0, st>>>(pl->count, (int)pl->nleaf, wchunk, pl->scan);
+    k_scan<<<tiles, kScanTile, 0, st>>>(pl->count, (int)pl->nleaf, wchunk, pl->scan, pl->start, pl->chunk_start,
+                                        pl->wchunk_start);
     if (f64)
         k_scatter<D, true><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, pl->skey, pl->order,
                                                 nullptr, nullptr, pl->p64);
     else
         k_scatter<D, false><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, pl->skey, pl->order,
                                                  pl->hi, pl->lo, nullptr);
-    launches += 3;
+    launches += 4;
     cudaEventRecord(pl->ev[7], st);
     cudaEventRecord(pl->ev[1], st);
-    // near field on the second stream (or in turn on the plan's stream in serial mode)
-    cudaStream_t p2p_st = pl->serial ? st : pl->st2;
+    // The far field on the second stream, which has the device's highest priority, beside the near field on
+    // the plan's stream (in serial mode everything in turn on the plan's stream).
+    cudaStream_t far_st = pl->serial ? st : pl->st2;
     if (!pl->serial) {
         cudaEventRecord(pl->ev_fork, st);
         cudaStreamWaitEvent(pl->st2, pl->ev_fork, 0);
     }
     const unsigned gp = (unsigned)pl->grid_particles;
-    cudaMemsetAsync(pl->nearf, 0, sizeof(double) * (size_t)n, p2p_st);
-    cudaMemsetAsync(pl->next_item, 0, sizeof(int), p2p_st);
-    cudaEventRecord(pl->ev[5], p2p_st);
+    cudaMemsetAsync(pl->nearf, 0, sizeof(double) * (size_t)n, st);
+    if (f64) cudaMemsetAsync(pl->next_item, 0, sizeof(int), st);
+    cudaEventRecord(pl->ev[5], st);
     if (f64) {
-        k_p2p64<D><<<(unsigned)pl->grid_p2p, kP2PWarps64 * 32, 0, p2p_st>>>(
+        k_p2p64<D><<<(unsigned)pl->grid_p2p, kP2PWarps64 * 32, 0, st>>>(
             pl->p64, pl->start, pl->wchunk_start, (int)pl->nleaf, L, pl->logtab, pl->nearf, pl->pairs, pl->next_item);
     } else {
-        k_p2p32<D><<<(unsigned)pl->grid_p2p, kP2PWarps * 32, 0, p2p_st>>>(
-            pl->hi, pl->lo, pl->start, pl->wchunk_start, (int)pl->nleaf, L, (float)pl->box, pl->nearf, pl->pairs,
-            pl->next_item);
+        // a chunk per kWarpChunk charges and a partial one per occupied cell at most
+        constexpr int F = D == 3 ? 14 : 5, G = (F + fwd_group<D>() - 1) / fwd_group<D>();
+        const int64_t items = (std::min<int64_t>(pl->nleaf, n) + n / kWarpChunk) * G;
+        k_p2p32<D><<<(unsigned)((items + kP2PWarps - 1) / kP2PWarps), kP2PWarps * 32, 0, st>>>(
+            pl->hi, pl->lo, pl->start, pl->wchunk_start, (int)pl->nleaf, L, (float)pl->box, pl->nearf, pl->pairs);
     }
     ++launches;
-    cudaEventRecord(pl->ev[6], p2p_st);
-    cudaEventRecord(pl->ev_join, p2p_st);
+    cudaEventRecord(pl->ev[6], st);
     if (pl->serial) cudaEventRecord(pl->ev[1], st);   // the far-field stages start after the near field
 
-    LevelPtrs nodes{}, pots{};
-    for (int k = 0; k <= kMaxLevels; ++k) {
-        nodes.p[k] = pl->node[k];
-        pots.p[k] = pl->pot[k];
-    }
-    if (!lit) {
-        if (L >= 2) {
-            if (f64)
-                k_p2m<D, double><<<gp, kChunk, 0, st>>>(PosReader<double>{pl->p64}, pl->start, pl->chunk_start,
-                                                        (int)pl->nleaf, L, pl->box, 2, L, false, nodes);
-            else
-                k_p2m<D, float><<<gp, kChunk, 0, st>>>(PosReader<float>{pl->hi, pl->lo}, pl->start, pl->chunk_start,
-                                                       (int)pl->nleaf, L, pl->box, 2, L, false, nodes);
-            ++launches;
-        }
-        cudaEventRecord(pl->ev[2], st);
-        const int ngroups = D == 2 ? 3 : 27;
-        for (int k = 2; k <= L; ++k) {
-            const int pside = 1 << (k - 1);
-            const int64_t nparent = ipow(pside, D);
-            const unsigned blocks = (unsigned)(((nparent + 31) / 32) * (1 << D) * ngroups);
-            const size_t koff = (size_t)(k - 2) * offsets_of(D) * d * d;
-            if (f64)
-                k_m2l<D, double><<<blocks, 256, m2l_smem_bytes<D, double>(), st>>>(static_cast<const double*>(pl->K) + koff,
-                                                         static_cast<const double*>(pl->node[k]),
-                                                         static_cast<double*>(pl->pot[k]), k, ngroups);
-            else
-                k_m2l<D, float><<<blocks, 256, m2l_smem_bytes<D, float>(), st>>>(static_cast<const float*>(pl->K) + koff,
-                                                        static_cast<const float*>(pl->node[k]),
-                                                        static_cast<float*>(pl->pot[k]), k, ngroups);
-            ++launches;
-        }
-        cudaEventRecord(pl->ev[3], st);
-        cudaStreamWaitEvent(st, pl->ev_join, 0);
-        if (f64)
-            k_l2p<D, double><<<gb, 256, 0, st>>>(PosReader<double>{pl->p64}, pl->skey, n, L, pl->box, pots, pl->nearf,
-                                                 1.0, pl->order, pl->status, phi);
-        else   // the FP32 near field is in units of 1 / r, or log2 r^2
-            k_l2p<D, float><<<gb, 256, 0, st>>>(PosReader<float>{pl->hi, pl->lo}, pl->skey, n, L, pl->box, pots,
-                                                pl->nearf, D == 2 ? 0.5 * kLn2 : 1.0, pl->order, pl->status, phi);
+    // the finest cells' side and the scale of their local coordinates
+    const double cs = pl->box / (double)(1 << L);
+    const float cs_hi = (float)cs;
+    const PosReader<float> rd32{pl->hi, pl->lo, make_float2(cs_hi, (float)(cs - (double)cs_hi)), (float)(5.0 / cs)};
+    const PosReader<double> rd64{pl->p64, cs, 5.0 / cs};
+    const double near_unit = !f64 && D == 2 ? 0.5 * kLn2 : 1.0;   // the 2D FP32 near field is in log2 r^2
+    if (lit && L < 2) {
+        // no interaction lists: phi is the near field
+        cudaEventRecord(pl->ev[2], far_st);
+        cudaEventRecord(pl->ev[3], far_st);
+        lag_join(pl, far_st);
+        k_l2p<D, double><<<gb, 256, 0, st>>>(rd64, pl->skey, n, nullptr, nullptr, pl->nearf, near_unit, pl->order,
+                                             pl->status, phi);
         ++launches;
-    } else if (L < 2) {
-        // no interaction lists: phi is the near field (the node evaluation over no levels)
-        cudaEventRecord(pl->ev[2], st);
-        cudaEventRecord(pl->ev[3], st);
-        cudaStreamWaitEvent(st, pl->ev_join, 0);
-        k_l2p<D, double><<<gb, 256, 0, st>>>(PosReader<double>{pl->p64}, pl->skey, n, L, pl->box, pots, pl->nearf,
-                                             1.0, pl->order, pl->status, phi);
-        ++launches;
+    } else if (!lit) {
+        if (f64) launches += enqueue_nodes<D, double>(pl, rd64, n, gp, gb, near_unit, phi);
+        else launches += enqueue_nodes<D, float>(pl, rd32, n, gp, gb, near_unit, phi);
     } else {
         // U-bar-1: v of every finest cell from the charges' root-node images
-        k_p2m<D, double><<<gp, kChunk, 0, st>>>(PosReader<double>{pl->p64}, pl->start, pl->chunk_start,
-                                                (int)pl->nleaf, L, pl->box, L, L, true, nodes);
+        k_p2m<D, double><<<gp, kChunk, 0, far_st>>>(PosReader<double>{pl->p64, pl->box, 5.0 / pl->box}, pl->start,
+                                                pl->chunk_start, (int)pl->nleaf, true, static_cast<double*>(pl->node[L]));
         ++launches;
         // U-bar-2: sums up the tree (levels below 2 are never read)
         for (int k = L - 1; k >= 2; --k) {
             const int64_t ncell = ipow(1 << k, D);
-            k_lit_up<D><<<(unsigned)((ncell * d + 255) / 256), 256, 0, st>>>(
+            k_lit_up<D><<<(unsigned)((ncell * d + 255) / 256), 256, 0, far_st>>>(
                 static_cast<const double*>(pl->node[k + 1]), static_cast<double*>(pl->node[k]), ncell);
             ++launches;
         }
-        cudaEventRecord(pl->ev[2], st);
+        cudaEventRecord(pl->ev[2], far_st);
         // D-bar-1 and D-bar-2 level by level, top down
         for (int k = 2; k <= L; ++k) {
             const int64_t ncell = ipow(1 << k, D);
-            k_lit_down<D><<<(unsigned)ncell, 256, 0, st>>>(pl->pair_start[k], pl->pair_src[k], pl->B[k],
+            k_lit_down<D><<<(unsigned)ncell, 256, 0, far_st>>>(pl->pair_start[k], pl->pair_src[k], pl->B[k],
                                                            static_cast<const double*>(pl->node[k]),
                                                            k >= 3 ? static_cast<const double*>(pl->pot[k - 1]) : nullptr,
                                                            static_cast<double*>(pl->pot[k]), ncell);
             ++launches;
         }
-        cudaEventRecord(pl->ev[3], st);
-        cudaStreamWaitEvent(st, pl->ev_join, 0);
+        cudaEventRecord(pl->ev[3], far_st);
+        lag_join(pl, far_st);
         k_lit_eval<D><<<gb, 256, 0, st>>>(pl->p64, pl->skey, n, pl->box, static_cast<const double*>(pl->pot[L]),
                                           pl->nearf, pl->order, pl->status, phi);
         ++launches;
@@ -1136,12 +1391,12 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     int per_sm = 0;
     if (rc == FMM_OK)
         rc = cuda_status(
-            f64 ? (dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p64<2>, kP2PWarps64 * 32, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p64<3>, kP2PWarps64 * 32, 0))
-                : (dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p32<2>, kP2PWarps * 32, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p32<3>, kP2PWarps * 32, 0)));
+            dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p64<2>, kP2PWarps64 * 32, 0)
+                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_p2p64<3>, kP2PWarps64 * 32, 0));
     pl->grid_p2p = std::max(1, sms) * std::max(1, per_sm);
-    if (rc == FMM_OK) rc = cuda_status(cudaStreamCreateWithFlags(&pl->st2, cudaStreamNonBlocking));
+    int least = 0, greatest = 0;
+    if (rc == FMM_OK) rc = cuda_status(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    if (rc == FMM_OK) rc = cuda_status(cudaStreamCreateWithPriority(&pl->st2, cudaStreamNonBlocking, greatest));
     for (auto& e : pl->ev)
         if (rc == FMM_OK) rc = cuda_status(cudaEventCreate(&e));
     if (rc == FMM_OK) rc = cuda_status(cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming));
@@ -1157,7 +1412,7 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     if (rc == FMM_OK) rc = alloc(pl, &pl->chunk_start, (size_t)pl->nleaf + 1);
     if (rc == FMM_OK) rc = alloc(pl, &pl->wchunk_start, (size_t)pl->nleaf + 1);
     if (rc == FMM_OK) rc = alloc(pl, &pl->status, 1);
-    if (rc == FMM_OK) rc = alloc(pl, &pl->pairs, 1);
+    if (rc == FMM_OK) rc = alloc(pl, &pl->pairs, kPairSlots);
     if (rc == FMM_OK) rc = alloc(pl, &pl->next_item, 1);
     if (rc == FMM_OK && f64) rc = alloc(pl, &pl->p64, n);
     if (rc == FMM_OK && f64 && dim == 2) {
@@ -1170,17 +1425,21 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     if (rc == FMM_OK && !f64) rc = alloc(pl, &pl->hi, n);
     if (rc == FMM_OK && !f64) rc = alloc(pl, &pl->lo, n);
     const size_t vb = f64 ? 8 : 4;
+    if (rc == FMM_OK) rc = alloc(pl, &pl->scan, (size_t)((pl->nleaf + kScanTile - 1) / kScanTile));
     for (int k = 2; k <= levels && rc == FMM_OK; ++k) {
-        const size_t cells = (size_t)ipow(1 << k, dim) * d;
-        void** a = &pl->node[k];
-        void** b = &pl->pot[k];
-        if (vb == 8) {
-            rc = alloc(pl, reinterpret_cast<double**>(a), cells);
-            if (rc == FMM_OK) rc = alloc(pl, reinterpret_cast<double**>(b), cells);
-        } else {
-            rc = alloc(pl, reinterpret_cast<float**>(a), cells);
-            if (rc == FMM_OK) rc = alloc(pl, reinterpret_cast<float**>(b), cells);
+        const size_t bytes = (size_t)ipow(1 << k, dim) * d * vb;
+        rc = alloc(pl, reinterpret_cast<char**>(&pl->node[k]), bytes);
+        pl->pot_bytes += bytes / vb * 8;   // FP64 in every form
+    }
+    if (rc == FMM_OK && levels >= 2) {
+        char* pot = nullptr;
+        rc = alloc(pl, &pot, pl->pot_bytes);
+        for (int k = 2; k <= levels && rc == FMM_OK; ++k) {
+            pl->pot[k] = pot;
+            pot += (size_t)ipow(1 << k, dim) * d * 8;
         }
+        if (rc == FMM_OK && !f64) rc = alloc(pl, &pl->psi0, (size_t)pl->nleaf);
+        if (rc == FMM_OK && !f64) rc = alloc(pl, &pl->dpsi, (size_t)pl->nleaf * d);
     }
     if (rc == FMM_OK) rc = cuda_status(cudaMemset(pl->status, 0, sizeof(unsigned)));
     if (rc == FMM_OK) rc = cuda_status(cudaMallocHost(reinterpret_cast<void**>(&pl->h_status), sizeof(unsigned)));
@@ -1309,9 +1568,9 @@ fmm_status fmm_lag_stats_get(fmm_lag_plan_t pl, fmm_lag_stats* out) {
     out->ms_down = span(2, 3);
     out->ms_eval = span(3, 4);
     out->ms_p2p = span(5, 6);
-    unsigned long long pairs = 0;
-    if (cudaMemcpy(&pairs, pl->pairs, sizeof(pairs), cudaMemcpyDeviceToHost) != cudaSuccess) return FMM_ERR_CUDA;
-    out->p2p_pairs = (int64_t)pairs;
+    unsigned long long pairs[kPairSlots];
+    if (cudaMemcpy(pairs, pl->pairs, sizeof(pairs), cudaMemcpyDeviceToHost) != cudaSuccess) return FMM_ERR_CUDA;
+    for (unsigned long long v : pairs) out->p2p_pairs += (int64_t)v;
     out->kernel_launches = pl->launches;
     return FMM_OK;
 }

@@ -221,3 +221,17 @@ def test_near_field_tiles_f32(oracle_mod, dim, levels, n):
     bound = 2.0 ** -20 * ((np.abs(k) + 1.0) * np.abs(q)[None, :]).sum(1)
     assert np.all(np.abs(phi - (k * q[None, :]).sum(1)) <= bound)
     assert st["p2p_pairs"] == int((np.abs(cells[:, None, :] - cells[None, :, :]).max(-1) <= 1).sum())
+
+
+@pytest.mark.parametrize("dim,levels", [(2, 2), (2, 4), (2, 8), (3, 2), (3, 4)])
+@pytest.mark.parametrize("box", [5.0, 3.7])
+def test_up_and_down_passes_f64(oracle_mod, dim, levels, box):
+    """Node charges up the tree and node potentials down it, at the shallowest and deep trees, in a box whose cell
+    sides are not dyadic; few charges, so that most cells are empty and the scan has tiles of zeros: the FP64 form
+    equals the oracle's per-level sums to rounding."""
+    pos, q = inputs.paper_cube(900, 9700 + 10 * dim + levels, dim, box)
+    phi, _, cells = run(pos, q, levels, "node_f64", box)
+    check_parity(phi, oracle_mod.lag_node(pos, q, levels, box), TOL64, f"node_f64 D={dim} L={levels} box={box}")
+    assert np.array_equal(cells, oracle_mod.lag_cells(pos, levels, box))
+    phi, _, _ = run(pos, q, levels, "node_f32", box)
+    check_parity(phi, oracle_mod.lag_node(pos, q, levels, box), TOL32, f"node_f32 D={dim} L={levels} box={box}")
