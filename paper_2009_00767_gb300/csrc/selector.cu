@@ -26,8 +26,14 @@ constexpr int kHistLevels = kLevMax - kLevMin + 1;
 constexpr int kFeat = kHistLevels * kBins + 1;   // 109
 constexpr int kIn = kFeat + 2;                   // + candidate levels / 12, p / 32
 constexpr int kOut = 2;
+constexpr size_t kOccFine = (size_t)1 << (2 * kLevMax);        // squares of the finest level counted
+constexpr size_t kOccTiles = (size_t)1 << (2 * (kLevMax - 5));   // its tiles of 32 x 32: level 6
+static_assert(kLevMin == 3 && kLevMax == 11, "k_occ_tile<5> takes levels 11..7, k_occ_tile<4> levels 6..3");
 
 // ---------------------------------------------------------------- occupancy statistics
+// One count per particle, in its square of the finest level; the coarser levels' populations are sums of
+// four.  What bounds it: the atomics in L2, so a ninth of them.  2^20 particles: a call of fmm_selector_features
+// and one of fmm_select take 213 us together, 1087 us with an atomic per particle and level.
 __global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double box, uint32_t* __restrict__ cnt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -36,32 +42,63 @@ __global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double bo
     const int side = 1 << kLevMax;
     const int ix = finest_coord(p.x, (double)side, sob, box, side);
     const int iy = finest_coord(p.y, (double)side, sob, box, side);
-    size_t off = 0;
-    for (int k = kLevMin; k <= kLevMax; ++k) {
-        const int sh = kLevMax - k;
-        atomicAdd(&cnt[off + ((size_t)(iy >> sh) << k) + (ix >> sh)], 1u);
-        off += (size_t)1 << (2 * k);
-    }
+    atomicAdd(&cnt[((size_t)iy << kLevMax) + ix], 1u);
 }
 
-__global__ void k_occ_hist(const uint32_t* __restrict__ cnt, size_t total, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[kHistLevels * kBins];
-    for (int i = threadIdx.x; i < kHistLevels * kBins; i += blockDim.x) h[i] = 0u;
+__device__ __forceinline__ int occ_bin(uint32_t c) { return min(kBins - 1, 31 - __clz(c + 1u)); }   // floor(log2(c + 1))
+
+// Occupancies of a 32 x 32 tile of level-k squares (cnt, row-major) and of the kLevels - 1 levels above them:
+// histograms to hist and, with five levels, the tile's own population, that of a square of level k - 5, to
+// `up`.  A 256-thread block, a thread per 2 x 2 squares; lanes vote on each bin, so that a level costs one
+// shared atomic per warp and bin.
+template <int kLevels>
+__global__ void __launch_bounds__(256) k_occ_tile(const uint32_t* __restrict__ cnt, int k, uint32_t* __restrict__ up,
+                                                  uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[kLevels * kBins];
+    __shared__ uint32_t pop[256];
+    const int t = threadIdx.x, lane = t & 31;
+    for (int i = t; i < kLevels * kBins; i += 256) h[i] = 0u;
     __syncthreads();
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        int k = kLevMin;
-        size_t off = 0;
-        while (e >= off + ((size_t)1 << (2 * k))) {
-            off += (size_t)1 << (2 * k);
-            ++k;
-        }
-        const uint32_t c = cnt[e];
-        const int bin = min(kBins - 1, 31 - __clz(c + 1u));   // floor(log2(c + 1))
-        atomicAdd(&h[(k - kLevMin) * kBins + bin], 1u);
+    const int tiles = 1 << (k - 5);
+    const int tx = blockIdx.x % tiles, ty = blockIdx.x / tiles;
+    const int x = t & 15, y = t >> 4;
+    const size_t at = ((size_t)(32 * ty + 2 * y) << k) + 32 * tx + 2 * x;
+    const uint2 a = *reinterpret_cast<const uint2*>(cnt + at);
+    const uint2 b = *reinterpret_cast<const uint2*>(cnt + at + ((size_t)1 << k));
+    const int ba = occ_bin(a.x), bb = occ_bin(a.y), bc = occ_bin(b.x), bd = occ_bin(b.y);
+#pragma unroll
+    for (int i = 0; i < kBins; ++i) {
+        const int c = __popc(__ballot_sync(0xffffffffu, ba == i)) + __popc(__ballot_sync(0xffffffffu, bb == i)) +
+                      __popc(__ballot_sync(0xffffffffu, bc == i)) + __popc(__ballot_sync(0xffffffffu, bd == i));
+        if (lane == 0 && c) atomicAdd(&h[i], (uint32_t)c);
     }
+    pop[t] = a.x + a.y + b.x + b.y;
     __syncthreads();
-    for (int i = threadIdx.x; i < kHistLevels * kBins; i += blockDim.x)
-        if (h[i]) atomicAdd(&hist[i], h[i]);
+    // 16 x 16 squares of level k - 1, then a quarter of them a level
+#pragma unroll
+    for (int l = 1; l < kLevels; ++l) {
+        const int w = 32 >> l;   // squares a side at this level
+        const bool on = t < w * w;
+        const int bin = on ? occ_bin(pop[t]) : -1;
+        if ((t & ~31) < w * w)
+#pragma unroll
+            for (int i = 0; i < kBins; ++i) {
+                const int c = __popc(__ballot_sync(0xffffffffu, bin == i));
+                if (lane == 0 && c) atomicAdd(&h[l * kBins + i], (uint32_t)c);
+            }
+        const int hw = w / 2;
+        uint32_t v = 0;
+        if (t < hw * hw) {
+            const int o = 2 * (t / hw) * w + 2 * (t % hw);
+            v = pop[o] + pop[o + 1] + pop[o + w] + pop[o + w + 1];
+        }
+        __syncthreads();
+        if (t < hw * hw) pop[t] = v;
+        __syncthreads();
+    }
+    if (up && t == 0) up[blockIdx.x] = pop[0];
+    for (int i = t; i < kLevels * kBins; i += 256)
+        if (h[i]) atomicAdd(&hist[(k - i / kBins - kLevMin) * kBins + i % kBins], h[i]);
 }
 
 // ---------------------------------------------------------------- dense layers
@@ -142,9 +179,9 @@ struct fmm_selector_s {
     // activations for a batch of up to cap rows
     int cap;
     float *x, *h1, *h2, *y, *t, *dy, *dh2, *dh1, *lrow;
-    uint32_t* cnt;                   // occupancy counters of levels 3..11
+    uint32_t* cnt;                   // populations of level 11, then of level 6
     uint32_t* hist;
-    size_t ncnt;
+    uint32_t* h_hist;                // pinned
 };
 
 namespace {
@@ -254,13 +291,12 @@ fmm_status fmm_selector_create(fmm_selector_t* out, int hidden, uint64_t seed, v
     s->hidden = hidden;
     s->stream = static_cast<cudaStream_t>(stream);
     s->np = kIn * hidden + hidden + hidden * hidden + hidden + hidden * kOut + kOut;
-    s->ncnt = 0;
-    for (int k = kLevMin; k <= kLevMax; ++k) s->ncnt += (size_t)1 << (2 * k);
     bool ok = cudaMalloc(&s->w, sizeof(float) * s->np) == cudaSuccess &&
               cudaMalloc(&s->g, sizeof(float) * s->np) == cudaSuccess &&
               cudaMalloc(&s->m, sizeof(float) * s->np) == cudaSuccess &&
               cudaMalloc(&s->v, sizeof(float) * s->np) == cudaSuccess &&
-              cudaMalloc(&s->cnt, sizeof(uint32_t) * s->ncnt) == cudaSuccess &&
+              cudaMalloc(&s->cnt, sizeof(uint32_t) * (kOccFine + kOccTiles)) == cudaSuccess &&
+              cudaMallocHost(&s->h_hist, sizeof(uint32_t) * kHistLevels * kBins) == cudaSuccess &&
               cudaMalloc(&s->hist, sizeof(uint32_t) * kHistLevels * kBins) == cudaSuccess;
     std::vector<float> w;
     init_weights(s, seed, w);
@@ -281,6 +317,7 @@ void fmm_selector_destroy(fmm_selector_t s) {
     void* bufs[] = {s->w, s->g, s->m, s->v, s->cnt, s->hist};
     for (void* b : bufs)
         if (b) cudaFree(b);
+    if (s->h_hist) cudaFreeHost(s->h_hist);
     delete s;
 }
 
@@ -290,13 +327,16 @@ int fmm_selector_num_params(fmm_selector_t s) { return s ? s->np : -1; }
 fmm_status fmm_selector_features(fmm_selector_t s, const double* xy, int64_t n, double box, float* feat_host) {
     if (!s || !xy || n < 1 || !feat_host || !(box > 0.0)) return FMM_ERR_INVALID_ARG;
     cudaStream_t st = s->stream;
-    if (cudaMemsetAsync(s->cnt, 0, sizeof(uint32_t) * s->ncnt, st) != cudaSuccess ||
+    if (cudaMemsetAsync(s->cnt, 0, sizeof(uint32_t) * kOccFine, st) != cudaSuccess ||
         cudaMemsetAsync(s->hist, 0, sizeof(uint32_t) * kHistLevels * kBins, st) != cudaSuccess)
         return FMM_ERR_CUDA;
     k_occ_count<<<nblk(n, 256), 256, 0, st>>>(reinterpret_cast<const double2*>(xy), n, box, s->cnt);
-    k_occ_hist<<<1024, 256, 0, st>>>(s->cnt, s->ncnt, s->hist);
-    uint32_t h[kHistLevels * kBins];
-    if (cudaMemcpyAsync(h, s->hist, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    uint32_t* level6 = s->cnt + kOccFine;
+    k_occ_tile<5><<<(unsigned)kOccTiles, 256, 0, st>>>(s->cnt, kLevMax, level6, s->hist);
+    k_occ_tile<4><<<4, 256, 0, st>>>(level6, 6, nullptr, s->hist);
+    const uint32_t* h = s->h_hist;
+    if (cudaMemcpyAsync(s->h_hist, s->hist, sizeof(uint32_t) * kHistLevels * kBins, cudaMemcpyDeviceToHost, st) !=
+            cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return FMM_ERR_CUDA;
     for (int k = kLevMin; k <= kLevMax; ++k)

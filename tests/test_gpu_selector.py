@@ -81,3 +81,17 @@ def test_trained_selector_beats_the_fixed_fallback():
     missed = [r for r in rows if r["err_pick"] > 1e-6]
     assert not missed, f"picks that miss 1e-6: {missed}"
     assert sum(r["ms_pick"] for r in rows) < sum(r["ms_fallback"] for r in rows)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 1025, 300000])
+def test_features_of_tiles(sel, n):
+    """Squares on the borders of the counting kernels' 32 x 32 tiles and the corners of the box, one particle to
+    crowds beyond the last bin (2^11): the same counts as the counting oracle, so the same floats."""
+    import torch
+    from oracle import mlp
+    side = 5.0 / 2 ** 11
+    r = np.random.RandomState(n)
+    xy = (np.array([0, 31, 32, 1023, 1024, 2016, 2047])[r.randint(0, 7, (n, 2))] + 0.5) * side
+    xy[0] = [5.0, 0.0]
+    f = sel.features(torch.from_numpy(xy).to("cuda:0"))
+    assert np.array_equal(f, mlp.occupancy_features(xy).astype(np.float32))
