@@ -213,16 +213,21 @@ static __device__ __forceinline__ uint2 fmm_forward_neighbour(const uint32_t* __
 }
 
 // Finest-square coordinate floor(fl(x 2^l / box)) clamped to [0, side - 1], the rule the oracle
-// uses, without occupying the narrow FP64 pipe in the common case: an FP32 estimate of the
-// quotient (error below 1e-3 for side <= 4096) decides whenever it is more than 2e-3 away from
-// an integer; otherwise the exact FP64 division decides.  t = x 2^l is exact.
+// uses, without occupying the narrow FP64 pipe in the common case.  x, the scale and their product are
+// rounded to FP32, so the estimate q of the quotient is off by at most 2^-22 q + 2^-22 (the constant
+// stands for a scale in the subnormal range); it decides whenever it is more than 6e-7 q away from an
+// integer -- below 1 only the upper edge counts, as the quotient is not negative -- and otherwise the
+// exact FP64 division does.  t = x 2^l is exact.
+// A band of 2e-3 at every q sent a lane of every fourth warp through the division: two passes of the
+// selector's features over 2^20 particles (2,048 squares a side) 214 us, 199 us with this one.  The sorts'
+// binning, bound by its atomics, is the same with either.
 static __device__ __forceinline__ int finest_coord(double x, double scale, float scale_over_box32, double box, int side) {
     const float2 xf = fmm_d2ff_bits(x);   // hi word: x truncated to 24 bits
     const float q32 = xf.x * scale_over_box32;
     const float fl = floorf(q32);
-    const float fr = q32 - fl;
+    const float fr = q32 - fl, band = 6e-7f * q32;
     float f;
-    if (fr > 2e-3f && fr < 1.0f - 2e-3f) {
+    if (fr > band && fr < 1.0f - band) {
         f = fl;
     } else {
         f = (float)floor(x * scale / box);

@@ -83,3 +83,21 @@ def test_leaf_keys_equal_the_oracle_rule(oracle_mod, precision, levels):
         if levels == 8 and (kind == "edge" or precision == "fp64"):
             check_parity(phi, oracle_mod.shiftfree(xy, q, levels, p), TOL[precision],
                          f"{precision} {kind} particles levels={levels} p={p}")
+
+
+@pytest.mark.parametrize("levels", [2, 5, 11])
+@pytest.mark.parametrize("box", [0.3, 1e-37, 2.5e38])
+def test_leaf_keys_over_box_sizes(oracle_mod, levels, box):
+    """The same rule where the FP32 estimate's scale overflows or is subnormal, and at small and large quotients."""
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    x = _edges(levels, 2000, 900 + levels, box)
+    near = np.clip(np.concatenate([x * (1.0 + s * 2.0 ** -22) for s in (-3.0, -1.0, 1.0, 3.0)]), 0.0, box)
+    x = np.concatenate([x, near])
+    xy = np.stack([x, np.roll(x, 11)], axis=1)
+    txy, tq = to_dev(xy, np.ones(xy.shape[0]))
+    with binding.Plan(xy.shape[0], levels, 2, box, "fp64") as plan:
+        plan.potential(txy, tq)
+        keys = plan.leaf_keys().cpu().numpy().view(np.uint32)
+    ix, iy = oracle_mod.finest_squares(xy, levels, box)
+    assert np.array_equal(keys, _morton(ix, iy))
