@@ -806,13 +806,22 @@ __global__ void k_split_psi(const double* __restrict__ psi, int64_t nval, double
 
 // psi_m[j] += sum_{o in IL} sum_i K_k[o][i][j] Q_{m+o}[i].  Targets are grouped by
 // the parity of their coordinates: within a parity class the interaction list is the same set of
-// offsets (o_a in [-2 - p_a, 3 - p_a], Chebyshev distance >= 2), so a block takes 32 targets of
-// one class and a group of offsets, and applies each offset's d x d matrix to 32 source columns
-// (a small dense product with the matrix in shared memory).
+// offsets (o_a in [-2 - p_a, 3 - p_a], Chebyshev distance >= 2), so a block takes a tile of targets of
+// one class and a group of offsets, and applies each offset's d x d matrix to the tile's source columns,
+// a small dense product from shared memory.  The next offset's matrix and columns arrive by cp.async
+// beside the current product.
+// What bounds it: FP32 at 4 x 4 sums a thread, where 64 FMAs take 12 wavefronts of shared memory; a thread
+// per node and eight targets took nine loads for eight FMAs.  200,000 charges in 3D, levels 3: 124 -> 40 us
+// alone; 2^20 in 2D, levels 7: 66 -> 20 us.  FP64 (0.82 ms for 80,000 in 3D, levels 3) is bound by its pipe.
+constexpr int kM2LThreads = 128;
+template <int D>
+__host__ __device__ constexpr int m2l_tile() { return D == 2 ? 128 : 32; }   // targets a block
 template <int D, typename T>
-constexpr size_t m2l_smem_bytes() {
-    return ((size_t)nodes_of(D) * nodes_of(D) + (size_t)nodes_of(D) * 33) * sizeof(T);
-}
+__host__ __device__ constexpr int m2l_stride() { return nodes_of(D) + 16 / (int)sizeof(T); }   // of a source column
+template <int D, typename T>
+__host__ __device__ constexpr int m2l_buf() { return nodes_of(D) * nodes_of(D) + m2l_tile<D>() * m2l_stride<D, T>(); }
+template <int D, typename T>
+constexpr size_t m2l_smem_bytes() { return 2 * (size_t)m2l_buf<D, T>() * sizeof(T); }
 
 // All levels in one launch: level k's blocks begin at base[k].
 struct M2LLevels {
@@ -821,13 +830,77 @@ struct M2LLevels {
     int base[kMaxLevels + 2];
 };
 
+template <typename T>
+struct alignas(16) Vec4 {
+    T v[4];
+};
+
+// 16 bytes to shared memory, or 16 zero bytes
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool have) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(have ? 16 : 0) : "memory");
+}
+
+// bits of v (below 2^8) D places apart
+template <int D>
+__device__ __forceinline__ uint32_t spread_bits(uint32_t v) {
+    if constexpr (D == 2) return fmm_spread2(v);
+    v = (v | (v << 8)) & 0x00f00fu;
+    v = (v | (v << 4)) & 0x0c30c3u;
+    return (v | (v << 2)) & 0x249249u;
+}
+
+// sums of targets tg + r NTG (r < R) at nodes 4 jg .. 4 jg + 3 over one offset, added to acc.  FP32: with
+// Kahan's compensation, as a plain running sum over a group's offsets (up to 7 x 64 terms in 3D) would leave
+// about 1e-6 of the far field in rounding.
+template <int D, typename T, int R, int RT>
+__device__ __forceinline__ void m2l_product(const T* __restrict__ sK, const T* __restrict__ sQ, int jg, int tg,
+                                            T (&acc)[RT][4], T (&comp)[RT][4]) {
+    constexpr int d = nodes_of(D), S = m2l_stride<D, T>(), NTG = m2l_tile<D>() / RT;
+    T t[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[r][j] = T(0);
+#pragma unroll 2
+    for (int i = 0; i < d; i += 4) {
+        Vec4<T> kv[4], qv[R];
+#pragma unroll
+        for (int ii = 0; ii < 4; ++ii) kv[ii] = *reinterpret_cast<const Vec4<T>*>(sK + (i + ii) * d + 4 * jg);
+#pragma unroll
+        for (int r = 0; r < R; ++r) qv[r] = *reinterpret_cast<const Vec4<T>*>(sQ + (tg + r * NTG) * S + i);
+#pragma unroll
+        for (int ii = 0; ii < 4; ++ii)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) t[r][j] += kv[ii].v[j] * qv[r].v[ii];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if constexpr (sizeof(T) == 4) {
+                const T y = t[r][j] - comp[r][j];
+                const T sum = acc[r][j] + y;
+                comp[r][j] = (sum - acc[r][j]) - y;
+                acc[r][j] = sum;
+            } else {
+                acc[r][j] += t[r][j];
+            }
+        }
+}
+
 template <int D, typename T>
-__global__ void __launch_bounds__(256) k_m2l(M2LLevels lv, int ngroups) {
-    constexpr int d = nodes_of(D), TT = 32, NT = 256, NTG = NT / d, RT = TT / NTG;
-    constexpr int NOFF = D == 2 ? 27 : 189;
+__global__ void __launch_bounds__(kM2LThreads) k_m2l(M2LLevels lv, int ngroups) {
+    constexpr int d = nodes_of(D), TT = m2l_tile<D>(), S = m2l_stride<D, T>(), JG = d / 4, NTG = kM2LThreads / JG,
+                  RT = TT / NTG;
+    constexpr int NOFF = D == 2 ? 27 : 189, RAW = D == 2 ? 36 : 216;
+    constexpr int PER16 = 16 / (int)sizeof(T), CH = d / PER16, NQ = CH * TT / kM2LThreads;   // 16-byte pieces of a column
+    static_assert(RT == 4 && NQ * kM2LThreads == CH * TT, "whole tiles");
     extern __shared__ __align__(16) unsigned char m2l_smem[];
-    T* s_K = reinterpret_cast<T*>(m2l_smem);                              // [d][d]
-    T(*s_Q)[TT + 1] = reinterpret_cast<T(*)[TT + 1]>(s_K + d * d);        // [d][TT + 1]
+    __shared__ int s_off[NOFF];   // the group's offsets as base-6 digits
+    T* buf = reinterpret_cast<T*>(m2l_smem);
     int k = 2;
     while ((int)blockIdx.x >= lv.base[k + 1]) ++k;
     const T* K = static_cast<const T*>(lv.K[k]);
@@ -841,69 +914,92 @@ __global__ void __launch_bounds__(256) k_m2l(M2LLevels lv, int ngroups) {
     blk /= ngroups;
     const int tile = blk % ntiles, par = blk / ntiles;
     const int p[3] = {par & 1, (par >> 1) & 1, (par >> 2) & 1};
-    const int tid = threadIdx.x, j = tid % d, tg = tid / d;
-    // this group's offsets among the class's NOFF
-    const int per = (NOFF + ngroups - 1) / ngroups, e0 = g * per, e1 = min(NOFF, e0 + per);
-    T acc[RT], comp[RT];
+    const int tid = threadIdx.x, jg = tid % JG, tg = tid / JG;
+    const int per = (NOFF + ngroups - 1) / ngroups, e0 = g * per, cnt = min(NOFF, e0 + per) - e0;
+    auto offset = [&](int raw, int a) { return (a == 0 ? raw : (a == 1 ? raw / 6 : raw / 36)) % 6 - 2 - p[a]; };
+    if (tid < 32) {   // offsets e0 .. e0 + cnt - 1 of the class, x fastest
+        int before = 0;
+        for (int r0 = 0; r0 < RAW; r0 += 32) {
+            const int raw = r0 + tid;
+            int cheb = max(abs(offset(raw, 0)), abs(offset(raw, 1)));
+            if (D == 3) cheb = max(cheb, abs(offset(raw, 2)));
+            const bool valid = raw < RAW && cheb >= 2;
+            const unsigned m = __ballot_sync(0xffffffffu, valid);
+            const int e = before + __popc(m & ((1u << tid) - 1u)) - e0;
+            if (valid && e >= 0 && e < cnt) s_off[e] = raw;
+            before += __popc(m);
+        }
+    }
+    // the targets whose source columns this thread loads pieces of, and the tile's end
+    int tc[NQ][D];
+    const int rows = min(TT, nparent - tile * TT);
 #pragma unroll
-    for (int r = 0; r < RT; ++r) acc[r] = comp[r] = T(0);
-    int e = 0;   // running index of the class's offsets
-    for (int oz = (D == 3 ? -2 - p[2] : 0); oz <= (D == 3 ? 3 - p[2] : 0); ++oz)
-        for (int oy = -2 - p[1]; oy <= 3 - p[1]; ++oy)
-            for (int ox = -2 - p[0]; ox <= 3 - p[0]; ++ox) {
-                const int cheb = max(abs(ox), max(abs(oy), abs(oz)));
-                if (cheb < 2) continue;
-                const int my = e++;
-                if (my < e0 || my >= e1) continue;
-                const int oidx = (ox + 3) + 7 * (oy + 3) + (D == 3 ? 49 * (oz + 3) : 0);
-                __syncthreads();
-                const float4* Ko = reinterpret_cast<const float4*>(K + (size_t)oidx * d * d);
-                for (int x = tid; x < d * d * (int)sizeof(T) / 16; x += NT) reinterpret_cast<float4*>(s_K)[x] = Ko[x];
-                for (int x = tid; x < d * TT; x += NT) {
-                    const int tt = x / d, i = x % d;
-                    const int P = tile * TT + tt;
-                    T v = T(0);
-                    if (P < nparent) {
-                        const int pc[3] = {P % pside, (P / pside) % pside, D == 3 ? P / (pside * pside) : 0};
-                        const int sc[3] = {2 * pc[0] + p[0] + ox, 2 * pc[1] + p[1] + oy, 2 * pc[2] + p[2] + oz};
-                        bool in = sc[0] >= 0 && sc[0] < side && sc[1] >= 0 && sc[1] < side;
-                        if (D == 3) in = in && sc[2] >= 0 && sc[2] < side;
-                        if (in) v = Q[(size_t)morton_enc(D, sc) * d + i];
-                    }
-                    s_Q[i][tt] = v;
-                }
-                __syncthreads();
-                T t[RT];
+    for (int m = 0; m < NQ; ++m) {
+        const int P = tile * TT + (tid + m * kM2LThreads) / CH;
+        tc[m][0] = 2 * (P % pside) + p[0];
+        tc[m][1] = 2 * ((P / pside) % pside) + p[1];
+        if constexpr (D == 3) tc[m][2] = 2 * (P / (pside * pside)) + p[2];   // outside the grid past the last target
+    }
+    __syncthreads();
+    auto stage = [&](int e) {
+        const int raw = s_off[e];
+        int o[D], oidx = 0;
 #pragma unroll
-                for (int r = 0; r < RT; ++r) t[r] = T(0);
-#pragma unroll 8
-                for (int i = 0; i < d; ++i) {
-                    const T kv = s_K[i * d + j];
+        for (int a = D - 1; a >= 0; --a) {
+            o[a] = offset(raw, a);
+            oidx = 7 * oidx + o[a] + 3;
+        }
+        T* sK = buf + (e & 1) * m2l_buf<D, T>();
+        T* sQ = sK + d * d;
+        const T* Ko = K + (size_t)oidx * d * d;
+        for (int x = tid; x < d * d / PER16; x += kM2LThreads) cp_async16(sK + x * PER16, Ko + x * PER16, true);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) t[r] += kv * s_Q[i][tg * RT + r];
-                }
-                // one offset's d-term product is added to the running sum with Kahan's compensation
-                // in FP32: a plain running sum over a group's offsets (up to 21 x 64 terms in 3D)
-                // would leave about 1e-6 of the far field in rounding
+        for (int m = 0; m < NQ; ++m) {
+            const int x = tid + m * kM2LThreads, tt = x / CH, c = x % CH;
+            bool in = tt < rows;
+            uint32_t cell = 0;
 #pragma unroll
-                for (int r = 0; r < RT; ++r) {
-                    if constexpr (sizeof(T) == 4) {
-                        const T y = t[r] - comp[r];
-                        const T sum = acc[r] + y;
-                        comp[r] = (sum - acc[r]) - y;
-                        acc[r] = sum;
-                    } else {
-                        acc[r] += t[r];
-                    }
-                }
+            for (int a = 0; a < D; ++a) {
+                const int v = tc[m][a] + o[a];
+                in = in && v >= 0 && v < side;
+                cell |= spread_bits<D>((uint32_t)v & 0xffu) << a;
             }
+            cp_async16(sQ + tt * S + c * PER16, in ? Q + (size_t)cell * d + c * PER16 : Q, in);
+        }
+    };
+    T acc[RT][4], comp[RT][4];
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[r][j] = comp[r][j] = T(0);
+    stage(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int e = 0; e < cnt; ++e) {
+        if (e + 1 < cnt) stage(e + 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const T* sK = buf + (e & 1) * m2l_buf<D, T>();
+        // level 2 has few targets of a class: one row of sums holds them
+        if (rows <= NTG) m2l_product<D, T, 1, RT>(sK, sK + d * d, jg, tg, acc, comp);
+        else m2l_product<D, T, RT, RT>(sK, sK + d * d, jg, tg, acc, comp);
+        __syncthreads();
+    }
+    // out by way of shared memory, so that a warp's atomics fall on consecutive nodes
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
-        const int P = tile * TT + tg * RT + r;
-        if (P >= nparent) continue;
-        const int pc[3] = {P % pside, (P / pside) % pside, D == 3 ? P / (pside * pside) : 0};
-        const int tc[3] = {2 * pc[0] + p[0], 2 * pc[1] + p[1], 2 * pc[2] + p[2]};
-        atomicAdd(psi + (size_t)morton_enc(D, tc) * d + j, (double)acc[r]);
+        Vec4<T> v;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v.v[j] = acc[r][j];
+        *reinterpret_cast<Vec4<T>*>(buf + (tg + r * NTG) * d + 4 * jg) = v;
+    }
+    __syncthreads();
+    for (int x = tid; x < rows * d; x += kM2LThreads) {
+        const int P = tile * TT + x / d;
+        uint32_t cell = spread_bits<D>((uint32_t)(2 * (P % pside) + p[0])) |
+                        spread_bits<D>((uint32_t)(2 * ((P / pside) % pside) + p[1])) << 1;
+        if constexpr (D == 3) cell |= spread_bits<D>((uint32_t)(2 * (P / (pside * pside)) + p[2])) << 2;
+        atomicAdd(psi + (size_t)cell * d + x % d, (double)buf[x]);
     }
 }
 
@@ -1226,10 +1322,10 @@ int enqueue_nodes(fmm_lag_plan_s* pl, const PosReader<T>& rd, int64_t n, unsigne
             lv.Q.p[k] = pl->node[k];
             lv.psi.p[k] = pl->pot[k];
             lv.base[k] = blocks;
-            blocks += (int)(((ipow(1 << (k - 1), D) + 31) / 32) * (1 << D) * ngroups);
+            blocks += (int)(((ipow(1 << (k - 1), D) + m2l_tile<D>() - 1) / m2l_tile<D>()) * (1 << D) * ngroups);
         }
         lv.base[L + 1] = blocks;
-        k_m2l<D, T><<<(unsigned)blocks, 256, m2l_smem_bytes<D, T>(), st>>>(lv, ngroups);
+        k_m2l<D, T><<<(unsigned)blocks, kM2LThreads, m2l_smem_bytes<D, T>(), st>>>(lv, ngroups);
         ++launches;
     }
     cudaEventRecord(pl->ev[3], st);
@@ -1443,9 +1539,11 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     }
     if (rc == FMM_OK) rc = cuda_status(cudaMemset(pl->status, 0, sizeof(unsigned)));
     if (rc == FMM_OK) rc = cuda_status(cudaMallocHost(reinterpret_cast<void**>(&pl->h_status), sizeof(unsigned)));
-    if (rc == FMM_OK && dim == 3 && f64 && !lit)
-        rc = cuda_status(cudaFuncSetAttribute(k_m2l<3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)m2l_smem_bytes<3, double>()));
+    if (rc == FMM_OK && dim == 3 && !lit)
+        rc = cuda_status(f64 ? cudaFuncSetAttribute(k_m2l<3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)m2l_smem_bytes<3, double>())
+                             : cudaFuncSetAttribute(k_m2l<3, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)m2l_smem_bytes<3, float>()));
     if (rc == FMM_OK && !lit && levels >= 2) {
         const std::vector<double> K = build_operators(dim, levels, box);
         if (f64) {
