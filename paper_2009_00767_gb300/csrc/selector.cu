@@ -28,12 +28,12 @@ constexpr int kIn = kFeat + 2;                   // + candidate levels / 12, p /
 constexpr int kOut = 2;
 constexpr size_t kOccFine = (size_t)1 << (2 * kLevMax);        // squares of the finest level counted
 constexpr size_t kOccTiles = (size_t)1 << (2 * (kLevMax - 5));   // its tiles of 32 x 32: level 6
-static_assert(kLevMin == 3 && kLevMax == 11, "k_occ_tile<5> takes levels 11..7, k_occ_tile<4> levels 6..3");
+static_assert(kLevMin == 3 && kLevMax == 11 && kHistLevels * kBins <= 256, "k_occ_hist: occ_tile<5> levels 11..7, occ_tile<4> levels 6..3");
 
 // ---------------------------------------------------------------- occupancy statistics
 // One count per particle, in its square of the finest level; the coarser levels' populations are sums of
-// four.  What bounds it: the atomics in L2, so a ninth of them.  2^20 particles: a call of fmm_selector_features
-// and one of fmm_select take 213 us together, 1087 us with an atomic per particle and level.
+// four.  What bounds it: the atomics in L2, so a ninth of them.  2^20 particles: 22 us; a call of
+// fmm_selector_features and one of fmm_select take 141 us together, 1087 us with an atomic per particle and level.
 __global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double box, uint32_t* __restrict__ cnt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -45,60 +45,92 @@ __global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double bo
     atomicAdd(&cnt[((size_t)iy << kLevMax) + ix], 1u);
 }
 
-__device__ __forceinline__ int occ_bin(uint32_t c) { return min(kBins - 1, 31 - __clz(c + 1u)); }   // floor(log2(c + 1))
-
-// Occupancies of a 32 x 32 tile of level-k squares (cnt, row-major) and of the kLevels - 1 levels above them:
-// histograms to hist and, with five levels, the tile's own population, that of a square of level k - 5, to
-// `up`.  A 256-thread block, a thread per 2 x 2 squares; lanes vote on each bin, so that a level costs one
-// shared atomic per warp and bin.
+// Occupancies of a 32 x 32 tile of level-k squares (cnt, row-major) and of kLevels - 1 <= 5 levels above them,
+// added to the block's histograms h.  A warp per tile and 4 x 8 squares a lane, so that the first three levels
+// are sums within a lane and the others shuffles, without a barrier.  A lane counts the bins of a level in the
+// 5-bit fields of one word (at most 16 squares at a time); one warp reduction per bin then adds three levels at
+// once, as fields of 11, 9 and 7 bits.  Returns the tile's population.
+__device__ __forceinline__ unsigned long long occ_field(uint32_t c) {
+    return 1ull << (5 * min(kBins - 1, 31 - __clz(c + 1u)));   // bin floor(log2(c + 1))
+}
 template <int kLevels>
-__global__ void __launch_bounds__(256) k_occ_tile(const uint32_t* __restrict__ cnt, int k, uint32_t* __restrict__ up,
-                                                  uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[kLevels * kBins];
-    __shared__ uint32_t pop[256];
-    const int t = threadIdx.x, lane = t & 31;
-    for (int i = t; i < kLevels * kBins; i += 256) h[i] = 0u;
-    __syncthreads();
-    const int tiles = 1 << (k - 5);
-    const int tx = blockIdx.x % tiles, ty = blockIdx.x / tiles;
-    const int x = t & 15, y = t >> 4;
-    const size_t at = ((size_t)(32 * ty + 2 * y) << k) + 32 * tx + 2 * x;
-    const uint2 a = *reinterpret_cast<const uint2*>(cnt + at);
-    const uint2 b = *reinterpret_cast<const uint2*>(cnt + at + ((size_t)1 << k));
-    const int ba = occ_bin(a.x), bb = occ_bin(a.y), bc = occ_bin(b.x), bd = occ_bin(b.y);
+__device__ __forceinline__ uint32_t occ_tile(const uint32_t* cnt, int k, int tile, int lane, uint32_t* h) {
+    const int tiles = 1 << (k - 5), tx = tile % tiles, ty = tile / tiles;
+    const uint32_t* at = cnt + ((size_t)(32 * ty + 8 * (lane >> 3)) << k) + 32 * tx + 4 * (lane & 7);
+    uint4 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = __ldcg(reinterpret_cast<const uint4*>(at + ((size_t)r << k)));
+    unsigned long long f[2] = {0ull, 0ull}, g = 0ull, e = 0ull;
+    uint32_t q[2] = {0u, 0u};   // the lane's two 4 x 4 squares
+#pragma unroll
+    for (int r = 0; r < 8; r += 2) {
+        const uint4 a = v[r], b = v[r + 1];
+        f[r / 4] += occ_field(a.x) + occ_field(a.y) + occ_field(a.z) + occ_field(a.w) + occ_field(b.x) + occ_field(b.y) +
+                    occ_field(b.z) + occ_field(b.w);
+        const uint32_t l = a.x + a.y + b.x + b.y, m = a.z + a.w + b.z + b.w;
+        g += occ_field(l) + occ_field(m);
+        q[r / 4] += l + m;
+    }
+    e = occ_field(q[0]) + occ_field(q[1]);
+    uint32_t s = q[0] + q[1];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);   // 8 x 8, in every second lane
+    unsigned long long d = (lane & 1) ? 0ull : occ_field(s), c = 0ull, b = 0ull;
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 8);   // 16 x 16
+    if (kLevels > 4) c = (lane & 11) ? 0ull : occ_field(s);
+    s += __shfl_xor_sync(0xffffffffu, s, 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);   // the tile
+    if (kLevels > 5) b = lane ? 0ull : occ_field(s);
+    uint32_t mine = 0u, mine2 = 0u;   // lane i: bin i of the levels
 #pragma unroll
     for (int i = 0; i < kBins; ++i) {
-        const int c = __popc(__ballot_sync(0xffffffffu, ba == i)) + __popc(__ballot_sync(0xffffffffu, bb == i)) +
-                      __popc(__ballot_sync(0xffffffffu, bc == i)) + __popc(__ballot_sync(0xffffffffu, bd == i));
-        if (lane == 0 && c) atomicAdd(&h[i], (uint32_t)c);
-    }
-    pop[t] = a.x + a.y + b.x + b.y;
-    __syncthreads();
-    // 16 x 16 squares of level k - 1, then a quarter of them a level
-#pragma unroll
-    for (int l = 1; l < kLevels; ++l) {
-        const int w = 32 >> l;   // squares a side at this level
-        const bool on = t < w * w;
-        const int bin = on ? occ_bin(pop[t]) : -1;
-        if ((t & ~31) < w * w)
-#pragma unroll
-            for (int i = 0; i < kBins; ++i) {
-                const int c = __popc(__ballot_sync(0xffffffffu, bin == i));
-                if (lane == 0 && c) atomicAdd(&h[l * kBins + i], (uint32_t)c);
-            }
-        const int hw = w / 2;
-        uint32_t v = 0;
-        if (t < hw * hw) {
-            const int o = 2 * (t / hw) * w + 2 * (t % hw);
-            v = pop[o] + pop[o + 1] + pop[o + w] + pop[o + w + 1];
+        auto field = [&](unsigned long long x) { return (uint32_t)(x >> (5 * i)) & 31u; };
+        const uint32_t u = __reduce_add_sync(0xffffffffu, field(f[0]) + field(f[1]) | field(g) << 11 | field(e) << 20);
+        const uint32_t w = __reduce_add_sync(0xffffffffu, field(d) | field(c) << 11 | field(b) << 20);
+        if (lane == i) {
+            mine = u;
+            mine2 = w;
         }
-        __syncthreads();
-        if (t < hw * hw) pop[t] = v;
-        __syncthreads();
     }
-    if (up && t == 0) up[blockIdx.x] = pop[0];
-    for (int i = t; i < kLevels * kBins; i += 256)
-        if (h[i]) atomicAdd(&hist[(k - i / kBins - kLevMin) * kBins + i % kBins], h[i]);
+    if (lane < kBins) {
+        uint32_t* hk = h + (k - kLevMin) * kBins + lane;
+        atomicAdd(hk, mine & 2047u);
+        atomicAdd(hk - kBins, mine >> 11 & 511u);
+        atomicAdd(hk - 2 * kBins, mine >> 20);
+        atomicAdd(hk - 3 * kBins, mine2 & 2047u);
+        if (kLevels > 4) atomicAdd(hk - 4 * kBins, mine2 >> 11 & 511u);
+        if (kLevels > 5) atomicAdd(hk - 5 * kBins, mine2 >> 20);
+    }
+    return s;
+}
+
+// All histograms from the finest level's populations, a warp per tile; the block that finishes last takes
+// levels 6..3 from the tiles' populations (`coarse`).  hist and done start at zero.
+// What bounds it: 16 MB from L2 and the bins' reductions.  12 us for 2^22 squares against 22 + 5 us for a block per
+// tile that voted on each bin with ballots, a barrier or two per level, and a launch for levels 6..3.
+constexpr int kOccWarps = 8;
+__global__ void __launch_bounds__(kOccWarps * 32) k_occ_hist(const uint32_t* cnt, uint32_t* coarse, uint32_t* hist,
+                                                             uint32_t* done) {
+    __shared__ uint32_t h[kHistLevels * kBins];
+    __shared__ bool last;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t < kHistLevels * kBins) h[t] = 0u;
+    __syncthreads();
+    const int tile = blockIdx.x * kOccWarps + warp;
+    const uint32_t pop = occ_tile<5>(cnt, kLevMax, tile, lane, h);
+    if (lane == 0) coarse[tile] = pop;
+    __threadfence();
+    __syncthreads();
+    if (t < kHistLevels * kBins && h[t]) atomicAdd(&hist[t], h[t]);
+    if (t == 0) last = atomicAdd(done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (t < kHistLevels * kBins) h[t] = 0u;
+    __syncthreads();
+    if (warp < 4) occ_tile<4>(coarse, 6, warp, lane, h);
+    __syncthreads();
+    if (t < kHistLevels * kBins && h[t]) atomicAdd(&hist[t], h[t]);
 }
 
 // ---------------------------------------------------------------- dense layers
@@ -111,6 +143,50 @@ __global__ void k_dense_fwd(const float* __restrict__ X, const float* __restrict
     float acc = b[o];
     for (int i = 0; i < in; ++i) acc = fmaf(X[(size_t)r * in + i], W[(size_t)i * out + o], acc);
     Y[e] = (relu && acc < 0.f) ? 0.f : acc;
+}
+
+// The network on one system's candidates, straight from its histograms: a block per candidate row, a thread
+// per unit, the same sums in the same order as k_dense_fwd.  Row r is (levels l_first + r / kCandP,
+// p = 8 + 4 (r % kCandP)).
+// What bounds it: latency.  The parameters come to shared memory at once where they fit (kStage; 45 kB at 64
+// units): 11.2 us against 20 us for the sums' own loads from L2, and three launches with copies either side and
+// a wait for the features before them.
+constexpr int kCandP = 6;   // p = 8, 12, .., 28
+constexpr int kStageThreads = 256;
+template <bool kStage>
+__global__ void __launch_bounds__(kStageThreads) k_mlp_candidates(const uint32_t* __restrict__ hist, float log_n, int l_first,
+                                 const float* __restrict__ w, int np, int H, float* __restrict__ y) {
+    extern __shared__ float act[];
+    float *x = act, *h1 = act + kIn, *h2 = h1 + H, *ws = h2 + H;
+    const int r = blockIdx.x;
+    if constexpr (kStage) {
+#pragma unroll 16
+        for (int i = threadIdx.x; i < np; i += blockDim.x) ws[i] = w[i];
+    }
+    for (int i = threadIdx.x; i < kIn; i += blockDim.x) {
+        const int lev = kLevMin + i / kBins;
+        x[i] = i < kFeat - 1 ? (float)hist[i] / (float)(1 << (2 * lev))   // counts up to 2^22: exact
+               : i == kFeat - 1 ? log_n : i == kFeat ? (float)(l_first + r / kCandP) / 12.f : (float)(8 + 4 * (r % kCandP)) / 32.f;
+    }
+    __syncthreads();
+    auto unit = [&](const float* in, int nin, const float* W, const float* b, int out, int o) {
+        float acc = b[o];
+#pragma unroll 16
+        for (int i = 0; i < nin; ++i) acc = fmaf(in[i], W[(size_t)i * out + o], acc);
+        return acc;
+    };
+    const float *W1 = kStage ? ws : w, *b1 = W1 + kIn * H, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H, *b3 = W3 + H * kOut;
+    for (int o = threadIdx.x; o < H; o += blockDim.x) {
+        const float a = unit(x, kIn, W1, b1, H, o);
+        h1[o] = a < 0.f ? 0.f : a;
+    }
+    __syncthreads();
+    for (int o = threadIdx.x; o < H; o += blockDim.x) {
+        const float a = unit(h1, H, W2, b2, H, o);
+        h2[o] = a < 0.f ? 0.f : a;
+    }
+    __syncthreads();
+    if (threadIdx.x < kOut) y[r * kOut + threadIdx.x] = unit(h2, H, W3, b3, kOut, threadIdx.x);
 }
 
 // dX[r][i] = (sum_o dY[r][o] W[i][o]) * (Xact[r][i] > 0), the mask of the ReLU that produced X
@@ -180,8 +256,9 @@ struct fmm_selector_s {
     int cap;
     float *x, *h1, *h2, *y, *t, *dy, *dh2, *dh1, *lrow;
     uint32_t* cnt;                   // populations of level 11, then of level 6
-    uint32_t* hist;
-    uint32_t* h_hist;                // pinned
+    uint32_t* hist;                  // the histograms, then k_occ_hist's count of finished blocks
+    uint32_t* h_hist;                // pinned: the histograms
+    float *cand, *h_y;               // the network's outputs for fmm_select's candidates, and pinned
 };
 
 namespace {
@@ -266,10 +343,21 @@ void init_weights(const fmm_selector_s* s, uint64_t seed, std::vector<float>& w)
     fill(offW3(s), s->hidden, s->hidden * kOut);
 }
 
-void candidate_row(const float* feat, int levels, int p, float* row) {
-    memcpy(row, feat, sizeof(float) * kFeat);
-    row[kFeat] = (float)levels / 12.f;
-    row[kFeat + 1] = (float)p / 32.f;
+constexpr size_t kHistBytes = sizeof(uint32_t) * kHistLevels * kBins;
+constexpr int kMaxCand = 5 * kCandP;   // fmm_select: five depths
+
+float log_feature(int64_t n) { return (float)(std::log2((double)n) / 22.0); }
+
+// the histograms of xy, into hist
+bool enqueue_occupancies(fmm_selector_s* s, const double* xy, int64_t n, double box) {
+    cudaStream_t st = s->stream;
+    if (cudaMemsetAsync(s->cnt, 0, sizeof(uint32_t) * kOccFine, st) != cudaSuccess ||
+        cudaMemsetAsync(s->hist, 0, kHistBytes + sizeof(uint32_t), st) != cudaSuccess)
+        return false;
+    k_occ_count<<<nblk(n, 256), 256, 0, st>>>(reinterpret_cast<const double2*>(xy), n, box, s->cnt);
+    k_occ_hist<<<(unsigned)(kOccTiles / kOccWarps), kOccWarps * 32, 0, st>>>(s->cnt, s->cnt + kOccFine, s->hist,
+                                                                             s->hist + kHistLevels * kBins);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 }  // namespace
@@ -296,8 +384,10 @@ fmm_status fmm_selector_create(fmm_selector_t* out, int hidden, uint64_t seed, v
               cudaMalloc(&s->m, sizeof(float) * s->np) == cudaSuccess &&
               cudaMalloc(&s->v, sizeof(float) * s->np) == cudaSuccess &&
               cudaMalloc(&s->cnt, sizeof(uint32_t) * (kOccFine + kOccTiles)) == cudaSuccess &&
-              cudaMallocHost(&s->h_hist, sizeof(uint32_t) * kHistLevels * kBins) == cudaSuccess &&
-              cudaMalloc(&s->hist, sizeof(uint32_t) * kHistLevels * kBins) == cudaSuccess;
+              cudaMallocHost(&s->h_hist, kHistBytes) == cudaSuccess &&
+              cudaMallocHost(&s->h_y, sizeof(float) * kMaxCand * kOut) == cudaSuccess &&
+              cudaMalloc(&s->cand, sizeof(float) * kMaxCand * kOut) == cudaSuccess &&
+              cudaMalloc(&s->hist, kHistBytes + sizeof(uint32_t)) == cudaSuccess;
     std::vector<float> w;
     init_weights(s, seed, w);
     ok = ok && cudaMemcpy(s->w, w.data(), sizeof(float) * s->np, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -314,10 +404,11 @@ fmm_status fmm_selector_create(fmm_selector_t* out, int hidden, uint64_t seed, v
 void fmm_selector_destroy(fmm_selector_t s) {
     if (!s) return;
     sel_free_acts(s);
-    void* bufs[] = {s->w, s->g, s->m, s->v, s->cnt, s->hist};
+    void* bufs[] = {s->w, s->g, s->m, s->v, s->cnt, s->hist, s->cand};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (s->h_hist) cudaFreeHost(s->h_hist);
+    if (s->h_y) cudaFreeHost(s->h_y);
     delete s;
 }
 
@@ -326,23 +417,15 @@ int fmm_selector_num_params(fmm_selector_t s) { return s ? s->np : -1; }
 // Features of the system xy (device, [n][2]) into feat_host[kFeat]; waits for the stream.
 fmm_status fmm_selector_features(fmm_selector_t s, const double* xy, int64_t n, double box, float* feat_host) {
     if (!s || !xy || n < 1 || !feat_host || !(box > 0.0)) return FMM_ERR_INVALID_ARG;
-    cudaStream_t st = s->stream;
-    if (cudaMemsetAsync(s->cnt, 0, sizeof(uint32_t) * kOccFine, st) != cudaSuccess ||
-        cudaMemsetAsync(s->hist, 0, sizeof(uint32_t) * kHistLevels * kBins, st) != cudaSuccess)
+    if (!enqueue_occupancies(s, xy, n, box) ||
+        cudaMemcpyAsync(s->h_hist, s->hist, kHistBytes, cudaMemcpyDeviceToHost, s->stream) != cudaSuccess ||
+        cudaStreamSynchronize(s->stream) != cudaSuccess)
         return FMM_ERR_CUDA;
-    k_occ_count<<<nblk(n, 256), 256, 0, st>>>(reinterpret_cast<const double2*>(xy), n, box, s->cnt);
-    uint32_t* level6 = s->cnt + kOccFine;
-    k_occ_tile<5><<<(unsigned)kOccTiles, 256, 0, st>>>(s->cnt, kLevMax, level6, s->hist);
-    k_occ_tile<4><<<4, 256, 0, st>>>(level6, 6, nullptr, s->hist);
     const uint32_t* h = s->h_hist;
-    if (cudaMemcpyAsync(s->h_hist, s->hist, sizeof(uint32_t) * kHistLevels * kBins, cudaMemcpyDeviceToHost, st) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return FMM_ERR_CUDA;
     for (int k = kLevMin; k <= kLevMax; ++k)
         for (int b = 0; b < kBins; ++b)
             feat_host[(k - kLevMin) * kBins + b] = (float)((double)h[(k - kLevMin) * kBins + b] / (double)(1ull << (2 * k)));
-    feat_host[kFeat - 1] = (float)(std::log2((double)n) / 22.0);
+    feat_host[kFeat - 1] = log_feature(n);
     return FMM_OK;
 }
 
@@ -472,23 +555,27 @@ fmm_status fmm_selector_load(fmm_selector_t s, const char* path) {
 fmm_status fmm_select(fmm_selector_t s, const double* xy, int64_t n, double box, double target_err,
                       double margin_decades, int* levels_out, int* p_out, int* used_fallback) {
     if (!s || !xy || n < 1 || !(target_err > 0.0) || !levels_out || !p_out) return FMM_ERR_INVALID_ARG;
-    float feat[kFeat];
-    fmm_status st = fmm_selector_features(s, xy, n, box, feat);
-    if (st != FMM_OK) return st;
+    if (!(box > 0.0)) return FMM_ERR_INVALID_ARG;
     const int l0 = (int)std::lround(std::log((double)n / 16.0) / std::log(4.0));
-    std::vector<int> cl, cp;
-    for (int l = l0 - 2; l <= l0 + 2; ++l) {
-        if (l < 2 || l > 11) continue;
-        for (int p = 8; p <= 28; p += 4) {
-            cl.push_back(l);
-            cp.push_back(p);
-        }
+    const int l_first = l0 - 2 < 2 ? 2 : l0 - 2, l_last = l0 + 2 > 11 ? 11 : l0 + 2;
+    const int rows = l_last >= l_first ? kCandP * (l_last - l_first + 1) : 0;
+    if (!enqueue_occupancies(s, xy, n, box)) return FMM_ERR_CUDA;
+    if (rows > 0) {
+        const int H = s->hidden;
+        const size_t acts = sizeof(float) * (kIn + 2 * H), all = acts + sizeof(float) * s->np;
+        if (all <= 48 * 1024)
+            k_mlp_candidates<true><<<rows, kStageThreads, all, s->stream>>>(s->hist, log_feature(n), l_first, s->w, s->np, H,
+                                                                            s->cand);
+        else
+            k_mlp_candidates<false><<<rows, kStageThreads, acts, s->stream>>>(s->hist, log_feature(n), l_first, s->w, s->np,
+                                                                              H, s->cand);
+        if (cudaGetLastError() != cudaSuccess || cudaMemcpyAsync(s->h_y, s->cand, sizeof(float) * rows * kOut,
+                                                                 cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+            return FMM_ERR_CUDA;
     }
-    const int rows = (int)cl.size();
-    std::vector<float> x((size_t)rows * kIn), y((size_t)rows * kOut);
-    for (int r = 0; r < rows; ++r) candidate_row(feat, cl[r], cp[r], &x[(size_t)r * kIn]);
-    st = fmm_selector_predict(s, x.data(), rows, y.data());
-    if (st != FMM_OK) return st;
+    if (cudaStreamSynchronize(s->stream) != cudaSuccess) return FMM_ERR_CUDA;
+    if (rows == 0) return FMM_ERR_INVALID_ARG;   // too few particles for any candidate
+    const float* y = s->h_y;
     const double lim = (std::log10(target_err) - margin_decades) / 8.0;
     int best = -1;
     for (int r = 0; r < rows; ++r)
@@ -498,8 +585,8 @@ fmm_status fmm_select(fmm_selector_t s, const double* xy, int64_t n, double box,
         *p_out = 20;
         if (used_fallback) *used_fallback = 1;
     } else {
-        *levels_out = cl[best];
-        *p_out = cp[best];
+        *levels_out = l_first + best / kCandP;
+        *p_out = 8 + 4 * (best % kCandP);
         if (used_fallback) *used_fallback = 0;
     }
     return FMM_OK;

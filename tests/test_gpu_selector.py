@@ -95,3 +95,29 @@ def test_features_of_tiles(sel, n):
     xy[0] = [5.0, 0.0]
     f = sel.features(torch.from_numpy(xy).to("cuda:0"))
     assert np.array_equal(f, mlp.occupancy_features(xy).astype(np.float32))
+
+
+@pytest.mark.parametrize("hidden", [1, 33, 64, 300])
+@pytest.mark.parametrize("n", [9, 40, 5000, 300000])
+def test_selection_is_the_networks_best_candidate(hidden, n):
+    """fmm_select against the same rule over features() and predict(): the same floats, so the same pick."""
+    import torch
+    from paper_2009_00767_gb300 import binding
+    s = binding.Selector(hidden=hidden, seed=7)
+    xy = torch.from_numpy(5.0 * np.random.RandomState(n).rand(n, 2)).to("cuda:0")
+    f = s.features(xy)
+    l0 = int(np.floor(np.log(n / 16.0) / np.log(4.0) + 0.5))
+    cand = [(l, p) for l in range(l0 - 2, l0 + 3) if 2 <= l <= 11 for p in range(8, 29, 4)]
+    x = np.stack([np.concatenate([f, np.float32([l]) / np.float32(12), np.float32([p]) / np.float32(32)]) for l, p in cand])
+    y = s.predict(x)
+    for target in (1e-2, 1.0, 1e3):
+        ok = np.nonzero(y[:, 0].astype(np.float64) <= (np.log10(target) - 0.3) / 8.0)[0]
+        want = cand[ok[np.argmin(y[ok, 1])]] + (False,) if len(ok) else (8, 20, True)
+        assert s.select(xy, target_err=target) == want
+    s.close()
+
+
+def test_selection_needs_a_candidate(sel):
+    import torch
+    with pytest.raises(Exception):
+        sel.select(torch.full((7, 2), 1.0, dtype=torch.float64, device="cuda:0"))
