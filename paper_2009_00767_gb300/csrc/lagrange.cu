@@ -4,7 +4,7 @@
 // Data layout in device memory:
 //   * the charges sorted by finest cell in Morton order, so that the charges of any cell at any
 //     level are one contiguous range: FP32 forms keep (x, y, z, q) as a float4 "hi" and the
-//     residues x - hi as a float4 "lo"; FP64 forms keep (x, y, z, q) as a Pos64;
+//     residues x - hi and the input index as a float4 "lo"; FP64 forms keep (x, y, z, q) as a Pos64;
 //   * per level k, the cells in Morton order with d = 4^D node values each (node index
 //     i + 4j + 16k): node charges Q_k and node potentials psi_k (node forms; psi_k in FP64), or
 //     the vectors v_k and dual vectors u_k (literal form);
@@ -110,7 +110,7 @@ struct fmm_lag_plan_s {
     int* start = nullptr;          // [nleaf + 1]
     int* chunk_start = nullptr;    // [nleaf + 1]
     int* wchunk_start = nullptr;   // [nleaf + 1] near-field warp chunks
-    int* order = nullptr;          // [n_max] sorted -> input index
+    int* order = nullptr;          // [n_max] sorted -> input index, FP64 forms (FP32: lo.w)
     Scan3* scan = nullptr;  // per tile of the scan
     float4* hi = nullptr;          // FP32 forms
     float4* lo = nullptr;
@@ -134,6 +134,7 @@ struct fmm_lag_plan_s {
     uint64_t bytes = 0;
     int launches = 0;
     int grid_particles = 0;
+    int sms = 0;
     cudaStream_t last_st = nullptr;   // the stream of the last call, for comparison only
     bool serial = false;   // every kernel in turn on the plan's stream (per-kernel timing)
     int grid_p2p = 0;      // resident blocks of the FP64 near-field kernel, all SMs
@@ -144,14 +145,10 @@ namespace {
 
 // ------------------------------------------------------------------------------ binning
 
-// Finest cell per charge with the FP64 floor/clamp rule (finest_coord), its Morton key and its rank within
-// the cell (atomic), plus the input checks.
+// Finest cell of charge i with the FP64 floor/clamp rule (finest_coord): its Morton key; plus the input checks.
 template <int D>
-__global__ void k_bin(const double* __restrict__ pos, const double* __restrict__ q, int64_t n, int L,
-                      double box, float side_over_box, uint32_t* __restrict__ key, uint32_t* __restrict__ rank,
-                      int* __restrict__ count, unsigned* __restrict__ status) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+__device__ __forceinline__ uint32_t bin_key(const double* __restrict__ pos, const double* __restrict__ q, int64_t i, int L,
+                                            double box, float side_over_box, unsigned* __restrict__ status) {
     const int side = 1 << L;
     const long long bb = __double_as_longlong(box);
     int c[3] = {0, 0, 0};
@@ -167,9 +164,51 @@ __global__ void k_bin(const double* __restrict__ pos, const double* __restrict__
         }
     }
     if (bad) atomicOr(status, bad);
-    const uint32_t k = morton_enc(D, c);
+    return morton_enc(D, c);
+}
+
+// Every charge's key and its rank within the cell (atomic).
+template <int D>
+__global__ void k_bin(const double* __restrict__ pos, const double* __restrict__ q, int64_t n, int L,
+                      double box, float side_over_box, uint32_t* __restrict__ key, uint32_t* __restrict__ rank,
+                      int* __restrict__ count, unsigned* __restrict__ status) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t k = bin_key<D>(pos, q, i, L, box, side_over_box, status);
     key[i] = k;
     rank[i] = (uint32_t)atomicAdd(count + k, 1);
+}
+
+// The same with few cells for the charges: a block ranks its share in shared memory and takes each cell's
+// places at once.
+// What bounds k_bin there: 512 populations are 16 cache lines, whose atomics queue up.
+constexpr int kBinFewCells = 4096, kBinFewThreads = 1024;
+// With fewer charges a block meets most cells once and saves nothing.  The whole sort, k_bin against k_bin_few:
+// 512 cells (3D) 20,000 charges 31.4 and 32.2 us, 40,000 36.2 and 32.5, 160,000 52.9 and 38.8; 4,096 cells
+// 60,000 35.7 and 37.3, 262,144 44.7 and 41.3, 2^20 80.3 and 62.0; 64 cells 5,000 29.3 and 30.4, 9,728 31.0 and
+// 30.1.
+inline bool bin_few(int64_t nleaf, int64_t n) { return nleaf <= kBinFewCells && n >= 64 * nleaf && n >= 8192; }
+
+template <int D>
+__global__ void __launch_bounds__(kBinFewThreads)
+k_bin_few(const double* __restrict__ pos, const double* __restrict__ q, int64_t n, int L, double box, float side_over_box,
+          uint32_t* __restrict__ key, uint32_t* __restrict__ rank, int* __restrict__ count, int nleaf,
+          unsigned* __restrict__ status) {
+    __shared__ int cells[kBinFewCells];
+    for (int c = threadIdx.x; c < nleaf; c += kBinFewThreads) cells[c] = 0;
+    __syncthreads();
+    const int64_t share = (n + gridDim.x - 1) / gridDim.x, i1 = min(n, (blockIdx.x + 1) * share);
+    const int64_t i0 = blockIdx.x * share + threadIdx.x;
+    for (int64_t i = i0; i < i1; i += kBinFewThreads) {
+        const uint32_t k = bin_key<D>(pos, q, i, L, box, side_over_box, status);
+        key[i] = k;
+        rank[i] = (uint32_t)atomicAdd(cells + k, 1);
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < nleaf; c += kBinFewThreads)
+        if (cells[c]) cells[c] = atomicAdd(count + c, cells[c]);
+    __syncthreads();
+    for (int64_t i = i0; i < i1; i += kBinFewThreads) rank[i] += (uint32_t)cells[key[i]];
 }
 
 // Exclusive scans of the populations and of the chunk counts (chunks of kChunk, and of wchunk for the near
@@ -233,24 +272,25 @@ __global__ void __launch_bounds__(kScanTile) k_scan(const int* __restrict__ coun
     }
 }
 
+// Charges into sorted order.  FP32 forms: the input index rides in lo.w, so that a charge is two scattered
+// 16-byte writes; the sorted keys are written by k_p2m, whose warps know their cell.
+// 2^20 charges in 2D: the call 406 -> 385 us against four scattered writes, input index and key among them.
 template <int D, bool k64>
 __global__ void k_scatter(const double* __restrict__ pos, const double* __restrict__ q, int64_t n,
                           const uint32_t* __restrict__ key, const uint32_t* __restrict__ rank,
-                          const int* __restrict__ start, uint32_t* __restrict__ skey, int* __restrict__ order,
-                          float4* __restrict__ hi, float4* __restrict__ lo, Pos64* __restrict__ p64) {
+                          const int* __restrict__ start, int* __restrict__ order, float4* __restrict__ hi,
+                          float4* __restrict__ lo, Pos64* __restrict__ p64) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t k = key[i];
-    const int64_t s = (int64_t)start[k] + rank[i];
+    const int64_t s = (int64_t)start[key[i]] + rank[i];
     const double x = pos[i * D], y = pos[i * D + 1], z = D == 3 ? pos[i * D + 2] : 0.0;
-    skey[s] = k;
-    order[s] = (int)i;
     if constexpr (k64) {
+        order[s] = (int)i;
         p64[s] = Pos64{x, y, z, q[i]};
     } else {
         const float hx = (float)x, hy = (float)y, hz = (float)z;
         hi[s] = make_float4(hx, hy, hz, (float)q[i]);
-        lo[s] = make_float4((float)(x - (double)hx), (float)(y - (double)hy), (float)(z - (double)hz), 0.f);
+        lo[s] = make_float4((float)(x - (double)hx), (float)(y - (double)hy), (float)(z - (double)hz), __int_as_float((int)i));
     }
 }
 
@@ -589,10 +629,12 @@ struct PosReader<float> {
         return ((hv - c.x) + (lv - c.y)) * inv;
     }
     __device__ float charge(int i) const { return hi[i].w; }
+    __device__ int input(int i) const { return __float_as_int(lo[i].w); }
 };
 template <>
 struct PosReader<double> {
     const Pos64* p;
+    const int* order;
     double s, inv;
     __device__ double centre(int c) const { return ((double)c + 0.5) * s; }
     __device__ double local(int i, int a, double c) const {
@@ -600,6 +642,7 @@ struct PosReader<double> {
         return ((a == 0 ? v.x : (a == 1 ? v.y : v.z)) - c) * inv;
     }
     __device__ double charge(int i) const { return p[i].w; }
+    __device__ int input(int i) const { return order[i]; }
 };
 
 struct LevelPtrs {
@@ -629,14 +672,14 @@ __device__ __forceinline__ void warp_reduce_nodes(T (&v)[V], int lane) {
 
 // STEP2 summed per finest cell: sum_c q_c h(c) over the cell's charges.  Node forms: weights of the cell's
 // own nodes; the coarser cells' node charges follow by k_up.  Literal U-bar-1: weights of the root box's
-// nodes (root).  A warp per chunk of up to kChunk charges of one cell, the charges over the lanes and the
+// nodes (root).  Also the sorted charges' keys.  A warp per chunk of up to kChunk charges of one cell, the charges over the lanes and the
 // nodes' sums in registers; the lanes' sums are combined by a shuffle reduce-scatter, one atomic per node.
 // 2^20 charges in 2D, levels 7: 45 us with the upward pass against 409 us for the charges' weights at each of six
 // levels, staged in shared memory.
 template <int D, typename T>
 __global__ void __launch_bounds__(kChunk) k_p2m(PosReader<T> rd, const int* __restrict__ start,
                                                 const int* __restrict__ chunk_start, int nleaf, bool root,
-                                                T* __restrict__ out) {
+                                                T* __restrict__ out, uint32_t* __restrict__ skey) {
     constexpr int d = nodes_of(D);
     const int total = chunk_start[nleaf];
     const int lane = threadIdx.x & 31;
@@ -652,6 +695,7 @@ __global__ void __launch_bounds__(kChunk) k_p2m(PosReader<T> rd, const int* __re
 #pragma unroll
         for (int j = 0; j < d; ++j) acc[j] = T(0);
         for (int i = t0 + lane; i < t1; i += 32) {
+            skey[i] = (uint32_t)b;
             T f[D][4];
 #pragma unroll
             for (int a = 0; a < D; ++a) lag_basis<T>(rd.local(i, a, centre[a]), f[a]);
@@ -1013,7 +1057,7 @@ __global__ void __launch_bounds__(kM2LThreads) k_m2l(M2LLevels lv, int ngroups) 
 // levels with its FP64 centre and division.
 template <int D, typename T>
 __global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_t n, const T* __restrict__ psi,
-                      const double* __restrict__ psi0, const double* __restrict__ nearf, double near_unit, const int* __restrict__ order,
+                      const double* __restrict__ psi0, const double* __restrict__ nearf, double near_unit,
                       const unsigned* __restrict__ status, double* __restrict__ phi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -1043,7 +1087,7 @@ __global__ void k_l2p(PosReader<T> rd, const uint32_t* __restrict__ skey, int64_
         }
     }
     if (*(volatile const unsigned*)status != 0u) return;
-    phi[order[i]] = fma(near_unit, nearf[i], base + (double)v);
+    phi[rd.input((int)i)] = fma(near_unit, nearf[i], base + (double)v);
 }
 
 // ------------------------------------------------------------------------------ literal form
@@ -1303,7 +1347,7 @@ int enqueue_nodes(fmm_lag_plan_s* pl, const PosReader<T>& rd, int64_t n, unsigne
     const auto shift_blocks = [](int64_t cells) { return (unsigned)((cells + kShiftWarps - 1) / kShiftWarps); };
     if (L >= 2) {
         k_p2m<D, T><<<gp, kChunk, 0, st>>>(rd, pl->start, pl->chunk_start, (int)pl->nleaf, false,
-                                           static_cast<T*>(pl->node[L]));
+                                           static_cast<T*>(pl->node[L]), pl->skey);
         ++launches;
         for (int k = L - 1; k >= 2; --k) {
             const int64_t cells = ipow(1 << k, D);
@@ -1348,7 +1392,7 @@ int enqueue_nodes(fmm_lag_plan_s* pl, const PosReader<T>& rd, int64_t n, unsigne
         }
     }
     lag_join(pl, st);
-    k_l2p<D, T><<<gb, 256, 0, pl->st>>>(rd, pl->skey, n, psi, psi0, pl->nearf, near_unit, pl->order, pl->status, phi);
+    k_l2p<D, T><<<gb, 256, 0, pl->st>>>(rd, pl->skey, n, psi, psi0, pl->nearf, near_unit, pl->status, phi);
     return launches + 1;
 }
 
@@ -1367,19 +1411,23 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
         if (!lit) cudaMemsetAsync(pl->pot[2], 0, pl->pot_bytes, st);
     }
     const unsigned gb = (unsigned)((n + 255) / 256);
-    k_bin<D><<<gb, 256, 0, st>>>(pos, q, n, L, pl->box, (float)((double)(1 << L) / pl->box), pl->key, pl->rank,
-                                 pl->count, pl->status);
+    const float side_over_box = (float)((double)(1 << L) / pl->box);
+    if (bin_few(pl->nleaf, n))
+        k_bin_few<D><<<(unsigned)pl->sms, kBinFewThreads, 0, st>>>(pos, q, n, L, pl->box, side_over_box, pl->key, pl->rank,
+                                                                   pl->count, (int)pl->nleaf, pl->status);
+    else
+        k_bin<D><<<gb, 256, 0, st>>>(pos, q, n, L, pl->box, side_over_box, pl->key, pl->rank, pl->count, pl->status);
     const unsigned tiles = (unsigned)((pl->nleaf + kScanTile - 1) / kScanTile);
     const int wchunk = f64 ? kWarpChunk64 : kWarpChunk;
     k_scan_sums<<<tiles, kScanTile, 0, st>>>(pl->count, (int)pl->nleaf, wchunk, pl->scan);
     k_scan<<<tiles, kScanTile, 0, st>>>(pl->count, (int)pl->nleaf, wchunk, pl->scan, pl->start, pl->chunk_start,
                                         pl->wchunk_start);
     if (f64)
-        k_scatter<D, true><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, pl->skey, pl->order,
-                                                nullptr, nullptr, pl->p64);
+        k_scatter<D, true><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, pl->order, nullptr, nullptr,
+                                               pl->p64);
     else
-        k_scatter<D, false><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, pl->skey, pl->order,
-                                                 pl->hi, pl->lo, nullptr);
+        k_scatter<D, false><<<gb, 256, 0, st>>>(pos, q, n, pl->key, pl->rank, pl->start, nullptr, pl->hi, pl->lo,
+                                                nullptr);
     launches += 4;
     cudaEventRecord(pl->ev[7], st);
     cudaEventRecord(pl->ev[1], st);
@@ -1412,23 +1460,23 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
     const double cs = pl->box / (double)(1 << L);
     const float cs_hi = (float)cs;
     const PosReader<float> rd32{pl->hi, pl->lo, make_float2(cs_hi, (float)(cs - (double)cs_hi)), (float)(5.0 / cs)};
-    const PosReader<double> rd64{pl->p64, cs, 5.0 / cs};
+    const PosReader<double> rd64{pl->p64, pl->order, cs, 5.0 / cs};
     const double near_unit = !f64 && D == 2 ? 0.5 * kLn2 : 1.0;   // the 2D FP32 near field is in log2 r^2
     if (lit && L < 2) {
         // no interaction lists: phi is the near field
         cudaEventRecord(pl->ev[2], far_st);
         cudaEventRecord(pl->ev[3], far_st);
         lag_join(pl, far_st);
-        k_l2p<D, double><<<gb, 256, 0, st>>>(rd64, pl->skey, n, nullptr, nullptr, pl->nearf, near_unit, pl->order,
-                                             pl->status, phi);
+        k_l2p<D, double><<<gb, 256, 0, st>>>(rd64, pl->skey, n, nullptr, nullptr, pl->nearf, near_unit, pl->status,
+                                             phi);
         ++launches;
     } else if (!lit) {
         if (f64) launches += enqueue_nodes<D, double>(pl, rd64, n, gp, gb, near_unit, phi);
         else launches += enqueue_nodes<D, float>(pl, rd32, n, gp, gb, near_unit, phi);
     } else {
         // U-bar-1: v of every finest cell from the charges' root-node images
-        k_p2m<D, double><<<gp, kChunk, 0, far_st>>>(PosReader<double>{pl->p64, pl->box, 5.0 / pl->box}, pl->start,
-                                                pl->chunk_start, (int)pl->nleaf, true, static_cast<double*>(pl->node[L]));
+        k_p2m<D, double><<<gp, kChunk, 0, far_st>>>(PosReader<double>{pl->p64, pl->order, pl->box, 5.0 / pl->box}, pl->start,
+                                                pl->chunk_start, (int)pl->nleaf, true, static_cast<double*>(pl->node[L]), pl->skey);
         ++launches;
         // U-bar-2: sums up the tree (levels below 2 are never read)
         for (int k = L - 1; k >= 2; --k) {
@@ -1483,6 +1531,7 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     fmm_status rc = cuda_status(cudaGetDevice(&pl->dev));
     int sms = 0;
     if (rc == FMM_OK) rc = cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl->dev));
+    pl->sms = std::max(1, sms);
     pl->grid_particles = std::max(1, sms) * 8;
     int per_sm = 0;
     if (rc == FMM_OK)
@@ -1501,7 +1550,7 @@ fmm_status fmm_lag_plan(fmm_lag_plan_t* out, int dim, int64_t n_max, int levels,
     if (rc == FMM_OK) rc = alloc(pl, &pl->key, n);
     if (rc == FMM_OK) rc = alloc(pl, &pl->rank, n);
     if (rc == FMM_OK) rc = alloc(pl, &pl->skey, n);
-    if (rc == FMM_OK) rc = alloc(pl, &pl->order, n);
+    if (rc == FMM_OK && f64) rc = alloc(pl, &pl->order, n);
     if (rc == FMM_OK) rc = alloc(pl, &pl->nearf, n);
     if (rc == FMM_OK) rc = alloc(pl, &pl->count, (size_t)pl->nleaf);
     if (rc == FMM_OK) rc = alloc(pl, &pl->start, (size_t)pl->nleaf + 1);

@@ -235,3 +235,15 @@ def test_up_and_down_passes_f64(oracle_mod, dim, levels, box):
     assert np.array_equal(cells, oracle_mod.lag_cells(pos, levels, box))
     phi, _, _ = run(pos, q, levels, "node_f32", box)
     check_parity(phi, oracle_mod.lag_node(pos, q, levels, box), TOL32, f"node_f32 D={dim} L={levels} box={box}")
+
+
+@pytest.mark.parametrize("form,tol", [("node_f32", TOL32), ("node_f64", TOL64)])
+@pytest.mark.parametrize("dim,levels,n", [(2, 0, 8192), (2, 3, 8193), (3, 2, 8191), (3, 2, 12345), (3, 3, 32769), (2, 5, 65537)])
+def test_binning_with_few_cells(oracle_mod, form, tol, dim, levels, n):
+    """Charges binned by way of shared memory, at the smallest numbers that take that kernel and just below, clumped
+    so that cells range from empty to crowded."""
+    pos, q = inputs.paper_cube(n, 5000 + 10 * dim + levels, dim)
+    pos[::3] = 2.0 + 0.25 * pos[::3]
+    phi, _, cells = run(pos, q, levels, form)
+    assert np.array_equal(cells, oracle_mod.lag_cells(pos, levels))
+    check_parity(phi, oracle_mod.lag_node(pos, q, levels), tol, f"{form} D={dim} L={levels} n={n}")
