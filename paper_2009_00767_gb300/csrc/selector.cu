@@ -32,13 +32,13 @@ static_assert(kLevMin == 3 && kLevMax == 11 && kHistLevels * kBins <= 256, "k_oc
 
 // ---------------------------------------------------------------- occupancy statistics
 // One count per particle, in its square of the finest level; the coarser levels' populations are sums of
-// four.  What bounds it: the atomics in L2, so a ninth of them.  2^20 particles: 22 us; a call of
-// fmm_selector_features and one of fmm_select take 141 us together, 1087 us with an atomic per particle and level.
-__global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double box, uint32_t* __restrict__ cnt) {
+// four.  What bounds it: the atomics in L2, so a ninth of them; sob = 2^kLevMax / box comes from the host, as an
+// FP64 division a thread took 22 us.  2^20 particles: 8 us; a call of fmm_selector_features and one of
+// fmm_select take 117 us together, 1087 us with an atomic per particle and level.
+__global__ void k_occ_count(const double2* __restrict__ xy, int64_t n, double box, float sob, uint32_t* __restrict__ cnt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double2 p = xy[i];
-    const float sob = (float)((double)(1 << kLevMax) / box);
     const int side = 1 << kLevMax;
     const int ix = finest_coord(p.x, (double)side, sob, box, side);
     const int iy = finest_coord(p.y, (double)side, sob, box, side);
@@ -354,7 +354,8 @@ bool enqueue_occupancies(fmm_selector_s* s, const double* xy, int64_t n, double 
     if (cudaMemsetAsync(s->cnt, 0, sizeof(uint32_t) * kOccFine, st) != cudaSuccess ||
         cudaMemsetAsync(s->hist, 0, kHistBytes + sizeof(uint32_t), st) != cudaSuccess)
         return false;
-    k_occ_count<<<nblk(n, 256), 256, 0, st>>>(reinterpret_cast<const double2*>(xy), n, box, s->cnt);
+    k_occ_count<<<nblk(n, 256), 256, 0, st>>>(reinterpret_cast<const double2*>(xy), n, box,
+                                           (float)((double)(1 << kLevMax) / box), s->cnt);
     k_occ_hist<<<(unsigned)(kOccTiles / kOccWarps), kOccWarps * 32, 0, st>>>(s->cnt, s->cnt + kOccFine, s->hist,
                                                                              s->hist + kHistLevels * kBins);
     return cudaGetLastError() == cudaSuccess;
