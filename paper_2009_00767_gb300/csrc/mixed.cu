@@ -816,8 +816,10 @@ k_p2p_field(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
     if (*(volatile const unsigned int*)status != 0u) return;
     const uint32_t leaf = lt.x;
     const uint32_t t0 = leaf_start[leaf], t1 = leaf_start[leaf + 1];
-    const uint32_t b0 = t0 + (uint32_t)FMM_P2P_BLOCK * lt.y;
-    const int T = (int)min((uint32_t)FMM_P2P_BLOCK, t1 - b0);
+    // a square's blocks are of (almost) equal size
+    const uint32_t pop = t1 - t0, nblk = (pop + FMM_P2P_BLOCK - 1) / FMM_P2P_BLOCK;
+    const uint32_t b0 = t0 + (uint32_t)((uint64_t)pop * lt.y / nblk);
+    const int T = (int)(t0 + (uint32_t)((uint64_t)pop * (lt.y + 1) / nblk) - b0);
     uint32_t pairs;
     const NearField nf = p2p_near_sym_field(sp, lo, leaf_start, leaf, t0, t1, b0, T, levels, s_leaf, tgt[warp],
                                             tlo[warp], tq[warp], seg[warp], lane, acc, accg, &pairs);

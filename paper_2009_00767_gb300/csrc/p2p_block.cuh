@@ -395,18 +395,24 @@ __device__ __forceinline__ unsigned long long p2p_near_crowd(const float4* __res
 // so FP32 square-local coordinates alone (about 1e-9 of the box) would limit it; each coordinate
 // also carries its FP32 rounding residue (written by the sort for field calls), and a pair's
 // difference takes the high words (exact for close pairs) plus the residues' difference.
+// What bounds it: instruction fetch first.  The loop over the target pairs is unrolled, so each instance for a
+// number of pairs is up to 7 kB; one body for both kinds of chunk and three instances instead of six of two
+// bodies each keep the warps of an SM in the same code.  200,003 particles in a ring (levels 7): 60 us against 91,
+// where a warp waited six issue slots for an instruction (0.1 now); then the waits on registers' latencies, with
+// 16 warps an SM.
 struct NearField {
     float2 phi, gx, gy;   // float-float sums of target `lane`
 };
 
-template <bool kOwn, int NP>
+// One chunk: the lane's source against the NP target pairs, both sides (the source's sums of an own-square chunk
+// are dropped).  tiny is 0 in the own square, where a coincident pair gives 0, and 2^-100 elsewhere.
+template <int NP>
 __device__ __forceinline__ float3 p2p_chunk_field(float2 (&pp)[NP], float2 (&px)[NP], float2 (&py)[NP],
                                                   const float4* __restrict__ tg, const float4* __restrict__ tl,
-                                                  const float2* __restrict__ tq, float4 src, float2 slo) {
+                                                  const float2* __restrict__ tq, float4 src, float2 slo, float tiny) {
     const float2 nsx = make_float2(-src.x, -src.x), nsy = make_float2(-src.y, -src.y);
     const float2 nlx = make_float2(-slo.x, -slo.x), nly = make_float2(-slo.y, -slo.y);
-    const float2 q2 = make_float2(src.z, src.z);
-    const float2 tiny = make_float2(0x1p-100f, 0x1p-100f);
+    const float2 q2 = make_float2(src.z, src.z), tiny2 = make_float2(tiny, tiny);
     float2 sp = make_float2(0.f, 0.f), sx = make_float2(0.f, 0.f), sy = make_float2(0.f, 0.f);
 #pragma unroll
     for (int tp = 0; tp < NP; ++tp) {
@@ -414,30 +420,18 @@ __device__ __forceinline__ float3 p2p_chunk_field(float2 (&pp)[NP], float2 (&px)
         // the coordinates' high words differ exactly for close pairs; the low words carry the rest
         const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(t.x, t.y), nsx), __fadd2_rn(make_float2(u.x, u.y), nlx));
         const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(t.z, t.w), nsy), __fadd2_rn(make_float2(u.z, u.w), nly));
-        float2 r2, lg, iv;
-        if (kOwn) {
-            r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-            lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-            iv = make_float2(mufu_rcp(r2.x), mufu_rcp(r2.y));
-            lg.x = r2.x > 0.f ? lg.x : 0.f;
-            lg.y = r2.y > 0.f ? lg.y : 0.f;
-            iv.x = r2.x > 0.f ? iv.x : 0.f;
-            iv.y = r2.y > 0.f ? iv.y : 0.f;
-        } else {
-            r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, tiny));
-            lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-            iv = make_float2(mufu_rcp(r2.x), mufu_rcp(r2.y));
-        }
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, tiny2));
+        const bool ax = r2.x > 0.f, ay = r2.y > 0.f;
+        const float2 lg = make_float2(ax ? mufu_lg2(r2.x) : 0.f, ay ? mufu_lg2(r2.y) : 0.f);
+        const float2 iv = make_float2(ax ? mufu_rcp(r2.x) : 0.f, ay ? mufu_rcp(r2.y) : 0.f);
         const float2 wx = __fmul2_rn(dx, iv), wy = __fmul2_rn(dy, iv);   // (dx, dy) / r^2
+        const float2 qt = tq[tp];
         pp[tp] = __ffma2_rn(q2, lg, pp[tp]);
         px[tp] = __ffma2_rn(q2, wx, px[tp]);
         py[tp] = __ffma2_rn(q2, wy, py[tp]);
-        if (!kOwn) {
-            const float2 qt = tq[tp];
-            sp = __ffma2_rn(qt, lg, sp);
-            sx = __ffma2_rn(qt, wx, sx);
-            sy = __ffma2_rn(qt, wy, sy);
-        }
+        sp = __ffma2_rn(qt, lg, sp);
+        sx = __ffma2_rn(qt, wx, sx);
+        sy = __ffma2_rn(qt, wy, sy);
     }
     return make_float3(sp.x + sp.y, -(sx.x + sx.y), -(sy.x + sy.y));   // the source's phi and gradient
 }
@@ -495,15 +489,11 @@ __device__ __forceinline__ NearField p2p_block_sym_field(const P2PSymSources& S,
             uint32_t nidx = idx;
             float2 nlo = clo;
             const float4 nxt = (c + 1 < r1) ? load_lo(S, lo, c + 1, lane, &nidx, &nlo) : cur;
-            if (c < S.nch_own) {
-                p2p_chunk_field<true, NP>(pp, px, py, tg, tl, tq, cur, clo);
-            } else {
-                const float3 sv = p2p_chunk_field<false, NP>(pp, px, py, tg, tl, tq, cur, clo);
-                if (idx != 0xffffffffu) {
-                    atomicAdd(acc + idx, fmm_f2d_bits(sv.x));
-                    atomicAdd(&accg[idx].x, fmm_f2d_bits(sv.y));
-                    atomicAdd(&accg[idx].y, fmm_f2d_bits(sv.z));
-                }
+            const float3 sv = p2p_chunk_field<NP>(pp, px, py, tg, tl, tq, cur, clo, c < S.nch_own ? 0.f : 0x1p-100f);
+            if (idx != 0xffffffffu) {   // a forward source
+                atomicAdd(acc + idx, fmm_f2d_bits(sv.x));
+                atomicAdd(&accg[idx].x, fmm_f2d_bits(sv.y));
+                atomicAdd(&accg[idx].y, fmm_f2d_bits(sv.z));
             }
             cur = nxt;
             idx = nidx;
@@ -568,12 +558,9 @@ __device__ __forceinline__ NearField p2p_near_sym_field(const float4* __restrict
         reinterpret_cast<float*>(&tq[lane >> 1])[lane & 1] = q;
     }
     __syncwarp();
-    switch ((T + 3) >> 2) {
-        case 1: return p2p_block_sym_field<2>(S, lo, tgt, tlo, tq, lane, acc, accg);
-        case 2: return p2p_block_sym_field<4>(S, lo, tgt, tlo, tq, lane, acc, accg);
-        case 3: return p2p_block_sym_field<6>(S, lo, tgt, tlo, tq, lane, acc, accg);
-        case 4: return p2p_block_sym_field<8>(S, lo, tgt, tlo, tq, lane, acc, accg);
-        case 5: return p2p_block_sym_field<10>(S, lo, tgt, tlo, tq, lane, acc, accg);
+    switch ((T + 7) >> 3) {
+        case 1: return p2p_block_sym_field<4>(S, lo, tgt, tlo, tq, lane, acc, accg);
+        case 2: return p2p_block_sym_field<8>(S, lo, tgt, tlo, tq, lane, acc, accg);
         default: return p2p_block_sym_field<12>(S, lo, tgt, tlo, tq, lane, acc, accg);
     }
 }
