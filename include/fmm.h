@@ -91,7 +91,7 @@ typedef struct {
     double ms_p2m;             /* moments of levels 2..levels */
     double ms_m2l;             /* interaction-list conversion of levels 2..levels */
     double ms_l2p;             /* local evaluation of levels 2..levels */
-    double ms_p2p;             /* near field + final phi in input order */
+    double ms_p2p;             /* near field */
     int64_t p2p_pairs;         /* ordered source-target pairs of the near field (counted on device) */
     int64_t max_leaf;          /* largest finest-square population */
     int kernel_launches;       /* kernels the library launched for that call */
@@ -101,7 +101,8 @@ typedef struct {
     /* Mixed path: the near field (from the sort on), the coarse levels' chain (from the fine P2M
      * on: upward pass to levels levels-3 .. 2, M2L and L2P of levels 2..5) and the fine levels'
      * P2M and M2L run on three streams at once, so ms_p2m, ms_m2l and ms_l2p above are sums of
-     * these spans and the stages overlap in time.  FP64 path: ms_m2l_fine = ms_m2l, the others 0. */
+     * these spans and the stages overlap in time.  FP64 path: the near field runs beside P2M, M2L and the
+     * downward pass (counted in ms_l2p); ms_m2l_fine = ms_m2l, the others 0. */
     double ms_p2m_fine;        /* P2M of the finest three levels */
     double ms_p2m_coarse;      /* the coarser levels' moments by the upward pass (M2M) */
     double ms_m2l_fine;        /* M2L of levels 6 and finer (tensor-core prep + kernel, or FP32) */
@@ -127,9 +128,10 @@ typedef struct {
 fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box,
                     int precision, void* stream);
 
-/* How many streams a mixed-precision call spreads its work over: 3 (the default: after the
- * fine levels' P2M the near field, the coarse levels' chain and the fine levels' M2L run at
- * once on the plan's stream and two streams of its own, joined back before L2P) or 1 (every
+/* How many streams a call spreads its work over: 3 (the default: after the fine levels' P2M
+ * the near field, the coarse levels' chain and the fine levels' M2L run at once on the plan's
+ * stream and two streams of its own, joined back before L2P; an FP64 call runs its far field
+ * beside its near field, on one stream of the plan's own) or 1 (every
  * kernel in turn on the plan's stream, so that fmm_plan_stats times each kernel alone).  The
  * results are the same either way.  FMM_ERR_INVALID_ARG for another count or a NULL plan. */
 fmm_status fmm_set_concurrency(fmm_plan_t plan, int streams);

@@ -231,8 +231,8 @@ void read_times(fmm_plan_s* plan) {
     if (plan->precision == FMM_FP64) {
         plan->last.ms_p2m = span(1, 2);
         plan->last.ms_m2l = span(2, 3);
-        plan->last.ms_l2p = span(3, 4);
-        plan->last.ms_p2p = span(4, 5);
+        plan->last.ms_l2p = span(3, 15) + span(4, 5);   // the downward pass and the evaluation
+        plan->last.ms_p2p = span(8, 9);
         plan->last.ms_p2m_fine = plan->last.ms_p2m_coarse = plan->last.ms_m2l_coarse = 0.0;
         plan->last.ms_m2l_fine = plan->last.ms_m2l;
     } else {
@@ -419,10 +419,15 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         for (cudaEvent_t& e : set)
             if (cudaEventCreate(&e) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
     pl->ev = pl->ev_sets[0];
-    if (precision != FMM_FP64) {
+    int least = 0, greatest = 0;
+    if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) FMM_TRY(FMM_ERR_CUDA);
+    if (precision == FMM_FP64) {
+        // the far field's stream: its small launches go before the near field's blocks
+        if (cudaStreamCreateWithPriority(&pl->stream2, cudaStreamNonBlocking, greatest) != cudaSuccess)
+            FMM_TRY(FMM_ERR_CUDA);
+    } else {
         // the mixed path's near field and coarse levels run on streams of the plan's own
         if (cudaStreamCreateWithFlags(&pl->stream2, cudaStreamNonBlocking) != cudaSuccess ||
-
             cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&pl->ev_join, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&pl->ev_join3, cudaEventDisableTiming) != cudaSuccess ||
@@ -433,9 +438,7 @@ fmm_status fmm_plan(fmm_plan_t* out, int64_t n, int levels, int p, double box, i
         // The coarse levels' chain (upward pass, coarse M2L and L2P) is a string of small launches
         // behind the fine P2M; at the device's highest priority its blocks go first whenever the
         // near field's blocks leave an SM, instead of after all of them.
-        int least = 0, greatest = 0;
-        if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&pl->stream3, cudaStreamNonBlocking, greatest) != cudaSuccess)
+        if (cudaStreamCreateWithPriority(&pl->stream3, cudaStreamNonBlocking, greatest) != cudaSuccess)
             FMM_TRY(FMM_ERR_CUDA);
         cudaEvent_t* evs[] = {&pl->ev_sorted, &pl->ev_stage_free[0], &pl->ev_stage_free[1], &pl->ev_up_done,
                               &pl->ev_l2p_done, &pl->ev_down_done[0], &pl->ev_down_done[1]};

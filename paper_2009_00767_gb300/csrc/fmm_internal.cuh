@@ -13,8 +13,7 @@
 //   A32[k]                   (mixed) FP32 moments of level k, same layout (the mixed path has no
 //                            FP64 A[k]); slot 0 holds M_0 as a float-float pair
 //   (mixed) B[k] slot 0 holds Re b'_0 as a float-float pair
-//   phi_far[n]               FP64 path: far field, then far + near, box-sorted order; mixed
-//                            path: the near field as float-float pairs (log2 r^2 units)
+//   phi_far[n]               the near field, box-sorted order; mixed path: in log2 r^2 units
 //   ftab                     (FP64 path) the translations' real matrices R[k][l] and C(m, j), and the
 //                            powers d^-k of the interaction-list offsets
 // Because keys are Morton-ordered, the particles of every square of every level are one
@@ -107,8 +106,8 @@ struct fmm_plan_s {
     float2* sorted_lo;           // mixed path, field calls: the local coordinates' FP32 rounding residues
     FmmLevelPtrs grids;
     size_t a_bytes[FMM_MAX_LEVELS + 1];
-    double* phi_far;                  // FP64 path: far field; mixed path: near-field accumulator per particle
-    double2* near_grad;               // mixed path: near-field gradient accumulator (fmm_potential_field)
+    double* phi_far;                  // near-field accumulator per particle
+    double2* near_grad;               // near-field gradient accumulator (fmm_potential_field)
     float2* far_part;                 // mixed path: float-float far field of the coarse levels per particle
 
     double* ftab;       // FP64 path: the far field's real matrices and powers (fp64_math.cuh)
@@ -147,11 +146,13 @@ struct fmm_plan_s {
     // the work forks three ways -- the near field on stream2, the coarse levels' chain (P2M,
     // conversion, M2L and L2P of levels 2..5) on stream3, the fine levels' P2M and M2L on the plan's
     // stream -- and joins back before the fine levels' L2P.
+    // FP64 path: the far field on stream2 beside the near field on the plan's stream.
     cudaStream_t stream2, stream3;
     cudaEvent_t ev_fork, ev_join, ev_join3;   // untimed fork / join events
     cudaEvent_t ev_a32;   // stream3's FP32 moment grids are written (levels 2 .. l-3; from l = 9 on the
                           // fine levels' M2L on the plan's stream reads some of them)
-    // Timing events.  FP64 path: stage boundaries [0..5] (sort, P2M, M2L, L2P, P2P).  Mixed path:
+    // Timing events.  FP64 path: [0] start, [1] sort done, [2] upward pass done, [3] M2L done, [15] downward
+    // pass done (these three on stream2), [8, 9] the near field, [4] L2P start, [5] end.  Mixed path:
     // [0] start, [1] sort done, [2] fine P2M done, [14] fine M2L start, [3] fine M2L done, [4] L2P
     // start (after the joins), [5] end, all on the plan's stream; [6, 7] the tensor-core M2L
     // kernel; [8, 9] the near-field kernel (stream2); [10, 11] the upward pass, [11, 13] the coarse

@@ -317,49 +317,55 @@ __global__ void __launch_bounds__(kFarThreads) k_m2l_f64(M2LArgs a) {
 }
 
 // -------------------------------------------------------------------------------- L2P
-// The finest square's local expansion at each particle by Horner's rule.
+// The finest square's local expansion at each particle by Horner's rule, added to the near field (near, grad)
+// and written in input order, unless the inputs failed the device checks.
 // kField: also the far field's gradient, grad phi = (Re f', -Im f') with f'(z) = sum_l l b_l w^(l-1) / s
-// (one Horner pass for the expansion and its derivative), per sorted particle into grad_far.
+// (one Horner pass for the expansion and its derivative), and E = -grad phi.
 template <bool kField>
 __global__ void k_l2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __restrict__ skey, int64_t n,
                           int levels, int p, double s, double inv_s, const double2* __restrict__ B,
-                          double* __restrict__ phi_far, double2* __restrict__ grad_far) {
+                          const double* __restrict__ near, const double2* __restrict__ grad,
+                          const unsigned int* __restrict__ status, double* __restrict__ phi, double* __restrict__ field) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    if (levels < 2) {   // no far field
-        phi_far[i] = 0.0;
-        if (kField) grad_far[i] = make_double2(0.0, 0.0);
-        return;
-    }
+    if (*(volatile const unsigned int*)status != 0u) return;
     const fmm_p64 P = sp[i];
-    const uint32_t key = skey[i];
-    const uint32_t bx = fmm_compact2(key), by = fmm_compact2(key >> 1);
-    const double wx = (P.x - ((double)bx + 0.5) * s) * inv_s;
-    const double wy = (P.y - ((double)by + 0.5) * s) * inv_s;
-    const double2* Bt = B + ((size_t)by * (1u << levels) + bx) * (p + 1);
-    double2 acc = Bt[p], d = make_double2(0.0, 0.0);
-    for (int l = p - 1; l >= 0; --l) {
-        const double2 b = Bt[l];
-        if (kField) {   // d <- d w + acc before acc moves on: d ends as the derivative
-            const double dr = fma(d.x, wx, fma(-d.y, wy, acc.x));
-            const double di = fma(d.x, wy, fma(d.y, wx, acc.y));
-            d.x = dr;
-            d.y = di;
+    double2 acc = make_double2(0.0, 0.0), d = make_double2(0.0, 0.0);
+    if (levels >= 2) {   // else no far field
+        const uint32_t key = skey[i];
+        const uint32_t bx = fmm_compact2(key), by = fmm_compact2(key >> 1);
+        const double wx = (P.x - ((double)bx + 0.5) * s) * inv_s;
+        const double wy = (P.y - ((double)by + 0.5) * s) * inv_s;
+        const double2* Bt = B + ((size_t)by * (1u << levels) + bx) * (p + 1);
+        acc = Bt[p];
+        for (int l = p - 1; l >= 0; --l) {
+            const double2 b = Bt[l];
+            if (kField) {   // d <- d w + acc before acc moves on: d ends as the derivative
+                const double dr = fma(d.x, wx, fma(-d.y, wy, acc.x));
+                const double di = fma(d.x, wy, fma(d.y, wx, acc.y));
+                d.x = dr;
+                d.y = di;
+            }
+            const double r = fma(acc.x, wx, fma(-acc.y, wy, b.x));
+            const double im = fma(acc.x, wy, fma(acc.y, wx, b.y));
+            acc.x = r;
+            acc.y = im;
         }
-        const double r = fma(acc.x, wx, fma(-acc.y, wy, b.x));
-        const double im = fma(acc.x, wy, fma(acc.y, wx, b.y));
-        acc.x = r;
-        acc.y = im;
     }
-    phi_far[i] = acc.x;
-    if (kField) grad_far[i] = make_double2(d.x * inv_s, -d.y * inv_s);
+    const int64_t o = (int64_t)P.w;
+    phi[o] = acc.x + near[i];
+    if (kField) {
+        const double2 g = grad[i];
+        field[2 * o] = -(d.x * inv_s + g.x);
+        field[2 * o + 1] = d.y * inv_s - g.y;
+    }
 }
 
-// -------------------------------------------------------------------------------- P2P + final phi
+// -------------------------------------------------------------------------------- P2P
 // The near field, each pair of the own and adjacent squares once (p2p64.cuh): one warp per block of up to
 // FMM_P2P_BLOCK targets of a finest square (blk_map, from the sort's scan), whose later sources are the
-// rest of the own square and the forward neighbours E, NE, N, NW.  Every result is added to the far field
-// with an FP64 atomic; k_finish_f64 then writes phi in input order.
+// rest of the own square and the forward neighbours E, NE, N, NW.  Every result is added to the particle's
+// sum with an FP64 atomic.
 // 2^20 uniform particles, levels 8: 1.93 ms against 15.0 ms for a kernel that took every ordered pair with
 // the library's log.
 // kField: also grad phi, q (dx, dy) / r^2 to the target and the opposite to the source.
@@ -420,22 +426,6 @@ k_p2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __restrict__ leaf_star
         [&](const P64Acc<kField>& a) { p2p64_add<kField>(phi, grad, b0 + lane, a); });
 }
 
-// phi (and E = -grad phi) in input order
-template <bool kField>
-__global__ void k_finish_f64(const fmm_p64* __restrict__ sp, int64_t n, const double* __restrict__ acc,
-                             const double2* __restrict__ grad, const unsigned int* __restrict__ status,
-                             double* __restrict__ phi, double* __restrict__ field) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (*(volatile const unsigned int*)status != 0u) return;   // inputs failed the device checks
-    const int64_t o = (int64_t)sp[i].w;
-    phi[o] = acc[i];
-    if (kField) {
-        field[2 * o] = -grad[i].x;
-        field[2 * o + 1] = -grad[i].y;
-    }
-}
-
 // -------------------------------------------------------------------------------- FP64 direct sum
 __global__ void k_direct_f64(int64_t n, const double2* __restrict__ xy, const double* __restrict__ q,
                              const int64_t* __restrict__ targets, double* __restrict__ out) {
@@ -462,7 +452,13 @@ __global__ void k_direct_f64(int64_t n, const double2* __restrict__ xy, const do
 }  // namespace
 
 int fmm_launch_fp64(fmm_plan_s* pl, double* phi, double* field) {
-    cudaStream_t st = pl->stream;
+    // The far field runs on the plan's own stream, at the device's highest priority, beside the near field on
+    // the caller's.  Both are bound by the FP64 pipe; what overlaps is the chain of small launches of the
+    // coarse levels, which leaves most of the chip idle, and with few particles all of it: 4,096 particles
+    // (levels 4, p = 16) 174 -> 135 us, 2^20 (levels 8, p = 20) 5.17 -> 5.05 ms.
+    // In turn on the caller's stream with fmm_set_concurrency(plan, 1) and without a plan (no stream2).
+    const bool owned = pl->stream2 != nullptr, two = owned && !pl->serial;
+    cudaStream_t near_st = pl->stream, st = two ? pl->stream2 : pl->stream;
     const int64_t n = pl->n;
     const int L = pl->levels, p = pl->p, p1 = p + 1;
     const double s = pl->box / (double)(1 << L), inv_s = (double)(1 << L) / pl->box;
@@ -477,9 +473,12 @@ int fmm_launch_fp64(fmm_plan_s* pl, double* phi, double* field) {
     const size_t shm_m2l = sizeof(double) * tab + sizeof(double2) * (kFmmOrbits * p1 + 2 * 4 * p1 * per);
     int launches = 0;
     // P2M of the finest level (its grid starts at zero), then the upward pass
-    cudaEventRecord(pl->ev[1], st);
+    cudaEventRecord(pl->ev[1], near_st);
+    // the finest grid is free from the call's start on (the previous call's L2P ended there)
+    if (two && cudaStreamWaitEvent(st, pl->ev[0], 0) != cudaSuccess) return -1;
+    if (L >= 2 && cudaMemsetAsync(pl->grids.A[L], 0, pl->a_bytes[L], st) != cudaSuccess) return -1;
+    if (two && cudaStreamWaitEvent(st, pl->ev[1], 0) != cudaSuccess) return -1;
     if (L >= 2) {
-        if (cudaMemsetAsync(pl->grids.A[L], 0, pl->a_bytes[L], st) != cudaSuccess) return -1;
         const int64_t warps = (n + 31) / 32;
         const unsigned blocks = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
         const size_t shm = sizeof(double) * kWarpsPerBlock * 32 * (2 * p1 + 1);
@@ -520,47 +519,50 @@ int fmm_launch_fp64(fmm_plan_s* pl, double* phi, double* field) {
         ++launches;
     }
     cudaEventRecord(pl->ev[3], st);
-    // the downward pass, then L2P at the finest level
+    // the downward pass
     for (int k = 2; k < L; ++k) {
         k_l2l_f64<<<((1 << (2 * k)) + per - 1) / per, threads, shm_down, st>>>(
             static_cast<const double2*>(pl->grids.B[k]), static_cast<double2*>(pl->grids.B[k + 1]), binom, k, p1);
         ++launches;
     }
-    {
-        const unsigned blocks = (unsigned)((n + 127) / 128);
-        const double2* B = static_cast<const double2*>(pl->grids.B[L]);
-        if (field)
-            k_l2p_f64<true><<<blocks, 128, 0, st>>>(pl->sorted64, pl->sorted_key, n, L, p, s, inv_s, B, pl->phi_far,
-                                                    pl->near_grad);
-        else
-            k_l2p_f64<false><<<blocks, 128, 0, st>>>(pl->sorted64, pl->sorted_key, n, L, p, s, inv_s, B, pl->phi_far,
-                                                     nullptr);
-        ++launches;
-    }
-    cudaEventRecord(pl->ev[4], st);
-    // P2P, then phi in input order
+    if (owned) cudaEventRecord(pl->ev[15], st);
+    // the near field, on the caller's stream
+    if (cudaMemsetAsync(pl->phi_far, 0, sizeof(double) * (size_t)n, near_st) != cudaSuccess ||
+        (field && cudaMemsetAsync(pl->near_grad, 0, sizeof(double2) * (size_t)n, near_st) != cudaSuccess))
+        return -1;
+    if (owned) cudaEventRecord(pl->ev[8], near_st);
     {
         const uint32_t nleaf = 1u << (2 * L);
         const int64_t wmax = (int64_t)nleaf + n / FMM_P2P_BLOCK + 1;
         // few blocks: two warps a CTA, so that they reach more SMs
         const int warps = wmax < kP2PSmall ? 2 : kP2PWarps64;
-        const unsigned blocks = (unsigned)((wmax + warps - 1) / warps), nblk = (unsigned)((n + 255) / 256);
-        if (field) {
-            k_p2p_f64<true><<<blocks, warps * 32, 0, st>>>(pl->sorted64, pl->leaf_start, pl->leaf_bstart, pl->blk_map,
-                                                           nleaf, L, pl->logtab, pl->phi_far, pl->near_grad,
-                                                           pl->d_status, pl->d_counters);
-            k_finish_f64<true><<<nblk, 256, 0, st>>>(pl->sorted64, n, pl->phi_far, pl->near_grad, pl->d_status, phi,
-                                                     field);
-        } else {
-            k_p2p_f64<false><<<blocks, warps * 32, 0, st>>>(pl->sorted64, pl->leaf_start, pl->leaf_bstart,
-                                                            pl->blk_map, nleaf, L, pl->logtab, pl->phi_far, nullptr,
-                                                            pl->d_status, pl->d_counters);
-            k_finish_f64<false><<<nblk, 256, 0, st>>>(pl->sorted64, n, pl->phi_far, nullptr, pl->d_status, phi,
-                                                      nullptr);
-        }
-        launches += 2;
+        const unsigned blocks = (unsigned)((wmax + warps - 1) / warps);
+        if (field)
+            k_p2p_f64<true><<<blocks, warps * 32, 0, near_st>>>(pl->sorted64, pl->leaf_start, pl->leaf_bstart,
+                                                                pl->blk_map, nleaf, L, pl->logtab, pl->phi_far,
+                                                                pl->near_grad, pl->d_status, pl->d_counters);
+        else
+            k_p2p_f64<false><<<blocks, warps * 32, 0, near_st>>>(pl->sorted64, pl->leaf_start, pl->leaf_bstart,
+                                                                 pl->blk_map, nleaf, L, pl->logtab, pl->phi_far, nullptr,
+                                                                 pl->d_status, pl->d_counters);
+        ++launches;
     }
-    cudaEventRecord(pl->ev[5], st);
+    if (owned) cudaEventRecord(pl->ev[9], near_st);
+    if (two && cudaStreamWaitEvent(near_st, pl->ev[15], 0) != cudaSuccess) return -1;
+    cudaEventRecord(pl->ev[4], near_st);
+    // L2P at the finest level, with the near field and in input order
+    {
+        const unsigned blocks = (unsigned)((n + 127) / 128);
+        const double2* B = static_cast<const double2*>(pl->grids.B[L]);
+        if (field)
+            k_l2p_f64<true><<<blocks, 128, 0, near_st>>>(pl->sorted64, pl->sorted_key, n, L, p, s, inv_s, B, pl->phi_far,
+                                                         pl->near_grad, pl->d_status, phi, field);
+        else
+            k_l2p_f64<false><<<blocks, 128, 0, near_st>>>(pl->sorted64, pl->sorted_key, n, L, p, s, inv_s, B, pl->phi_far,
+                                                          nullptr, pl->d_status, phi, nullptr);
+        ++launches;
+    }
+    cudaEventRecord(pl->ev[5], near_st);
     if (cudaGetLastError() != cudaSuccess) return -1;
     return launches;
 }
