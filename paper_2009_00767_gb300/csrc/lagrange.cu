@@ -324,6 +324,10 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 // wavefronts for two targets) serve four pairs.  200,000 charges in 3D, levels 3: 467 us against 739 us for
 // 64 targets over the lanes and a butterfly over the lanes per source tile (31 shuffles, 62 selects) for the
 // source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us.
+// In 2D, with a few chunks an item, the warps of an SM are at many places of the unrolled code and wait for
+// instructions, so the code is kept small: the chunk itself and a last half chunk share a body, and whole
+// chunks are masked in every cell (the call 384 -> 366 us; in 3D, where one body runs for long, the call would
+// grow by 0.8% and 6%).
 constexpr int kP2PWarps = 4;     // warps per block, each on its own work items
 template <int D>
 __host__ __device__ constexpr int fwd_group() { return D == 3 ? 4 : 5; }   // forward cells per work item
@@ -464,10 +468,6 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
 #pragma unroll
     for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
     double acc = 0.0;
-    if (self) {
-        const bool have = lane < T;
-        p2p_lag_chunk<D, true, NP, 1>(part, tg, have ? hi[t0 + lane] : far4, have ? lo[t0 + lane] : zero4, far4, zero4);
-    }
     const uint32_t nsrc = end[4];
     auto load = [&](uint32_t slot, float4& h, float4& l, uint32_t& idx) {
         h = far4;
@@ -482,19 +482,33 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
             l = lo[idx];
         }
     };
+    // the chunk's own charges, one-sided: in 2D the loop's first pass
+    auto own = [](int c) { return D == 2 && c < 0; };
+    auto load_own = [&](float4& h, float4& l) {
+        h = lane < T ? hi[t0 + lane] : far4;
+        l = lane < T ? lo[t0 + lane] : zero4;
+    };
+    if (D == 3 && self) {
+        float4 h, l;
+        load_own(h, l);
+        p2p_lag_chunk<D, true, NP, 1>(part, tg, h, l, far4, zero4);
+    }
     int run = 0;
 #pragma unroll 1
-    for (uint32_t c = 0; c < nsrc; c += 64u) {
-        float4 ha, la, hb, lb;
-        uint32_t ia, ib;
-        load(c + (uint32_t)lane, ha, la, ia);
-        load(c + 32u + (uint32_t)lane, hb, lb, ib);
-        float2 v;
-        if (c + 32u >= nsrc)   // a last half chunk (masked, which is right for every pair)
-            v = p2p_lag_chunk<D, true, NP, 1>(part, tg, ha, la, hb, lb);
-        else
-            v = c < n_own ? p2p_lag_chunk<D, true, NP, 2>(part, tg, ha, la, hb, lb)
-                          : p2p_lag_chunk<D, false, NP, 2>(part, tg, ha, la, hb, lb);
+    for (int c = D == 2 && self ? -1 : 0; c < (int)nsrc; c = own(c) ? 0 : c + 64) {
+        float4 ha = far4, la = zero4, hb = far4, lb = zero4;
+        uint32_t ia = 0xffffffffu, ib = 0xffffffffu;
+        if (own(c)) {
+            load_own(ha, la);
+        } else {
+            load((uint32_t)(c + lane), ha, la, ia);
+            load((uint32_t)(c + 32 + lane), hb, lb, ib);
+        }
+        const float2 v = own(c) || c + 32 >= (int)nsrc   // a last half chunk
+                             ? p2p_lag_chunk<D, true, NP, 1>(part, tg, ha, la, hb, lb)
+                         : D == 2 || (uint32_t)c < n_own   // masked, which is right for every pair
+                             ? p2p_lag_chunk<D, true, NP, 2>(part, tg, ha, la, hb, lb)
+                             : p2p_lag_chunk<D, false, NP, 2>(part, tg, ha, la, hb, lb);
         if (ia != 0xffffffffu) atomicAdd(nearf + ia, f2d(v.x));
         if (ib != 0xffffffffu) atomicAdd(nearf + ib, f2d(v.y));
         run += 2;
