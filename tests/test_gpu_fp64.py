@@ -178,3 +178,28 @@ def test_far_field_orders(oracle_mod, p, lev):
     rp, rf = oracle_mod.shiftfree_field(xy, q, lev, p)
     check_parity(phi.cpu().numpy(), rp, TOL, f"fp64 far p={p} levels={lev}")
     check_parity(field.cpu().numpy().ravel(), np.asarray(rf).ravel(), TOL, f"fp64 far field p={p} levels={lev}")
+
+
+@pytest.mark.parametrize("n,levels,p", [(2, 0, 4), (300, 1, 6), (2000, 2, 8), (4096, 4, 16), (30001, 6, 9)])
+def test_far_field_beside_the_near_field(oracle_mod, n, levels, p):
+    """Two streams against one and the oracle, on calls in a row with new inputs and no wait between them."""
+    import torch
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    systems = [inputs.uniform(n, 3000 + n + k) for k in range(3)]
+    dev = [to_dev(xy, q) for xy, q in systems]
+    with binding.Plan(n, levels, p, 5.0, "fp64") as plan:
+        outs = {}
+        for streams in (3, 1):
+            binding.fmm_set_concurrency(plan.handle, streams)
+            phis = [torch.empty_like(q) for _, q in dev]
+            fields = [torch.empty_like(xy) for xy, _ in dev]
+            for (xy, q), phi, field in zip(dev, phis, fields):
+                plan.potential_field(xy, q, phi, field, sync=False)
+                plan.potential(xy, q, phi, sync=False)
+            plan.sync()
+            outs[streams] = [(a.cpu().numpy(), b.cpu().numpy()) for a, b in zip(phis, fields)]
+    for (xy, q), two, one in zip(systems, outs[3], outs[1]):
+        check_parity(two[0], oracle_mod.shiftfree(xy, q, levels, p), 1e-12, f"n={n} levels={levels}")
+        check_parity(two[0], one[0], 1e-12, "one stream against two")
+        check_parity(two[1].ravel(), one[1].ravel(), 1e-12, "field, one stream against two")
