@@ -302,7 +302,7 @@ int fmm_launch_scan(const uint32_t* counts, int64_t m, uint32_t* block_sums, uin
 // squares' items in the crowd list.
 int fmm_launch_leaf_blocks(const uint32_t* leaf_start, int64_t m, uint32_t block, uint32_t* nb, uint32_t* block_sums,
                            uint32_t* bstart, uint2* map, P2PCrowd crowd, cudaStream_t st);
-// targets per near-field block of the mixed path (the batched form uses 32)
+// targets per near-field block of a plan (the batched form takes 16 or 24, autotuned)
 #define FMM_P2P_BLOCK 24
 
 // largest i in [0, m) with pre[i] <= w, for a non-decreasing pre with pre[0] <= w: a 32-ary

@@ -340,7 +340,8 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 // the two-word differences.  A lane holds two sources, so that the targets' shared-memory broadcasts (8
 // wavefronts for two targets) serve four pairs.  200,000 charges in 3D, levels 3: 467 us against 739 us for
 // 64 targets over the lanes and a butterfly over the lanes per source tile (31 shuffles, 62 selects) for the
-// source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us.
+// source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us, and 198 with
+// the two changes below.
 // In 2D, with a few chunks an item, the warps of an SM are at many places of the unrolled code and wait for
 // instructions, so the code is kept small: the chunk itself and a last half chunk share a body, and whole
 // chunks are masked in every cell (the call 384 -> 366 us; in 3D, where one body runs for long, the call would
