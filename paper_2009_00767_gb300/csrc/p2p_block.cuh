@@ -240,12 +240,15 @@ __device__ __forceinline__ float2 p2p_near_sym(const float4* __restrict__ sp, co
 }
 
 // ---------------------------------------------------------------- crowded squares
-// The symmetric near field of squares above FMM_CROWD_POP particles (listed by the sort).  Each lane holds two sources, so that a target pair
-// read from shared memory serves four pairs and the independent work covers the latencies of the MUFU and
-// of the source loads; and the own square is taken once for both sides too: a block of up to kCrowdTargets
-// targets against itself one-sided, then its "later" sources -- the rest of the own square after the block,
-// masked at r^2 = 0, and the forward neighbours.  The sources of a large square's blocks are split into up
-// to kCrowdParts work items, so that a square of ten thousand particles does not end as one long tail.
+// The symmetric near field of squares above FMM_CROWD_POP particles (listed by the sort).  Each lane holds
+// two sources, so that a target pair read from shared memory serves four pairs and the independent work
+// covers the latencies of the MUFU and of the source loads; and the own square is taken once for both sides
+// too: a block of up to kCrowdTargets targets against itself one-sided, then its "later" sources -- the rest
+// of the own square after the block, masked at r^2 = 0, and the forward neighbours, whose pairs at r^2 = 0
+// count as r^2 = 2^-100 as above.  Own and forward sources share a chunk, so there the term is a source's
+// own: 0.5 ms of the call below, where one body masked them all alike (and gave 0 for such a forward pair).
+// The sources of a large square's blocks are split into up to kCrowdParts work items, so that a square of
+// ten thousand particles does not end as one long tail.
 // What bounds it: the MUFU, one lg2 a pair (16 a clock and SM), with the FMA pipe (6 packed instructions
 // of two cycles for two pairs) and issue close behind.
 // 2^24 clustered particles (32 Gaussians, levels 10, 2.1e11 ordered pairs): 28.5 ms against 33.5 ms for blocks
@@ -259,17 +262,18 @@ struct P2PCrowdShared {
     int4 seg[5];   // ranges of later sources: {sorted index minus slot, frame shift x, y, first slot past it}
 };
 
-// two sources of the lane against the NP target pairs, both sides; pairs at r^2 = 0 give 0 with kMask.
-// Returns the sources' sums.
+// two sources of the lane against the NP target pairs, both sides.  kMask: a source of the own square has
+// tiny = 0, so that a pair at r^2 = 0 gives 0; else every tiny is 2^-100.  Returns the sources' sums.
 template <bool kMask, int NP>
 __device__ __forceinline__ float2 p2p_chunk_sym2(float2 (&part)[NP], const float4* __restrict__ tg,
-                                                 const float2* __restrict__ tq, float4 a, float4 b) {
+                                                 const float2* __restrict__ tq, float4 a, float4 b, float tiny_a,
+                                                 float tiny_b) {
     const float2 ax = make_float2(-a.x, -a.x), ay = make_float2(-a.y, -a.y), aq = make_float2(a.z, a.z);
     const float2 bx = make_float2(-b.x, -b.x), by = make_float2(-b.y, -b.y), bq = make_float2(b.z, b.z);
-    const float2 tiny = make_float2(0x1p-100f, 0x1p-100f);
     float2 sa = make_float2(0.f, 0.f), sb = make_float2(0.f, 0.f);
-    auto log2_r2 = [&](float2 dx, float2 dy) {
-        const float2 r2 = __ffma2_rn(dx, dx, kMask ? __fmul2_rn(dy, dy) : __ffma2_rn(dy, dy, tiny));
+    auto log2_r2 = [&](float2 dx, float2 dy, float tiny) {
+        if (!kMask) tiny = 0x1p-100f;
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, make_float2(tiny, tiny)));
         float2 lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
         if (kMask) {
             lg.x = r2.x > 0.f ? lg.x : 0.f;
@@ -281,8 +285,8 @@ __device__ __forceinline__ float2 p2p_chunk_sym2(float2 (&part)[NP], const float
     for (int tp = 0; tp < NP; ++tp) {
         const float4 t = tg[tp];
         const float2 q = tq[tp], tx = make_float2(t.x, t.y), ty = make_float2(t.z, t.w);
-        const float2 la = log2_r2(__fadd2_rn(tx, ax), __fadd2_rn(ty, ay));
-        const float2 lb = log2_r2(__fadd2_rn(tx, bx), __fadd2_rn(ty, by));
+        const float2 la = log2_r2(__fadd2_rn(tx, ax), __fadd2_rn(ty, ay), tiny_a);
+        const float2 lb = log2_r2(__fadd2_rn(tx, bx), __fadd2_rn(ty, by), tiny_b);
         part[tp] = __ffma2_rn(bq, lb, __ffma2_rn(aq, la, part[tp]));
         sa = __ffma2_rn(q, la, sa);
         sb = __ffma2_rn(q, lb, sb);
@@ -322,8 +326,10 @@ __device__ __forceinline__ void p2p_crowd_item(const float4* __restrict__ sp, ui
     for (uint32_t c = c0; c < c1; c += 64u) {
         uint32_t na, nb;   // the next sources' loads are in flight meanwhile
         const float4 xa = load(c + 64u + (uint32_t)lane, &na), xb = load(c + 96u + (uint32_t)lane, &nb);
-        const float2 v = c < n_own ? p2p_chunk_sym2<true, NP>(part, sh.tg, sh.tq, a, b)
-                                   : p2p_chunk_sym2<false, NP>(part, sh.tg, sh.tq, a, b);
+        // a chunk may hold the last of the own square and the first of the forward ones
+        const float ta = c + (uint32_t)lane < n_own ? 0.f : 0x1p-100f, tb = c + 32u + (uint32_t)lane < n_own ? 0.f : 0x1p-100f;
+        const float2 v = c < n_own ? p2p_chunk_sym2<true, NP>(part, sh.tg, sh.tq, a, b, ta, tb)
+                                   : p2p_chunk_sym2<false, NP>(part, sh.tg, sh.tq, a, b, ta, tb);
         if (ia != 0xffffffffu) atomicAdd(acc + ia, fmm_f2d_bits(v.x));
         if (ib != 0xffffffffu) atomicAdd(acc + ib, fmm_f2d_bits(v.y));
         a = xa;

@@ -332,3 +332,25 @@ def test_crowded_squares(n, lev):
     cell = np.minimum((xy * 2 ** lev / 4.0).astype(int), 2 ** lev - 1)
     cnt = np.bincount(cell[:, 0] + 2 ** lev * cell[:, 1])
     assert st["p2p_pairs"] == n * (n - 1) and st["max_leaf"] == int(cnt.max())
+
+
+@pytest.mark.parametrize("n_a,n_b", [(65, 40), (100, 100), (128, 70), (200, 3)])
+def test_crowded_squares_pairs_across_an_edge(oracle_mod, n_a, n_b):
+    """Particles 2^-40 either side of an edge share one FP32 point of the target square's frame.  Such a pair is
+    taken at r^2 = 2^-100 (near field header), wherever its source falls among the square's chunks.  Box of side 4,
+    levels 1, the other coordinate on a grid of 2^-20: rounding as in test_crowded_squares."""
+    from gpu_util import run_fmm
+    rng = np.random.default_rng(8600 + n_a + n_b)
+    k = min(n_a, n_b)
+    y = np.round(rng.choice(1 << 20, size=n_a + n_b, replace=False) * 1.5) / 2.0 ** 20
+    xy = np.stack((np.concatenate((np.full(n_a, 2.0 - 2.0 ** -40), np.full(n_b, 2.0 + 2.0 ** -40))), y), 1)
+    xy[n_a:n_a + k, 1] = xy[:k, 1]   # the pairs
+    q = np.where(rng.random(n_a + n_b) < 0.5, -1.0, 1.0)
+    phi, _ = run_fmm(xy, q, 1, 8, "fp32", box=4.0)
+    ref = oracle_mod.direct(xy, q)
+    shift = -50.0 * np.log(2.0) - np.log(2.0 ** -39)   # of log r for a pair
+    ref[:k] += q[n_a:n_a + k] * shift
+    ref[n_a:n_a + k] += q[:k] * shift
+    d = np.hypot(xy[:, None, 0] - xy[None, :, 0], xy[:, None, 1] - xy[None, :, 1])
+    tol = 2.0 ** -20 * ((np.abs(np.log(np.where(d > 0, d, 1.0))) + 1.0) @ np.abs(q) + 10.0)
+    assert np.all(np.abs(phi - ref) <= tol), f"largest {np.max(np.abs(phi - ref)):.3g}"
