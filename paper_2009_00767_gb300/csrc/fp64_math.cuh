@@ -55,7 +55,9 @@ __device__ __forceinline__ double fmm_log(double x, const double2* __restrict__ 
     return fma(r, s, fma(ed, 0.69314718055994530942, t.y));
 }
 
-// 1 / x for a normal x: the MUFU's start y0, good to about 20 bits, then y0 (1 + e + e^2) with e = 1 - x y0, the series of 1 / (1 - e) up to a remainder of e^3 < 2^-57.
+// 1 / x for a normal x below 2^1022 (the MUFU flushes a subnormal result): the MUFU's start y0, good to about 20
+// bits, then y0 (1 + e + e^2) with e = 1 - x y0, the series of 1 / (1 - e) up to a remainder of e^3 < 2^-57.
+__device__ __forceinline__ bool fmm_rcp_range(double x) { return (unsigned)__double2hiint(x) - 0x00100000u < 0x7fc00000u; }
 __device__ __forceinline__ double fmm_rcp(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

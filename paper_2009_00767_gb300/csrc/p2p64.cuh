@@ -44,11 +44,11 @@ __device__ __forceinline__ void p2p64_pair(P64Acc<kField>& a, P64Shared<D, kFiel
         const double dz = sh.tgt[2][t] - s.z;
         r2 = fma(dz, dz, r2);
     }
-    const bool normal = (unsigned)__double2hiint(r2) - 0x00100000u < 0x7fe00000u;
     double k;   // a coincident pair gives 0
     if constexpr (D == 2) {
         k = fmm_log(r2, tab);
     } else {
+        const bool normal = (unsigned)__double2hiint(r2) - 0x00100000u < 0x7fe00000u;
         k = normal ? fmm_rsqrt(r2) : (r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0);
     }
     double* v = sh.rows[row + t];
@@ -56,7 +56,7 @@ __device__ __forceinline__ void p2p64_pair(P64Acc<kField>& a, P64Shared<D, kFiel
     const double tq = sh.tgt[D][t];
     a.phi = fma(tq, k, a.phi);
     if constexpr (kField) {
-        const double iv = normal ? fmm_rcp(r2) : (r2 > 0.0 ? 1.0 / r2 : 0.0);
+        const double iv = fmm_rcp_range(r2) ? fmm_rcp(r2) : (r2 > 0.0 ? 1.0 / r2 : 0.0);
         const double wx = dx * iv, wy = dy * iv;
         v[1] = fma(s.q, wx, v[1]);
         v[2] = fma(s.q, wy, v[2]);

@@ -1,6 +1,6 @@
-"""The FP64 near fields' log and reciprocal square root (fp64_math.cuh), one value at a time.
+"""The FP64 near fields' log, reciprocal and reciprocal square root (fp64_math.cuh), one value at a time.
 
-One unit charge at the origin and zero charges at (x, 0) in a tree of one cell: the potential at x
+One unit charge at the origin and zero charges at (x, 0) in a tree of one cell: the potential (or the field) at x
 is the function of the one distance alone, as every other pair adds a zero.  Distances: all exponents, 1 +- 2^-k,
 both ends and the centre of every interval of the logarithm's table, random ones about 1, and r^2 at the ends of
 the normal range and below it.  The reference is the function of fl(x^2) in extended precision.
@@ -63,6 +63,31 @@ def test_log(case):
     with binding.Plan(q.size, 0, 4, BOX, "fp64") as plan:
         phi = plan.potential(txy, tq).cpu().numpy()[1:]
     check(phi, 0.5 * np.log(r2), 4, f"log, {case}")
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_reciprocal(case):
+    """x fl(1 / r^2): 1 / r^2 within one unit and the product's rounding, so within 2 units of a value up to twice
+    the spacing: 4.  A subnormal 1 / r^2 has no more than its own spacing."""
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    x, r2, pos, q = system(case, 2)
+    # 1 / r^2 overflows below 2^-1022; zero charges that are as close to each other would add 0 times infinity, so
+    # the smallest distances come one to a call
+    keep = r2 >= np.longdouble(2.0) ** -1022
+    together = np.concatenate(([True], x >= 2.0 ** -450))
+    e = np.zeros(x.size)
+    with binding.Plan(int(together.sum()), 0, 4, BOX, "fp64") as plan:
+        _, field = plan.potential_field(*to_dev(pos[together], q[together]))
+    e[together[1:]] = -field.cpu().numpy()[1:, 0]
+    with binding.Plan(2, 0, 4, BOX, "fp64") as plan:
+        for i in np.flatnonzero(keep & ~together[1:]):
+            _, field = plan.potential_field(*to_dev(pos[[0, i + 1]], q[[0, i + 1]]))
+            e[i] = -field.cpu().numpy()[1, 0]
+    ref = x.astype(np.longdouble) / r2
+    slack = np.where(r2 > np.longdouble(2.0) ** 1022, x.astype(np.longdouble) * np.longdouble(2.0) ** -1074, 0.0)
+    near = np.clip(e.astype(np.longdouble), ref - slack, ref + slack)   # the nearest value that is allowed exactly
+    check(e[keep], near[keep], 4, f"reciprocal, {case}")
 
 
 @pytest.mark.parametrize("case", CASES)
