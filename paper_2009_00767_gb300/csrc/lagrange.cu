@@ -90,9 +90,8 @@ __host__ __device__ inline double kernel64(int D, double r2) {
 
 constexpr unsigned kFlagOutOfBox = 1u, kFlagNonFinite = 2u;
 
-// The MUFU reciprocal square root with subnormal inputs flushed to zero: a near-field r^2 is never
-// subnormal (coincident pairs give exactly 0, which maps to an infinity that the own cell's mask
-// removes), so the subnormal handling of rsqrtf is dead weight in the pair loop.
+// The MUFU reciprocal square root, which takes a subnormal input for zero: no r^2 that counts is subnormal (the
+// own cell's mask drops those, a forward pair has its tiny), so rsqrtf's handling of them is not needed.
 __device__ __forceinline__ float mufu_rsqrt(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -332,9 +331,11 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 // lane; the targets' coordinates and charges are shared-memory broadcasts, and two targets' arithmetic
 // runs in packed FP32x2.  A pair's 1/r (or log r) feeds a register partial of the target and the sum of the
 // source, which stays in its lane and goes out with one FP64 atomic.  The chunk
-// against itself is one-sided.  Pairs inside A are masked at r = 0 (only there can a pair coincide).
-// Differences come from two-word coordinates, (hi_t - hi_s) + (lo_t - lo_s), so a close pair's distance
-// keeps about 48 bits.  After kP2PRun chunks the lanes' partials of a target are summed across the warp
+// against itself is one-sided.  Differences come from two-word coordinates, (hi_t - hi_s) + (lo_t - lo_s), so a
+// close pair's distance keeps about 48 bits.  Pairs inside A below r^2 = 2^-126, FP32's smallest normal number,
+// count as coincident and give 0.  Two charges either side of a cell's edge may share one two-word point: the
+// pairs with the forward cells add tiny = (2^-50 box)^2 to r^2, which moves no pair that the words tell apart
+// by more than their own rounding (1.4% of 200,000 charges' call in 3D; a maximum with tiny instead 5%).  After kP2PRun chunks the lanes' partials of a target are summed across the warp
 // (warp_reduce_scatter) and added in FP64.
 // What bounds it: the FMA pipe, 14 packed instructions (two cycles each) for two targets in 3D, 9 of them
 // the two-word differences.  A lane holds two sources, so that the targets' shared-memory broadcasts (8
@@ -417,11 +418,11 @@ struct LagTargets {
     float2 lz[D == 3 ? kWarpChunk / 2 : 1];
 };
 
-// A lane's source, its coordinates negated and duplicated: {-x, -x} (high and low words), {q, q}.
+// A lane's source, its coordinates negated and duplicated: {-x, -x} (high and low words), {q, q}, {tiny, tiny}.
 template <int D>
 struct LagSource {
-    float2 x[D], l[D], q;
-    __device__ LagSource(float4 h, float4 lo) {
+    float2 x[D], l[D], q, tiny;
+    __device__ LagSource(float4 h, float4 lo, float2 t) {
         x[0] = make_float2(-h.x, -h.x);
         x[1] = make_float2(-h.y, -h.y);
         l[0] = make_float2(-lo.x, -lo.x);
@@ -431,23 +432,24 @@ struct LagSource {
             l[2] = make_float2(-lo.z, -lo.z);
         }
         q = make_float2(h.w, h.w);
+        tiny = t;
     }
 };
 
-// 1 / r (3D) or log2 r^2 (2D) of the lane's source and target pair t; kMask: 0 for a coincident pair
+// 1 / r (3D) or log2 r^2 (2D) of the lane's source and target pair t; kMask: 0 for a coincident pair (tiny = 0)
 template <int D, bool kMask>
 __device__ __forceinline__ float2 p2p_lag_pair(const LagSource<D>& s, float4 A, float4 B, float4 C, float2 lz) {
     const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), s.x[0]), __fadd2_rn(make_float2(C.x, C.y), s.l[0]));
     const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), s.x[1]), __fadd2_rn(make_float2(C.z, C.w), s.l[1]));
-    float2 r2 = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+    float2 r2 = __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, s.tiny));
     if constexpr (D == 3) {
         const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), s.x[2]), __fadd2_rn(lz, s.l[2]));
         r2 = __ffma2_rn(dz, dz, r2);
     }
     float2 k = D == 3 ? make_float2(mufu_rsqrt(r2.x), mufu_rsqrt(r2.y)) : make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
     if constexpr (kMask) {
-        k.x = r2.x > 0.f ? k.x : 0.f;
-        k.y = r2.y > 0.f ? k.y : 0.f;
+        k.x = r2.x >= 0x1p-126f ? k.x : 0.f;
+        k.y = r2.y >= 0x1p-126f ? k.y : 0.f;
     }
     return k;
 }
@@ -455,8 +457,8 @@ __device__ __forceinline__ float2 p2p_lag_pair(const LagSource<D>& s, float4 A, 
 // the lane's kS sources (1 or 2) against the chunk's 2 NP targets; returns the sources' sums
 template <int D, bool kMask, int NP, int kS>
 __device__ __forceinline__ float2 p2p_lag_chunk(float2 (&part)[NP], const LagTargets<D>& tg, float4 ha, float4 la,
-                                                float4 hb, float4 lb) {
-    const LagSource<D> a(ha, la), b(hb, lb);
+                                                float4 hb, float4 lb, float2 ta, float2 tb) {
+    const LagSource<D> a(ha, la, ta), b(hb, lb, tb);
     float2 sa = make_float2(0.f, 0.f), sb = make_float2(0.f, 0.f);
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
@@ -478,10 +480,11 @@ __device__ __forceinline__ float2 p2p_lag_chunk(float2 (&part)[NP], const LagTar
 template <int D, int NP>
 __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, const float4* __restrict__ lo, int t0,
                                                int T, bool self, const uint32_t (&first)[5], const uint32_t (&end)[5],
-                                               uint32_t n_own, const LagTargets<D>& tg, float far, int lane,
-                                               double* __restrict__ nearf) {
+                                               uint32_t n_own, const LagTargets<D>& tg, float far, float2 tiny,
+                                               int lane, double* __restrict__ nearf) {
     constexpr int W = NP <= 2 ? 4 : (NP <= 4 ? 8 : (NP <= 8 ? 16 : 32));
     const float4 far4 = make_float4(far, far, far, 0.f), zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float2 none = make_float2(0.f, 0.f);
     float2 part[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
@@ -509,7 +512,7 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
     if (D == 3 && self) {
         float4 h, l;
         load_own(h, l);
-        p2p_lag_chunk<D, true, NP, 1>(part, tg, h, l, far4, zero4);
+        p2p_lag_chunk<D, true, NP, 1>(part, tg, h, l, far4, zero4, none, none);
     }
     int run = 0;
 #pragma unroll 1
@@ -522,11 +525,13 @@ __device__ __forceinline__ double p2p_lag_item(const float4* __restrict__ hi, co
             load((uint32_t)(c + lane), ha, la, ia);
             load((uint32_t)(c + 32 + lane), hb, lb, ib);
         }
+        // a masked chunk may hold sources of the own cell and of forward ones
+        const float ta = own(c) || (uint32_t)(c + lane) < n_own ? 0.f : tiny.x, tb = (uint32_t)(c + 32 + lane) < n_own ? 0.f : tiny.x;
         const float2 v = own(c) || c + 32 >= (int)nsrc   // a last half chunk
-                             ? p2p_lag_chunk<D, true, NP, 1>(part, tg, ha, la, hb, lb)
-                         : D == 2 || (uint32_t)c < n_own   // masked, which is right for every pair
-                             ? p2p_lag_chunk<D, true, NP, 2>(part, tg, ha, la, hb, lb)
-                             : p2p_lag_chunk<D, false, NP, 2>(part, tg, ha, la, hb, lb);
+                             ? p2p_lag_chunk<D, true, NP, 1>(part, tg, ha, la, hb, lb, make_float2(ta, ta), make_float2(tb, tb))
+                         : D == 2 || (uint32_t)c < n_own
+                             ? p2p_lag_chunk<D, true, NP, 2>(part, tg, ha, la, hb, lb, make_float2(ta, ta), make_float2(tb, tb))
+                             : p2p_lag_chunk<D, false, NP, 2>(part, tg, ha, la, hb, lb, tiny, tiny);
         if (ia != 0xffffffffu) atomicAdd(nearf + ia, f2d(v.x));
         if (ib != 0xffffffffu) atomicAdd(nearf + ib, f2d(v.y));
         run += 2;
@@ -547,8 +552,7 @@ template <int D>
 __global__ void __launch_bounds__(kP2PWarps * 32, 5)
 k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int* __restrict__ start,
         const int* __restrict__ wchunk_start, const int* __restrict__ wchunk_cell, int nleaf, int L, float box,
-        double* __restrict__ nearf,
-        unsigned long long* __restrict__ pairs) {
+        float2 tiny, double* __restrict__ nearf, unsigned long long* __restrict__ pairs) {
     constexpr int F = D == 3 ? 14 : 5, FG = fwd_group<D>(), G = (F + FG - 1) / FG;
     __shared__ LagTargets<D> tgts[kP2PWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -556,6 +560,8 @@ k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int*
     const int side = 1 << L;
     // empty source and target slots are zero charges outside the box, away from every charge and each other
     const float src_far = -0.25f * box, tgt_far = 1.25f * box;
+    // from the constant bank where registers are short (3D); in 2D a register: 352 us for 2^20 charges against 355
+    const float2 term = D == 2 ? make_float2(fmaxf((0x1p-50f * box) * (0x1p-50f * box), 0x1p-126f), 0.f) : tiny;
     const int64_t w = (int64_t)blockIdx.x * kP2PWarps + wid;
     if (w >= (int64_t)wchunk_start[nleaf] * G) return;
     const int cidx = (int)(w / G), g = (int)(w % G);
@@ -585,9 +591,9 @@ k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int*
     double acc;
     const bool self = g == 0;
     switch ((T + 7) >> 3) {   // the chunk's target pairs, rounded up to a multiple of four
-        case 1: acc = p2p_lag_item<D, 4>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-        case 2: acc = p2p_lag_item<D, 8>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
-        default: acc = p2p_lag_item<D, 12>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, lane, nearf); break;
+        case 1: acc = p2p_lag_item<D, 4>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, term, lane, nearf); break;
+        case 2: acc = p2p_lag_item<D, 8>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, term, lane, nearf); break;
+        default: acc = p2p_lag_item<D, 12>(hi, lo, t0, T, self, first, end, n_own, tg, src_far, term, lane, nearf); break;
     }
     if (lane < T) atomicAdd(nearf + t0 + lane, acc);
 }
@@ -1474,9 +1480,10 @@ fmm_status enqueue(fmm_lag_plan_s* pl, const double* pos, const double* q, int64
         // a chunk per kWarpChunk charges and a partial one per occupied cell at most
         constexpr int F = D == 3 ? 14 : 5, G = (F + fwd_group<D>() - 1) / fwd_group<D>();
         const int64_t items = (std::min<int64_t>(pl->nleaf, n) + n / kWarpChunk) * G;
+        const float apart = 0x1p-50f * (float)pl->box, tiny = std::max(apart * apart, 0x1p-126f);
         k_p2p32<D><<<(unsigned)((items + kP2PWarps - 1) / kP2PWarps), kP2PWarps * 32, 0, st>>>(
-            pl->hi, pl->lo, pl->start, pl->wchunk_start, pl->wchunk_cell, (int)pl->nleaf, L, (float)pl->box, pl->nearf,
-            pl->pairs);
+            pl->hi, pl->lo, pl->start, pl->wchunk_start, pl->wchunk_cell, (int)pl->nleaf, L, (float)pl->box,
+            make_float2(tiny, tiny), pl->nearf, pl->pairs);
     }
     ++launches;
     cudaEventRecord(pl->ev[6], st);

@@ -247,3 +247,48 @@ def test_binning_with_few_cells(oracle_mod, form, tol, dim, levels, n):
     phi, _, cells = run(pos, q, levels, form)
     assert np.array_equal(cells, oracle_mod.lag_cells(pos, levels))
     check_parity(phi, oracle_mod.lag_node(pos, q, levels), tol, f"{form} D={dim} L={levels} n={n}")
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_f32_near_pairs_below_the_normal_range(dim):
+    """Charges of one cell whose r^2 is subnormal in FP32 or underflows count as coincident (0); every other pair
+    is itself.  The bound is that of an FP32 term (2^-20) on the sum of the terms' magnitudes."""
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    rng = np.random.default_rng(8800 + dim)
+    pos = rng.random((90, dim))
+    pos[:4] = 0.0
+    pos[1, 0], pos[2, 0], pos[3, dim - 1] = 1e-20, 3e-20, 1e-30
+    q = np.where(rng.random(90) < 0.5, -1.0, 1.0)
+    r = np.sqrt(((pos[:, None] - pos[None]) ** 2).sum(-1))
+    r[:4, :4] = 0.0
+    k = np.where(r > 0, np.log(np.where(r > 0, r, 1.0)) if dim == 2 else 1.0 / np.where(r > 0, r, 1.0), 0.0)
+    with binding.LagPlan(dim, 90, 0, 1.0, "node_f32") as plan:
+        phi = plan.potential(*to_dev(pos, q)).cpu().numpy()
+    assert np.all(np.abs(phi - k @ q) <= 2.0 ** -20 * (np.abs(k) + 1.0) @ np.abs(q))
+
+
+@pytest.mark.parametrize("n_a,n_b", [(10, 10), (40, 100), (100, 100), (200, 30)])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_f32_near_pairs_across_an_edge(dim, n_a, n_b):
+    """Charges a unit in the last place either side of an edge that no FP32 pair tells apart: the pair counts as
+    2^-50 of the box apart, wherever its source falls among the cell's chunks.  Bound as above."""
+    from gpu_util import to_dev
+    from paper_2009_00767_gb300 import binding
+    box, n, k = 3.7, n_a + n_b, min(n_a, n_b)
+    x1 = 1.85
+    while np.floor(x1 * 2.0 / box) >= 1.0:
+        x1 = np.nextafter(x1, 0.0)
+    x0 = np.nextafter(x1, 4.0)
+    rng = np.random.default_rng(8900 + n)
+    pos = np.zeros((n, dim))
+    pos[:, 0] = np.where(np.arange(n) < n_a, x1, x0)
+    pos[:, 1] = rng.choice(1 << 16, size=n, replace=False) / 2.0 ** 16   # exact in FP32, 2^-16 or more apart
+    pos[n_a:n_a + k, 1] = pos[:k, 1]
+    q = np.where(rng.random(n) < 0.5, -1.0, 1.0)
+    r = np.abs(pos[:, None, 1] - pos[None, :, 1])
+    r[np.arange(k), n_a + np.arange(k)] = r[n_a + np.arange(k), np.arange(k)] = box * 2.0 ** -50
+    kern = np.where(r > 0, np.log(np.where(r > 0, r, 1.0)) if dim == 2 else 1.0 / np.where(r > 0, r, 1.0), 0.0)
+    with binding.LagPlan(dim, n, 1, box, "node_f32") as plan:
+        phi = plan.potential(*to_dev(pos, q)).cpu().numpy()
+    assert np.all(np.abs(phi - kern @ q) <= 2.0 ** -20 * (np.abs(kern) + 1.0) @ np.abs(q))
