@@ -816,10 +816,15 @@ k_p2p_field(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
     if (*(volatile const unsigned int*)status != 0u) return;
     const uint32_t leaf = lt.x;
     const uint32_t t0 = leaf_start[leaf], t1 = leaf_start[leaf + 1];
-    // a square's blocks are of (almost) equal size
+    // a square's blocks are of (almost) equal size; the division only where there are several, as a block of few
+    // targets has little else to do (2^20 particles at four a square of level 9: 341 us, 354 with it, 377 in 64 bits)
     const uint32_t pop = t1 - t0, nblk = (pop + FMM_P2P_BLOCK - 1) / FMM_P2P_BLOCK;
-    const uint32_t b0 = t0 + (uint32_t)((uint64_t)pop * lt.y / nblk);
-    const int T = (int)(t0 + (uint32_t)((uint64_t)pop * (lt.y + 1) / nblk) - b0);
+    uint32_t b0 = t0, T = pop;
+    if (nblk > 1u) {
+        const uint32_t size = pop / nblk, more = pop - size * nblk;   // the first `more` blocks have one target more
+        b0 = t0 + lt.y * size + min(lt.y, more);
+        T = size + (lt.y < more ? 1u : 0u);
+    }
     uint32_t pairs;
     const NearField nf = p2p_near_sym_field(sp, lo, leaf_start, leaf, t0, t1, b0, T, levels, s_leaf, tgt[warp],
                                             tlo[warp], tq[warp], seg[warp], lane, acc, accg, &pairs);

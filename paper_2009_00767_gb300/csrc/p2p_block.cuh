@@ -402,10 +402,11 @@ __device__ __forceinline__ unsigned long long p2p_near_crowd(const float4* __res
 // also carries its FP32 rounding residue (written by the sort for field calls), and a pair's
 // difference takes the high words (exact for close pairs) plus the residues' difference.
 // What bounds it: instruction fetch first.  The loop over the target pairs is unrolled, so each instance for a
-// number of pairs is up to 7 kB; one body for both kinds of chunk and three instances instead of six of two
-// bodies each keep the warps of an SM in the same code.  200,003 particles in a ring (levels 7): 60 us against 91,
+// number of pairs is up to 7 kB; one body for both kinds of chunk and four instances instead of six of two
+// bodies each keep the warps of an SM in the same code.  200,003 particles in a ring (levels 7): 62 us against 91,
 // where a warp waited six issue slots for an instruction (0.1 now); then the waits on registers' latencies, with
-// 16 warps an SM.
+// 16 warps an SM.  Uniform particles at level 8, the kernel alone: 56 us at one a square (56 with the six
+// instances), 72 at two (72), 85 at four (84), 113 at eight (129), 202 at 16 (353), 528 at 31 (817).
 struct NearField {
     float2 phi, gx, gy;   // float-float sums of target `lane`
 };
@@ -564,9 +565,13 @@ __device__ __forceinline__ NearField p2p_near_sym_field(const float4* __restrict
         reinterpret_cast<float*>(&tq[lane >> 1])[lane & 1] = q;
     }
     __syncwarp();
-    switch ((T + 7) >> 3) {
-        case 1: return p2p_block_sym_field<4>(S, lo, tgt, tlo, tq, lane, acc, accg);
-        case 2: return p2p_block_sym_field<8>(S, lo, tgt, tlo, tq, lane, acc, accg);
+    // squares of a few particles fill only the smallest instance: 2^18 particles at one a square of level 9, 206 us
+    // against 228 us without it; instances for 12 and 20 targets too would cost 344 us against 202 at 16 a square
+    switch ((T + 3) >> 2) {
+        case 1: return p2p_block_sym_field<2>(S, lo, tgt, tlo, tq, lane, acc, accg);
+        case 2: return p2p_block_sym_field<4>(S, lo, tgt, tlo, tq, lane, acc, accg);
+        case 3:
+        case 4: return p2p_block_sym_field<8>(S, lo, tgt, tlo, tq, lane, acc, accg);
         default: return p2p_block_sym_field<12>(S, lo, tgt, tlo, tq, lane, acc, accg);
     }
 }

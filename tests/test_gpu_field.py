@@ -103,3 +103,14 @@ def test_field_device_checks():
             binding.fmm_potential_field(plan.handle, txy, tq, phi, E)
             assert plan.sync(check=False) == binding.FMM_ERR_OUT_OF_BOX
             assert bool((phi == 3.0).all()) and bool((E == 4.0).all())
+
+
+@pytest.mark.parametrize("lev", [0, 1, 3])
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 8, 9, 16, 17, 24, 25, 26, 47, 48, 49, 73, 300])
+def test_mixed_field_block_sizes(oracle_mod, n, lev):
+    """Blocks of 1 to 24 targets, squares of one block and of several that do and do not divide evenly."""
+    xy, q = inputs.uniform(n, inputs.config_seed(0, 640 + n))
+    phi, E = _run(xy, q, lev, 28, "fp32")
+    ref_phi, ref_E = oracle_mod.shiftfree_field(xy, q, lev, 28)
+    check_parity(phi, ref_phi, 1e-6, f"fp32 phi with the field, N={n} levels={lev}")
+    check_parity(E, ref_E, FIELD_TOL, f"fp32 field N={n} levels={lev}")
