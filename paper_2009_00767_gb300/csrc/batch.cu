@@ -16,6 +16,7 @@
 // once into a CUDA graph; the call's array pointers live in a small device block written before
 // each replay, so one graph serves every call.  fmm_batch_autotune times candidate launch shapes
 // (persistent blocks per SM, tensor-core tiles per CTA, near-field targets per block).
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -489,20 +490,18 @@ __global__ void __launch_bounds__(kT, 8) kb_p2p(BatchArgs a, MixedLevels lv) {
     }
 }
 
-// The squares in the crowd list (p2p_near_crowd), their items taken from a counter by
-// resident warps.
+// The squares in the crowd list (p2p_near_crowd), their items after each warp's first taken from a
+// counter by resident warps.
 __global__ void __launch_bounds__(kT, kCrowdBlocksPerSm) kb_p2p_crowd(BatchArgs a) {
     extern __shared__ long long pre[];
     __shared__ __align__(16) P2PCrowdShared sh[kT / 32];
-    load_prefix(pre, a.wp_leaf, a.nsys);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long total = *a.crowd.count;
-    if (*(volatile const unsigned int*)a.status != 0u) return;   // inputs failed the device checks
-    for (;;) {
-        unsigned long long w = 0;
-        if (lane == 0) w = atomicAdd(a.crowd.count + 1, 1ull);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= total) return;
+    if (total == 0ull || *(volatile const unsigned int*)a.status != 0u) return;   // none, or the inputs failed the checks
+    load_prefix(pre, a.wp_leaf, a.nsys);
+    const unsigned long long warps = (unsigned long long)gridDim.x * (kT / 32);
+    for (unsigned long long w = (unsigned long long)blockIdx.x * (kT / 32) + warp; w < total;
+         w = warps + fmm_crowd_next(a.crowd, lane)) {
         const uint2 it = a.crowd.list[w];
         const int s = find_sys(pre, a.nsys, (long long)it.x);
         const BatchSys& S = a.sys[s];
@@ -514,6 +513,9 @@ __global__ void __launch_bounds__(kT, kCrowdBlocksPerSm) kb_p2p_crowd(BatchArgs 
 }
 
 }  // namespace
+
+// bytes of the populations, behind which crowd_count lies
+static size_t crowd_count_at(long long nl) { return (sizeof(uint32_t) * (size_t)nl + 7) & ~(size_t)7; }
 
 // ---------------------------------------------------------------- the batch plan
 struct fmm_batch_s {
@@ -536,7 +538,7 @@ struct fmm_batch_s {
     uint32_t *keys, *rank, *counts, *leaf_start, *block_sums, *sorted_key, *leaf_nb, *bstart;
     uint2* bmap;
     uint2* crowd_list;
-    unsigned long long* crowd_count;
+    unsigned long long* crowd_count;   // behind counts, cleared with them
     float4* sorted32;
     float2 *a32, *b32;
     double* acc;                      // near field per sorted particle
@@ -560,7 +562,7 @@ void batch_free(fmm_batch_s* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     void* bufs[] = {b->d_sys, b->d_pre, b->d_call, b->keys, b->rank, b->counts, b->leaf_start, b->block_sums,
-                    b->leaf_nb, b->bstart, b->bmap, b->crowd_list, b->crowd_count,
+                    b->leaf_nb, b->bstart, b->bmap, b->crowd_list,
                     b->sorted_key, b->sorted32, b->a32, b->b32, b->acc, b->T32, b->U32, b->d_status};
     fmm_tc_free(b->tc);
     for (void* p : bufs)
@@ -594,9 +596,9 @@ int enqueue_batch_kernels(fmm_batch_s* b, const BatchArgs& a, const MixedLevels&
     const unsigned grid = (unsigned)(sms * b->grid_mult);
     const size_t pre_bytes = sizeof(long long) * (b->nsys + 1);
     int launches = 0;
-    if (cudaMemsetAsync(b->counts, 0, sizeof(uint32_t) * b->nl, st) != cudaSuccess ||
-        cudaMemsetAsync(b->acc, 0, sizeof(double) * b->nt, st) != cudaSuccess ||
-        cudaMemsetAsync(b->crowd_count, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess)
+    // counts and, behind them, crowd_count
+    if (cudaMemsetAsync(b->counts, 0, crowd_count_at(b->nl) + 2 * sizeof(unsigned long long), st) != cudaSuccess ||
+        cudaMemsetAsync(b->acc, 0, sizeof(double) * b->nt, st) != cudaSuccess)
         return -1;
     kb_bin<<<grid, kT, pre_bytes, st>>>(a, lv);
     ++launches;
@@ -612,7 +614,8 @@ int enqueue_batch_kernels(fmm_batch_s* b, const BatchArgs& a, const MixedLevels&
                                           b->bstart, b->bmap, a.crowd, st2);
     if (lb < 0) return -1;
     kb_p2p<<<grid, kT, pre_bytes, st2>>>(a, lv);
-    kb_p2p_crowd<<<(unsigned)(sms * kCrowdBlocksPerSm), kT, pre_bytes, st2>>>(a);
+    const size_t most = (fmm_crowd_items(b->nt) + kT / 32 - 1) / (kT / 32);
+    kb_p2p_crowd<<<(unsigned)std::min<size_t>(most, (size_t)sms * kCrowdBlocksPerSm), kT, pre_bytes, st2>>>(a);
     launches += lb + 2;
     if (st2 != st && cudaEventRecord(ev_join, st2) != cudaSuccess) return -1;
     kb_p2m_fine<P1B><<<grid, kT, pre_bytes, st>>>(a, lv);
@@ -880,18 +883,19 @@ fmm_status fmm_batch_plan(fmm_batch_t* out, int nsys, const int64_t* n, const in
     b->b_cells = bcells;
     bool ok = balloc(b, &b->d_sys, sizeof(BatchSys) * nsys) && balloc(b, &b->d_pre, sizeof(long long) * pre.size()) &&
               balloc(b, &b->d_call, sizeof(BatchCall)) && balloc(b, &b->keys, 4 * nt) && balloc(b, &b->rank, 4 * nt) &&
-              balloc(b, &b->counts, 4 * nl) && balloc(b, &b->leaf_start, 4 * (nl + 1)) &&
+              balloc(b, &b->counts, crowd_count_at(nl) + 2 * sizeof(unsigned long long)) && balloc(b, &b->leaf_start, 4 * (nl + 1)) &&
               balloc(b, &b->block_sums, 4 * ((size_t)fmm_scan_blocks(nl) + 1)) && balloc(b, &b->sorted_key, 4 * nt) &&
               balloc(b, &b->leaf_nb, 4 * nl) && balloc(b, &b->bstart, 4 * (nl + 1)) &&
               balloc(b, &b->bmap, sizeof(uint2) * ((size_t)nl + (size_t)nt / kP2PBlockMin + 1)) &&
               balloc(b, &b->crowd_list, sizeof(uint2) * fmm_crowd_items(nt)) &&
-              balloc(b, &b->crowd_count, 2 * sizeof(unsigned long long)) && balloc(b, &b->sorted32, 16 * nt) &&
+              balloc(b, &b->sorted32, 16 * nt) &&
               balloc(b, &b->a32, sizeof(float2) * b->a_cells * p1) && balloc(b, &b->b32, sizeof(float2) * bcells * p1) &&
               balloc(b, &b->acc, sizeof(double) * nt) && balloc(b, &b->d_status, sizeof(unsigned int));
     if (!ok) {
         batch_free(b);
         return FMM_ERR_OOM;
     }
+    b->crowd_count = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(b->counts) + crowd_count_at(nl));
     // operators and the upward pass's tables: the plan's FP64 builds, rounded to FP32 in the padded
     // layouts of the FP32 kernels
     {

@@ -18,6 +18,8 @@
 //        FP32, plus Re b'_0; the levels are summed in float-float.
 //   P2P  (E-2 of Sec. 2.1) in FP32 on square-local coordinates, log via the MUFU lg2 unit,
 //        lanes over sources and one register partial per target; phi = far + near.
+#include <algorithm>
+
 #include "mixed_common.cuh"
 #include "p2p_block.cuh"
 
@@ -771,8 +773,8 @@ k_p2p_mixed(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
     if (lane < T) atomicAdd(acc + b0 + lane, fmm_f2d_bits(near.x) + fmm_f2d_bits(near.y));
 }
 
-// The squares that the sort put into the crowd list (p2p_near_crowd): resident warps take their items from
-// a counter, so that they finish within one item of each other whatever the squares' sizes.
+// The squares that the sort put into the crowd list (p2p_near_crowd): resident warps take their items after the
+// first from a counter, so that they finish within one item of each other whatever the squares' sizes.
 __global__ void __launch_bounds__(kP2PWarps * 32, kCrowdBlocksPerSm)
 k_p2p_crowd(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_start, int levels, float s_leaf,
             double* __restrict__ acc, P2PCrowd crowd, const unsigned int* __restrict__ status,
@@ -781,11 +783,9 @@ k_p2p_crowd(const float4* __restrict__ sp, const uint32_t* __restrict__ leaf_sta
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long total = *crowd.count;
     if (total == 0ull || *(volatile const unsigned int*)status != 0u) return;   // none, or the inputs failed the checks
-    for (;;) {
-        unsigned long long w = 0;
-        if (lane == 0) w = atomicAdd(crowd.count + 1, 1ull);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= total) return;
+    const unsigned long long warps = (unsigned long long)gridDim.x * kP2PWarps;
+    for (unsigned long long w = (unsigned long long)blockIdx.x * kP2PWarps + warp; w < total;
+         w = warps + fmm_crowd_next(crowd, lane)) {
         const uint2 it = crowd.list[w];
         const uint32_t t0 = leaf_start[it.x], t1 = leaf_start[it.x + 1];
         const unsigned long long pairs =
@@ -871,7 +871,8 @@ int fmm_launch_p2p_concurrent(fmm_plan_s* pl, const MixedLevels& lv, bool with_f
         const P2PCrowd crowd = {pl->d_counters + 2 * FMM_COUNTER_SLOTS, pl->crowd_list};
         k_p2p_mixed<<<blocks, kP2PWarps * 32, 0, s2>>>(pl->sorted32, pl->leaf_start, pl->leaf_bstart, pl->blk_map,
                                                       nleaf, L, lv.s_leaf, pl->phi_far, pl->d_status, pl->d_counters);
-        k_p2p_crowd<<<(unsigned)(pl->sms * kCrowdBlocksPerSm), kP2PWarps * 32, 0, s2>>>(
+        const size_t most = (fmm_crowd_items(pl->n) + kP2PWarps - 1) / kP2PWarps;
+        k_p2p_crowd<<<(unsigned)std::min<size_t>(most, (size_t)pl->sms * kCrowdBlocksPerSm), kP2PWarps * 32, 0, s2>>>(
             pl->sorted32, pl->leaf_start, L, lv.s_leaf, pl->phi_far, crowd, pl->d_status, pl->d_counters);
     }
     cudaEventRecord(pl->ev[9], s2);
