@@ -280,11 +280,19 @@ __host__ __device__ inline uint32_t fmm_crowd_parts(uint32_t n) {
     const uint32_t p = (n + kCrowdPart - 1) / kCrowdPart;
     return p < (uint32_t)kCrowdParts ? p : (uint32_t)kCrowdParts;
 }
-// square `id` of n particles into the list
+// The warp's crowded squares into the list: square `id` of n particles on each lane (n = 0: none).  All lanes write
+// a square's items, which the near field waits for.
 static __device__ __forceinline__ void fmm_crowd_add(P2PCrowd c, uint32_t id, uint32_t n) {
-    const uint32_t items = fmm_crowd_blocks(n) * fmm_crowd_parts(n);
-    const unsigned long long at = atomicAdd(c.count, (unsigned long long)items);
-    for (uint32_t i = 0; i < items; ++i) c.list[at + i] = make_uint2(id, i);
+    const int lane = threadIdx.x & 31;
+    for (unsigned m = __ballot_sync(0xffffffffu, n > (uint32_t)FMM_CROWD_POP); m; m &= m - 1u) {
+        const int src = __ffs(m) - 1;
+        const uint32_t sq = __shfl_sync(0xffffffffu, id, src), pop = __shfl_sync(0xffffffffu, n, src);
+        const uint32_t items = fmm_crowd_blocks(pop) * fmm_crowd_parts(pop);
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(c.count, (unsigned long long)items);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        for (uint32_t i = (uint32_t)lane; i < items; i += 32u) c.list[at + i] = make_uint2(sq, i);
+    }
 }
 // the next item after every warp's first, which is its index: with few items the other warps need no atomic (a
 // batch of 16 systems of 300 particles in 4 squares each: 64 us a call, 74 with all from the counter)

@@ -188,7 +188,7 @@ __global__ void k_scan2_down(uint32_t* __restrict__ in, int64_t m, const unsigne
         v[j] = (base + j < m) ? pop_blocks(in[base + j]) : 0ull;
         nbk[j] = (uint32_t)(v[j] >> 32);
         crowded |= (uint32_t)v[j] > (uint32_t)FMM_LANE_MAX;
-        if ((uint32_t)v[j] > (uint32_t)FMM_CROWD_POP && crowd.list) fmm_crowd_add(crowd, (uint32_t)(base + j), (uint32_t)v[j]);
+        if (crowd.list) fmm_crowd_add(crowd, (uint32_t)(base + j), (uint32_t)v[j]);
         if (base + j < m) in[base + j] = 0u;   // the populations start the next call at zero
     }
     if (crowded && crowd_hint) *(volatile int*)crowd_hint = 1;
@@ -285,8 +285,8 @@ int fmm_launch_sort(fmm_plan_s* pl, const double* xy, const double* q, bool with
     const int nb = pl->scan_blocks;
     {
         // the near-field blocks come with the same scan (block_sums holds 64-bit partials), and in the mixed
-        // path the crowded squares' items
-        const P2PCrowd crowd = {pl->d_counters + 2 * FMM_COUNTER_SLOTS, pl->crowd_list};
+        // path the crowded squares' items (the field's near field does not use them)
+        const P2PCrowd crowd = {pl->d_counters + 2 * FMM_COUNTER_SLOTS, with_lo ? nullptr : pl->crowd_list};
         unsigned long long* sums = reinterpret_cast<unsigned long long*>(pl->block_sums);
         k_scan2_reduce<<<nb, kScanThreads, 0, st>>>(pl->counts, m, sums);
         if (nb <= kLocalTopMax) {
@@ -329,9 +329,8 @@ __global__ void k_leaf_blocks(const uint32_t* __restrict__ leaf_start, int64_t m
 __global__ void k_block_map(const uint32_t* __restrict__ bstart, const uint32_t* __restrict__ leaf_start, int64_t m,
                             uint2* __restrict__ map, P2PCrowd crowd) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    fmm_crowd_add(crowd, (uint32_t)i, i < m ? leaf_start[i + 1] - leaf_start[i] : 0u);
     if (i >= m) return;
-    const uint32_t n = leaf_start[i + 1] - leaf_start[i];
-    if (n > (uint32_t)FMM_CROWD_POP) fmm_crowd_add(crowd, (uint32_t)i, n);
     const uint32_t b0 = bstart[i], b1 = bstart[i + 1];
     for (uint32_t b = b0; b < b1; ++b) map[b] = make_uint2((uint32_t)i, b - b0);
 }
