@@ -502,6 +502,7 @@ fmm_status fmm_potential_host_async(fmm_plan_t plan, const double* xy_host, cons
         // Plan's stream: the rest of the method once the uploads are in (and, before L2P writes this
         // set's phi, once the call two back has downloaded it).  Download stream: phi, after L2P.
         cudaStream_t up = plan->s_up, down = plan->s_down;
+        plan->host_pending = 1;   // also where a later step fails: fmm_sync waits for what was enqueued
         // the plan's first host call waits for all of the device-array calls before it, not for their sorts
         if (!plan->host_used && cudaEventRecord(plan->ev_sorted, st) != cudaSuccess) return FMM_ERR_CUDA;
         plan->host_used = 1;
@@ -538,7 +539,6 @@ fmm_status fmm_potential_host_async(fmm_plan_t plan, const double* xy_host, cons
             return FMM_ERR_CUDA;
     }
     plan->stage_next = b ^ 1;
-    plan->host_pending = 1;
     return FMM_OK;
 }
 
