@@ -488,7 +488,9 @@ fmm_status fmm_potential_host_async(fmm_plan_t plan, const double* xy_host, cons
     double *xy = plan->d_xy_stage[b], *q = plan->d_q_stage[b], *phi = plan->d_phi_stage[b];
     fmm_status s;
     if (plan->precision == FMM_FP64 || plan->serial) {
-        // one stream: upload, method, download in turn
+        // one stream: upload, method, download in turn; a call of the other kind two back may still download from
+        // this set's phi
+        if (plan->ev_down_done[b] && cudaStreamWaitEvent(st, plan->ev_down_done[b], 0) != cudaSuccess) return FMM_ERR_CUDA;
         if (cudaMemcpyAsync(xy, xy_host, sizeof(double) * 2 * n, cudaMemcpyHostToDevice, st) != cudaSuccess ||
             cudaMemcpyAsync(q, q_host, sizeof(double) * n, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return FMM_ERR_CUDA;

@@ -354,3 +354,24 @@ def test_crowded_squares_pairs_across_an_edge(oracle_mod, n_a, n_b):
     d = np.hypot(xy[:, None, 0] - xy[None, :, 0], xy[:, None, 1] - xy[None, :, 1])
     tol = 2.0 ** -20 * ((np.abs(np.log(np.where(d > 0, d, 1.0))) + 1.0) @ np.abs(q) + 10.0)
     assert np.all(np.abs(phi - ref) <= tol), f"largest {np.max(np.abs(phi - ref)):.3g}"
+
+
+def test_host_calls_across_a_change_of_concurrency(oracle_mod):
+    """Host calls in a row without a wait, on three streams, then one, then three: each result its own call's."""
+    import torch
+    from paper_2009_00767_gb300 import binding
+    n, lev, p = 70000, 6, 8
+    systems = [inputs.uniform(n, 8650 + k) for k in range(6)]
+    pinned = [(torch.from_numpy(xy).pin_memory(), torch.from_numpy(q).pin_memory(), torch.zeros(n, dtype=torch.float64).pin_memory())
+              for xy, q in systems]
+    with binding.Plan(n, lev, p, 5.0, "bf16x2") as plan:
+        for k, (xy, q, phi) in enumerate(pinned):
+            if k in (2, 4):
+                binding.fmm_set_concurrency(plan.handle, 1 if k == 2 else 3)
+            binding.fmm_potential_host_async(plan.handle, xy, q, phi)
+        plan.sync()
+        alone = []
+        for xy, q in systems:
+            alone.append(plan.potential(torch.from_numpy(xy).cuda(), torch.from_numpy(q).cuda()).cpu().numpy())
+    for k, (a, (_, _, phi)) in enumerate(zip(alone, pinned)):
+        check_parity(phi.numpy(), a, MIXED_TOL, f"host call {k}")
