@@ -599,7 +599,7 @@ k_p2p32(const float4* __restrict__ hi, const float4* __restrict__ lo, const int*
 }
 
 // The near field in FP64 (node and literal FP64 forms): p2p64.cuh's warp per chunk of up to kWarpChunk64
-// targets and group of forward cells, items from the shared counter as above.
+// targets and group of forward cells.  Resident warps take the items from a counter.
 // 80,000 charges in 3D, levels 3: 3.40 ms against 19.7 ms for a kernel that took every ordered pair with FP64
 // sqrt and divide (260M ordered pairs, 13 FP64 instructions for two of them: 3.2 ms at the pipe's rate).
 constexpr int kP2PWarps64 = 4;
@@ -1715,7 +1715,7 @@ fmm_status fmm_lag_potential(fmm_lag_plan_t pl, const double* pos, const double*
 
 fmm_status fmm_lag_sync(fmm_lag_plan_t pl) {
     if (!pl) return FMM_ERR_INVALID_ARG;
-    // a call joins its near field's stream back before the final sum, so its stream is all there is to wait
+    // a call joins its far field's stream back before the evaluation, so its stream is all there is to wait
     // for; after a change of stream the last call's is waited for as well
     fmm_status rc = FMM_OK;
     if (pl->st != pl->last_st) rc = cuda_status(cudaEventSynchronize(pl->ev[4]));

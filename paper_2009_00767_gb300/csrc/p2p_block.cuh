@@ -9,13 +9,14 @@ namespace {
 // Near field (E-2 of Sec. 2.1): every particle of a finest square against the particles of that
 // square and its (up to) eight neighbours, in FP32 on square-local coordinates.
 //
-// One warp takes a block of up to 24 targets of one finest square.  The lanes walk the sources 32
-// at a time (the own square's first, then the neighbours'), each lane holding one source moved into the target square's
-// frame, and keep one FP32 partial sum per target in registers; the targets' coordinates are
-// shared-memory broadcasts, two targets per load.  The arithmetic of two targets runs in packed
-// FP32x2 instructions, so a pair costs one lg2 on the MUFU unit and two to three FP32 slots.
+// One warp takes a block of up to 24 targets of one finest square.  The lanes walk the sources 32 at a
+// time (the own square's first, then the four forward neighbours', whose pairs serve both sides, see
+// below), each lane holding one source moved into the target square's frame, and keep one FP32 partial
+// sum per target in registers; the targets' coordinates are shared-memory broadcasts, two targets per
+// load.  The arithmetic of two targets runs in packed FP32x2 instructions, so a pair costs one lg2 on
+// the MUFU unit and two to three FP32 slots.
 // Coincidence (r^2 = 0: the target itself, duplicate points) only arises within the own square,
-// whose chunks test r^2 > 0; a neighbour's pair adds 2^-100 to r^2 instead, which keeps the
+// whose chunks test r^2 > 0; a forward neighbour's pair adds 2^-100 to r^2 instead, which keeps the
 // logarithm finite should two particles of adjacent squares round to the same FP32 point and
 // changes no other pair.  After each run of kP2PRun chunks the partials of each target are
 // combined across the warp by a shuffle reduce-scatter (lane t ends with target t's sum) and
@@ -60,28 +61,21 @@ __device__ __forceinline__ float warp_reduce_scatter(const float2 (&p)[NP], int 
     return s;
 }
 
-// one chunk: the lane's source (sx, sy, q) against the NP target pairs of the block (the
+// one own-square chunk: the lane's source (sx, sy, q) against the NP target pairs of the block (the
 // coordinates of targets past the block's end are zero and their sums are dropped)
-template <bool kOwn, int NP>
+template <int NP>
 __device__ __forceinline__ void p2p_chunk(float2 (&part)[NP], const float4* __restrict__ tg, float4 src) {
     const float2 nsx = make_float2(-src.x, -src.x), nsy = make_float2(-src.y, -src.y);
     const float2 q2 = make_float2(src.z, src.z);
-    const float2 tiny = make_float2(0x1p-100f, 0x1p-100f);
 #pragma unroll
     for (int tp = 0; tp < NP; ++tp) {
         const float4 t = tg[tp];   // {x of target 2tp, x of 2tp + 1, y of 2tp, y of 2tp + 1}
         const float2 dx = __fadd2_rn(make_float2(t.x, t.y), nsx);
         const float2 dy = __fadd2_rn(make_float2(t.z, t.w), nsy);
-        float2 r2, lg;
-        if (kOwn) {
-            r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
-            lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-            lg.x = r2.x > 0.f ? lg.x : 0.f;
-            lg.y = r2.y > 0.f ? lg.y : 0.f;
-        } else {
-            r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, tiny));
-            lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
-        }
+        const float2 r2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+        float2 lg = make_float2(mufu_lg2(r2.x), mufu_lg2(r2.y));
+        lg.x = r2.x > 0.f ? lg.x : 0.f;
+        lg.y = r2.y > 0.f ? lg.y : 0.f;
         part[tp] = __ffma2_rn(q2, lg, part[tp]);
     }
 }
@@ -168,7 +162,7 @@ __device__ __forceinline__ float2 p2p_block_sym(const P2PSymSources& S, const fl
             uint32_t nidx = idx;
             const float4 nxt = (c + 1 < r1) ? S.load(c + 1, lane, &nidx) : cur;
             if (c < S.nch_own) {
-                p2p_chunk<true, NP>(part, tg, cur);
+                p2p_chunk<NP>(part, tg, cur);
             } else {
                 const float ssum = p2p_chunk_sym<NP>(part, tg, tq, cur);
                 if (idx != 0xffffffffu) atomicAdd(acc + idx, fmm_f2d_bits(ssum));
@@ -303,7 +297,7 @@ __device__ __forceinline__ void p2p_crowd_item(const float4* __restrict__ sp, ui
     float2 part[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) part[i] = make_float2(0.f, 0.f);
-    if (self) p2p_chunk<true, NP>(part, sh.tg, lane < T ? sp[b0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f));
+    if (self) p2p_chunk<NP>(part, sh.tg, lane < T ? sp[b0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f));
     const uint32_t e0 = (uint32_t)sh.seg[0].w, e1 = (uint32_t)sh.seg[1].w, e2 = (uint32_t)sh.seg[2].w,
                    e3 = (uint32_t)sh.seg[3].w;
     auto load = [&](uint32_t s, uint32_t* idx) {
