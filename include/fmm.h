@@ -11,14 +11,17 @@
  * (arXiv 2009.00767):
  *   - the computation box is split into a uniform quadtree of depth `levels`
  *     (Sec. 2.1 items 1-4);
- *   - for EVERY level k = 2..levels the multipole moments of every square are
- *     formed directly from the particles (the upward pass U-bar of Sec. 2.2.1,
- *     with no multipole-to-multipole shift);
+ *   - the multipole moments of every square of every level k = 2..levels are formed
+ *     (the upward pass U-bar of Sec. 2.2.1): those of the finest level (FP64) or the
+ *     finest three (the mixed forms) directly from the particles, the coarser
+ *     levels' from their four children's, re-expanded about the parent's centre
+ *     (a finite sum, exact for truncated expansions);
  *   - each square's interaction list (Sec. 2.1 item 5) is converted into a
  *     local expansion (D-bar-1 of Sec. 2.2.1);
- *   - each level's local expansion is evaluated directly at the particles and
- *     the levels are summed (D-bar-2 of Sec. 2.2.1 by linearity, with no
- *     local-to-local shift);
+ *   - the levels' local expansions are summed (D-bar-2 of Sec. 2.2.1): the mixed
+ *     forms evaluate each level's directly at the particles, by linearity, with no
+ *     local-to-local shift; FP64 re-expands each square's about its children's
+ *     centres (exact for truncated expansions) and evaluates the finest level's;
  *   - the near field of the own and eight adjacent finest squares is summed
  *     directly (Sec. 2.1 E-2).
  * The vectors and bilinear forms of Sec. 2.2.1 are realised as complex

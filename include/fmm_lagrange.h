@@ -40,9 +40,15 @@
  *                        list, the node potentials summed down to the finest cells (D-bar-2)
  *                        and interpolated back at the charges; equal to the literal form in
  *                        exact arithmetic and free of its cancellation.  FP64 throughout.
- *   FMM_LAG_NODE_F32     the node form in FP32 arithmetic with FP64 accumulation across
- *                        levels and source tiles; near-field differences from two-word (hi, lo)
- *                        FP32 coordinates.  About 1e-7 relative to the FP64 node form.
+ *   FMM_LAG_NODE_F32     the node form in FP32 arithmetic.  Node charges: FP32 sums, rounded to
+ *                        FP32 once a level on the way up; node potentials: FP64 sums over levels
+ *                        and offset groups, interpolated in FP32 as differences within a cell.
+ *                        Near field: differences from two-word (hi, lo) FP32 coordinates; a
+ *                        target's sum is FP32 over up to 512 sources (16 a lane, then a tree over
+ *                        the lanes) and FP64 beyond, a source's FP32 over the 24 targets of a
+ *                        chunk and FP64 beyond.  Charges of one cell closer than 2^-63 count as
+ *                        coincident; charges of adjacent cells that no two-word coordinate tells
+ *                        apart count as 2^-50 box apart.  About 1e-7 relative to the FP64 node form.
  * The method's own error (4 nodes per axis) is about 1e-4 .. 1e-3 of the potential.
  *
  * Conventions (as in fmm.h): device pointers on the plan's device, owned by the caller;

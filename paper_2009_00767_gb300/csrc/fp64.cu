@@ -371,7 +371,10 @@ __global__ void k_l2p_f64(const fmm_p64* __restrict__ sp, const uint32_t* __rest
 // kField: also grad phi, q (dx, dy) / r^2 to the target and the opposite to the source.
 constexpr int kP2PWarps64 = 8;
 // With fewer blocks than this, CTAs of two warps instead of eight: 152 SMs x 4 schedulers x 8 warps
-// are not filled either way, and the smaller CTAs reach more SMs.
+// are not filled either way, and the smaller CTAs reach more SMs.  The kernel alone, two against eight warps:
+// 427 blocks (4,096 particles, levels 4) 47 and 53 us, 898 (20,000, levels 3) 737 and 917, 2,757 (60,000, levels
+// 4) 1.48 and 1.87 ms; above the line the gain fades: 6,827 (65,536, levels 6) 154 and 168 us, 27,307 (2^18,
+// levels 7) 494 and 520.
 constexpr int64_t kP2PSmall = 4096;
 
 template <bool kField>
@@ -462,7 +465,9 @@ int fmm_launch_fp64(fmm_plan_s* pl, double* phi, double* field) {
     const int64_t n = pl->n;
     const int L = pl->levels, p = pl->p, p1 = p + 1;
     const double s = pl->box / (double)(1 << L), inv_s = (double)(1 << L) / pl->box;
-    // a grid of (2^k)^2 squares in CTAs of whole rows: few squares take smaller CTAs, to reach more SMs
+    // a grid of (2^k)^2 squares in CTAs of whole rows: few squares take smaller CTAs, to reach more SMs.  M2L with
+    // 64 and 128 threads: levels 4, p = 16 34.3 and 35.0 us, levels 5, p = 12 39.1 and 47.0; levels 6, p = 16 158
+    // and 145, levels 7 557 and 487 (the real matrix is copied to shared memory for fewer squares).
     const int threads = L <= 5 ? kFarThreadsSmall : kFarThreads, per = threads / p1;
     const int tab = (p1 * p1 + 1) & ~1;   // doubles of a real matrix in shared memory, 16-byte aligned
     const double* R = pl->ftab;
