@@ -335,13 +335,14 @@ __device__ __forceinline__ int chunk_leaf(const int* __restrict__ chunk_start, i
 // close pair's distance keeps about 48 bits.  Pairs inside A below r^2 = 2^-126, FP32's smallest normal number,
 // count as coincident and give 0.  Two charges either side of a cell's edge may share one two-word point: the
 // pairs with the forward cells add tiny = (2^-50 box)^2 to r^2, which moves no pair that the words tell apart
-// by more than their own rounding (1.4% of 200,000 charges' call in 3D; a maximum with tiny instead 5%).  After kP2PRun chunks the lanes' partials of a target are summed across the warp
-// (warp_reduce_scatter) and added in FP64.
+// by more than their own rounding (1.4% of 200,000 charges' call in 3D; a maximum with tiny instead 5%).
+// After kP2PRun chunks the lanes' partials of a target are summed across the warp (warp_reduce_scatter) and
+// added in FP64.
 // What bounds it: the FMA pipe, 14 packed instructions (two cycles each) for two targets in 3D, 9 of them
 // the two-word differences.  A lane holds two sources, so that the targets' shared-memory broadcasts (8
-// wavefronts for two targets) serve four pairs.  200,000 charges in 3D, levels 3: 467 us against 739 us for
+// wavefronts for two targets) serve four pairs.  200,000 charges in 3D, levels 3: 468 us against 739 us for
 // 64 targets over the lanes and a butterfly over the lanes per source tile (31 shuffles, 62 selects) for the
-// source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us, and 198 with
+// source's side, and 486 us with one source a lane; 2^20 in 2D, levels 7: 238, 368 and 256 us, and 200 with
 // the two changes below.
 // In 2D, with a few chunks an item, the warps of an SM are at many places of the unrolled code and wait for
 // instructions, so the code is kept small: the chunk itself and a last half chunk share a body, and whole
